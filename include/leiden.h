@@ -191,9 +191,11 @@ typedef struct {
   int64_t move_scanned_vertices;
   double move_bytes;                            /* algorithmic bytes of those launches */
   double total_ms;                              /* host wall time of the call */
-  /* host wall time per pass: local-moving phase (with the vertex buckets),
-   * refinement (with subset renumbering and the break), aggregation (with
-   * renumbering and the dendrogram lookup), and the whole pass */
+  /* time per pass: local-moving phase (with the vertex buckets), refinement
+   * (with subset renumbering and the break), aggregation (with renumbering and
+   * the dendrogram lookup), and the whole pass; host wall time, but for a pass
+   * that runs in one launch the phases are on the device clock (aggregation 0
+   * when it follows in launches of its own) */
   double t_move_ms[LEIDEN_STATS_PASSES];
   double t_refine_ms[LEIDEN_STATS_PASSES];
   double t_agg_ms[LEIDEN_STATS_PASSES];
@@ -431,6 +433,10 @@ uint64_t leiden_kernel_launches(void);
  * max_degree unbounded) spreads each row over many blocks with tables in
  * global scratch.  The tier table changes only the kernel shapes, never the
  * result: every vertex takes the same decision whichever tier processes it.
+ * With the default table, DET passes whose longest row has at most 8192
+ * distinct neighbours run on blocks that stay resident for the whole pass,
+ * with shapes of their own; a context given another table runs the kernels
+ * the table describes.
  * The default table is the one leiden_tiers_default returns; leiden_autotune
  * picks one per graph. */
 #define LEIDEN_MAX_TIERS 11

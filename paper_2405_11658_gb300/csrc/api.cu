@@ -18,6 +18,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "leiden.h"
+#include "team.h"
 
 using namespace lk;
 
@@ -43,6 +44,7 @@ struct leiden_ctx {
   int device = 0, sms = 152;
   int64_t max_n = 0, max_nnz = 0;
   TierTable tiers{};
+  bool tiers_set = false;  // the caller chose another table than the default
   int agg_uniform = 0;   // aggregation policy (leiden_ctx_set_agg_policy)
   std::vector<void *> allocs;
   int64_t device_bytes = 0;
@@ -72,14 +74,18 @@ struct leiden_ctx {
   HubWork hub{};
   int64_t hub_items = 0;
   u64 *ctr;
-  // pinned host
+  TeamCtl *tctl;
+  // pinned host, one allocation at h_ctr
   u64 *h_ctr;
+  TeamCtl *h_tctl = nullptr;  // the head of tctl
   int64_t *h_koff;
   // diagnostics of the last failure
   char err[256] = {0};
   // statistics
   leiden_run_stats stats{};
   int timing = 0;
+  // decide phases of the team path (device clock), all passes and the first
+  int64_t team_ns = 0, team_subsweeps = 0, team0_ns = 0, team0_subsweeps = 0;
   std::vector<cudaEvent_t> evs;
   // auxiliary streams: the independent tier kernels of one sub-sweep run on
   // them concurrently, forked from and joined back into the context stream
@@ -122,7 +128,6 @@ void free_all(leiden_ctx *c) {
   for (void *p : c->allocs) cudaFree(p);
   c->allocs.clear();
   if (c->h_ctr) cudaFreeHost(c->h_ctr);
-  if (c->h_koff) cudaFreeHost(c->h_koff);
   for (auto e : c->evs) cudaEventDestroy(e);
   c->evs.clear();
   for (int k = 0; k < leiden_ctx::NAUX; k++) {
@@ -135,6 +140,7 @@ void free_all(leiden_ctx *c) {
   c->ev_fork = nullptr;
   c->h_ctr = nullptr;
   c->h_koff = nullptr;
+  c->h_tctl = nullptr;
 }
 
 int sync(leiden_ctx *c) {
@@ -284,6 +290,19 @@ int64_t count_flags(leiden_ctx *c, const uint8_t *a, int64_t n) {
   cudaMemcpyAsync(&c->h_ctr[CTR_SCRATCH0], &c->ctr[CTR_SCRATCH0], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   if (sync(c)) return -1;
   return (int64_t)c->h_ctr[CTR_SCRATCH0];
+}
+
+// Largest row and largest K' of a level.
+int level_maxima(const Run &r, const int64_t *off, int64_t n, Buckets &b) {
+  leiden_ctx *c = r.c;
+  cudaMemsetAsync(&c->ctr[CTR_SCRATCH0], 0, 2 * sizeof(u64), c->st);
+  if (n > 0) LK_COUNTED maxdeg_k<<<c->sms * 4, 256, 0, c->st>>>(off, c->Kp, n, &c->ctr[CTR_SCRATCH0]);
+  cudaMemcpyAsync(&c->h_ctr[CTR_SCRATCH0], &c->ctr[CTR_SCRATCH0], 2 * sizeof(u64), cudaMemcpyDeviceToHost, c->st);
+  const int rc = sync(c);
+  if (rc) return rc;
+  b.maxdeg = (int64_t)c->h_ctr[CTR_SCRATCH0];
+  b.kmax = (int64_t)c->h_ctr[CTR_SCRATCH0 + 1];
+  return LEIDEN_OK;
 }
 
 int build_buckets(const Run &r, const int64_t *off, int64_t n, Buckets &b) {
@@ -500,6 +519,26 @@ template <typename WT, typename ST>
 int pass_body(Run &r, GraphView<WT> g, int lp, double tau, int dst, int64_t *nc_out, int64_t *nnz_out,
               const Buckets &b, std::chrono::steady_clock::time_point t_start);
 
+// Alg. leidenag of level g (nc communities in the dense C') into level buffer dst.
+template <typename WT>
+int aggregate_level(Run &r, GraphView<WT> g, int dst, int64_t nc, int64_t *nnz_out) {
+  leiden_ctx *c = r.c;
+  int64_t nnz2 = 0;
+  int rc;
+  {
+    Phase ph("aggregate");
+    rc = aggregate<WT>(g, c->Cp, nc, c->goff[dst], c->gidx[dst], c->gw[dst], &nnz2, agg_work(c), c->st);
+  }
+  if (rc) return rc;
+  cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
+  rc = sync(c);
+  if (rc) return rc;
+  rc = check_dev_flags(c, c->h_ctr[CTR_ERROR]);
+  if (rc) return rc;
+  *nnz_out = nnz2;
+  return LEIDEN_OK;
+}
+
 template <typename WT>
 int pass(Run &r, GraphView<WT> g, int lp, double tau, int dst, int64_t *nc_out, int64_t *nnz_out) {
   const auto t_start = std::chrono::steady_clock::now();
@@ -569,22 +608,144 @@ int pass_body(Run &r, GraphView<WT> g, int lp, double tau, int dst, int64_t *nc_
     return 1;
   }
   launch_lookup(r.N, c->Ctop, c->Cp, c->st);
-  int64_t nnz2 = 0;
-  {
-    Phase ph("aggregate");
-    rc = aggregate<WT>(g, c->Cp, nc, c->goff[dst], c->gidx[dst], c->gw[dst], &nnz2, agg_work(c), c->st);
-  }
-  if (rc) return rc;
-  cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
-  rc = sync(c);
-  if (rc) return rc;
-  rc = check_dev_flags(c, c->h_ctr[CTR_ERROR]);
-  if (rc) return rc;
-  *nnz_out = nnz2;
+  rc = aggregate_level<WT>(r, g, dst, nc, nnz_out);
   if (rec) {
     c->stats.t_agg_ms[lp] = ms_since(t_agg);
     c->stats.t_pass_ms[lp] = ms_since(t_start);
   }
+  return rc;
+}
+
+// The team path (team.cuh) runs a whole pass in one launch of resident
+// blocks.  It takes every DET pass of a context with the default tier table
+// whose rows have at most TEAM_MAX_CAND distinct candidates (longer rows need
+// the multi-block hub path).  Measured against one launch per tier and
+// sub-sweep (us per sub-sweep, both sides): 27 -> 11 at 4.4e3 vertices /
+// 8.0e4 entries, 45 -> 22 at 8.3e5 / 5.7e6, 235 -> 160 at 1.2e7 / 6.9e7 (grid
+// levels): the launches, the fork to the auxiliary streams and their join
+// cost more than the sub-sweep itself on the small levels, and on the large
+// ones the tiers of a class run back to back without a tail each.
+bool team_takes(const Run &r, int64_t n) {
+  return r.o->sched == LEIDEN_DET && !r.c->tiers_set && n > 0 && n < ((int64_t)1 << 30);
+}
+
+// Level sizes (vertices + entries) up to which a pass runs on one cluster: its
+// hardware barrier takes 0.3 us against 1.2 us for the grid barrier (1.1
+// against 1.9 with stores in flight), but 16 SMs limit the throughput.
+// Planted partition of 1e4 vertices (1.07e5): 6.2 -> 5.8 ms per Static.
+constexpr int64_t TEAM_CLUSTER_SIZE = 131072;
+constexpr int TEAM_CLUSTER_MAX = 16;
+// Vertices + entries per block below which more blocks only lengthen the
+// barrier (1024 .. 4096 within 2% of each other, 8192 slower by 5-10%).
+constexpr int64_t TEAM_BLOCK_SIZE = 2048;
+// Largest level aggregated through the team's one global table (16 bytes a
+// slot, at least 1.5 slots an entry): within L2 it is 2-4 times faster than
+// the multi-kernel path (0.28 against 0.79 ms at 2.2e6 entries, 0.86 against
+// 1.08 at 4.0e6); past it, slower (1.44 against 1.03 ms at 5.7e6).
+constexpr int64_t TEAM_AGG_NNZ = 5500000;
+
+// One pass on the team path; returns as pass() does, or 2 when the caller has
+// to aggregate.
+template <typename WT>
+int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int dst, const Buckets &b,
+                   int64_t *nc_out, Buckets &next, int64_t *nnz_out) {
+  leiden_ctx *c = r.c;
+  const auto t_start = std::chrono::steady_clock::now();
+  TeamArgs<WT> ta{};
+  ta.g = g;
+  ta.nnz = nnz;
+  TeamArrays &a = ta.a;
+  a.C = c->Cp; a.CB = c->CB; a.rep = c->rep; a.vlist = c->vlist;
+  a.K = c->Kp; a.Sig = c->Sp; a.Sig2 = c->S2;
+  a.ch = c->ch; a.ch2 = c->ch2; a.processed = c->processed; a.stamp = c->stamp; a.exists = c->flag;
+  a.prop_i = c->prop_i; a.prop_c = c->prop_c;
+  a.err = &c->ctr[CTR_ERROR];
+  a.hkey = c->gvals;
+  a.hval = c->gvals + c->gcap / 2;
+  a.cnt = c->cdist; a.cur = c->ccur; a.K2 = c->Ktmp;
+  a.off2 = c->goff[dst]; a.idx2 = c->gidx[dst]; a.w2 = c->gw[dst];
+  ta.A = r.A;
+  ta.p = r.p;
+  ta.two_m = r.two_m;
+  ta.den = denom(r);
+  ta.tau = tau;
+  ta.log2S = r.log2S;
+  ta.dynamic = (r.dynamic && lp == 0) ? 1 : 0;
+  ta.timing = c->timing;
+  ta.lp = lp;
+  ta.max_iters = r.o->max_iters;
+  ta.in_range = lp == 0 ? r.in_range0 : nullptr;
+  // aggregation table: at most two thirds full, keys and sums in the two
+  // halves of the scratch values (zero whenever nobody uses them)
+  int lh = 10;
+  while (((int64_t)1 << lh) < nnz + nnz / 2) lh++;
+  ta.agg_lh = (!c->agg_uniform && nnz <= TEAM_AGG_NNZ && ((int64_t)2 << lh) <= c->gcap) ? lh : 0;
+  ta.ctl = c->tctl;
+  cudaMemsetAsync(c->tctl, 0, sizeof(TeamCtl), c->st);
+  int64_t nb = std::min<int64_t>(c->sms, (nnz + g.n + TEAM_BLOCK_SIZE - 1) / TEAM_BLOCK_SIZE);
+  int kind = nb > 1 ? TEAM_GRID : TEAM_BLOCK;
+  const bool narrow = !LK_FORCE_WIDE_SCORES && narrow_scores(r, b);
+  // a context on a share of the SMs may not hold a whole cluster
+  if (nnz + g.n <= TEAM_CLUSTER_SIZE && !c->green.cu) {
+    const int cl = std::min<int>(TEAM_CLUSTER_MAX, (int)((nnz + g.n + 1023) / 1024));
+    if (cl > 1 && (narrow ? team_cluster_fits<WT, int64_t>(cl) : team_cluster_fits<WT, i128>(cl))) {
+      nb = cl;
+      kind = TEAM_CLUSTER;
+    }
+  }
+  int rc;
+  if (narrow) {
+    rc = launch_team_pass<WT, int64_t>(ta, (int)nb, kind, c->st);
+  } else {
+    rc = launch_team_pass<WT, i128>(ta, (int)nb, kind, c->st);
+    if (lp < LEIDEN_STATS_PASSES) c->stats.wide_passes |= 1u << lp;
+  }
+  if (rc) { check_cuda(c); return rc; }
+  std::swap(c->Sp, c->S2);
+  std::swap(c->ch, c->ch2);
+  cudaMemcpyAsync(c->h_tctl, c->tctl, TEAM_CTL_HEAD, cudaMemcpyDeviceToHost, c->st);
+  cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
+  rc = sync(c);
+  if (rc) return rc;
+  const TeamCtl &h = *c->h_tctl;
+  if (h.abort || h.status == TEAM_NONE) {
+    snprintf(c->err, sizeof(c->err), "a bounded device wait expired");
+    return LEIDEN_ETIMEOUT;
+  }
+  rc = check_dev_flags(c, c->h_ctr[CTR_ERROR]);
+  if (rc) return rc;
+  if (lp == 0) c->stats.changed0 = (int64_t)h.changed;
+  const double bytes = (double)h.scanned_e * (8.0 + sizeof(WT)) + (double)h.scanned_v * 42.0 + (double)h.cand * 8.0;
+  c->stats.move_scanned_entries += (int64_t)h.scanned_e;
+  c->stats.move_scanned_vertices += (int64_t)h.scanned_v;
+  c->stats.move_bytes += bytes;
+  c->team_ns += (int64_t)h.decide_ns;
+  c->team_subsweeps += (int64_t)h.subsweeps;
+  if (lp == 0) {
+    c->stats.move0_bytes += bytes;
+    c->stats.move0_scanned_entries += (int64_t)h.scanned_e;
+    c->team0_ns = (int64_t)h.decide_ns;
+    c->team0_subsweeps = (int64_t)h.subsweeps;
+  }
+  if (lp < LEIDEN_STATS_PASSES) {
+    c->stats.passes = lp + 1;
+    c->stats.iters[lp] = h.li;
+    c->stats.nv[lp] = g.n;
+    c->stats.moves[lp] = h.moves;
+    c->stats.refine_moves[lp] = (int64_t)h.rmoves;
+    c->stats.t_move_ms[lp] = (double)(h.stamp[1] - h.stamp[0]) * 1e-6;
+    c->stats.t_refine_ms[lp] = (double)(h.stamp[2] - h.stamp[1]) * 1e-6;
+    if (h.status == TEAM_AGGREGATED) c->stats.t_agg_ms[lp] = (double)(h.stamp[3] - h.stamp[2]) * 1e-6;
+    c->stats.t_pass_ms[lp] = ms_since(t_start);
+  }
+  if (h.status == TEAM_CONVERGED) return 1;
+  *nc_out = h.nc;
+  if (h.status == TEAM_NO_SHRINK) return 1;
+  launch_lookup(r.N, c->Ctop, c->CB, c->st);
+  if (h.status == TEAM_RENUMBERED) return 2;
+  *nnz_out = h.nnz2;
+  next.maxdeg = (int64_t)h.maxdeg;
+  next.kmax = (int64_t)h.kmax;
   return 0;
 }
 
@@ -601,12 +762,36 @@ int run_leiden(Run &r, const leiden_csr *g0) {
   int64_t nv = N;
   int lp;
   int64_t nnz_cur = g0->nnz;
+  bool known = false;   // lev holds the current level's maxima
+  Buckets lev;
   for (lp = 0; lp < r.o->max_passes; lp++) {
     if (lp < LEIDEN_STATS_PASSES) c->stats.nnz[lp] = nnz_cur;
     const int dst = cur < 0 ? 0 : 1 - cur;
     int64_t nc = 0, nnz2 = 0;
-    int rc = cur < 0 ? pass<int32_t>(r, g32, lp, tau, dst, &nc, &nnz2)
-                     : pass<int64_t>(r, g64, lp, tau, dst, &nc, &nnz2);
+    bool team = team_takes(r, nv);
+    int rc;
+    if (team && !known) {
+      rc = level_maxima(r, cur < 0 ? g32.off : g64.off, nv, lev);
+      if (rc) return rc;
+    }
+    team = team && std::min(lev.maxdeg, nv) <= TEAM_MAX_CAND && lev.maxdeg < ((int64_t)1 << 30);
+    known = false;
+    if (team) {
+      Buckets next;
+      rc = cur < 0 ? team_pass_host<int32_t>(r, g32, nnz_cur, lp, tau, dst, lev, &nc, next, &nnz2)
+                   : team_pass_host<int64_t>(r, g64, nnz_cur, lp, tau, dst, lev, &nc, next, &nnz2);
+      if (rc == 0) {
+        known = true;
+        lev.maxdeg = next.maxdeg;
+        lev.kmax = next.kmax;
+      } else if (rc == 2) {
+        rc = cur < 0 ? aggregate_level<int32_t>(r, g32, dst, nc, &nnz2)
+                     : aggregate_level<int64_t>(r, g64, dst, nc, &nnz2);
+      }
+    } else {
+      rc = cur < 0 ? pass<int32_t>(r, g32, lp, tau, dst, &nc, &nnz2)
+                   : pass<int64_t>(r, g64, lp, tau, dst, &nc, &nnz2);
+    }
     if (rc < 0) return rc;
     if (rc == 1) break;
     // next level: K' = Sigma' = row sums (written by the aggregation), C' =
@@ -615,11 +800,12 @@ int run_leiden(Run &r, const leiden_csr *g0) {
     g64 = GraphView<int64_t>{nc, c->goff[cur], c->gidx[cur], c->gw[cur]};
     nv = nc;
     nnz_cur = nnz2;
+    tau /= r.o->tol_drop;
+    if (known) continue;   // the team pass left the next level's state behind
     launch_copy_i64(c->Sp, c->Kp, nv, c->st);
     launch_iota(c->Cp, nv, c->st);
     cudaMemsetAsync(c->processed, 0, (size_t)(nv > 0 ? nv : 1), c->st);
     cudaMemsetAsync(c->ch, 1, (size_t)(nv > 0 ? nv : 1), c->st);
-    tau /= r.o->tol_drop;
   }
   launch_lookup(N, c->Ctop, c->Cp, c->st);
   return check_cuda(c);
@@ -699,6 +885,7 @@ int modularity_of(leiden_ctx *c, const leiden_csr *g, const int32_t *C, int64_t 
 
 void reset_stats(leiden_ctx *c) {
   c->stats = leiden_run_stats{};
+  c->team_ns = c->team_subsweeps = c->team0_ns = c->team0_subsweeps = 0;
 }
 
 // A run that stopped half-way may leave scratch tables or counters dirty;
@@ -720,8 +907,10 @@ void finish_timing(leiden_ctx *c) {
     ms += t;
     if (k < c->stats.move0_kernel_launches) ms0 += t;
   }
-  c->stats.move_kernel_ms = ms;
-  c->stats.move0_kernel_ms = ms0;
+  c->stats.move_kernel_ms = ms + (double)c->team_ns * 1e-6;
+  c->stats.move0_kernel_ms = ms0 + (double)c->team0_ns * 1e-6;
+  c->stats.move_kernel_launches += c->team_subsweeps;
+  c->stats.move0_kernel_launches += c->team0_subsweeps;
 }
 
 }  // namespace
@@ -746,10 +935,14 @@ void leiden_opts_default(leiden_opts *o) {
 
 int leiden_ctx_set_tiers(leiden_ctx *c, const leiden_tier_table *t) {
   if (!c) return LEIDEN_EINVAL;
-  if (!t) { c->tiers = default_tiers(); return LEIDEN_OK; }
+  if (!t) { c->tiers = default_tiers(); c->tiers_set = false; return LEIDEN_OK; }
   TierTable tt;
   if (tiers_from_public(t, &tt) != LEIDEN_OK) return LEIDEN_EINVAL;
   c->tiers = tt;
+  leiden_tier_table def, got;
+  tiers_to_public(default_tiers(), &def);
+  tiers_to_public(tt, &got);
+  c->tiers_set = memcmp(&def, &got, sizeof(def)) != 0;
   return LEIDEN_OK;
 }
 
@@ -818,6 +1011,7 @@ int ctx_init(leiden_ctx *c, int64_t max_n, int64_t max_nnz) {
   rc |= dal(c, &c->hidx, m); rc |= dal(c, &c->hw, m);
   rc |= dal(c, &c->gkeys, c->gcap); rc |= dal(c, &c->gvals, c->gcap);
   rc |= dal(c, &c->ctr, CTR_COUNT);
+  rc |= dal(c, &c->tctl, 1);
   rc |= dal(c, &c->big, n1);
   // giant-community buckets: a community of total degree T > 2048 gets at most
   // 2 * ceil(T / 2048) <= T / 512 buckets, so the total stays below nnz / 512
@@ -838,9 +1032,16 @@ int ctx_init(leiden_ctx *c, int64_t max_n, int64_t max_nnz) {
     }
   }
   if (rc == LEIDEN_OK) {
-    if (cudaMallocHost((void **)&c->h_ctr, CTR_COUNT * sizeof(u64)) != cudaSuccess ||
-        cudaMallocHost((void **)&c->h_koff, (MAX_KEYS + 8) * sizeof(int64_t)) != cudaSuccess)
+    // one pinned allocation: the counters, the bucket offsets, the team's words
+    constexpr size_t ctr_b = CTR_COUNT * sizeof(u64), koff_b = (MAX_KEYS + 8) * sizeof(int64_t);
+    char *h = nullptr;
+    if (cudaMallocHost((void **)&h, ctr_b + koff_b + TEAM_CTL_HEAD) != cudaSuccess) {
       rc = LEIDEN_ENOMEM;
+    } else {
+      c->h_ctr = reinterpret_cast<u64 *>(h);
+      c->h_koff = reinterpret_cast<int64_t *>(h + ctr_b);
+      c->h_tctl = reinterpret_cast<TeamCtl *>(h + ctr_b + koff_b);
+    }
   }
   if (rc != LEIDEN_OK) {
     cudaGetLastError();

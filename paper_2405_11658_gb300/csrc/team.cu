@@ -1,0 +1,105 @@
+// team.cu -- the cooperative launch of a team pass (team.cuh) for a context.
+#include <mutex>
+
+#include "team.cuh"
+
+namespace lk {
+
+template <typename WT, typename ST>
+__global__ void __launch_bounds__(TEAM_THREADS, 1) team_pass_k(TeamArgs<WT> args, int kind) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ TeamShared<ST> sm;
+  if (threadIdx.x == 0) sm.dead = 0;
+  __syncthreads();
+  Team t;
+  t.rank = blockIdx.x;
+  t.nb = gridDim.x;
+  t.kind = kind;
+  t.gen = 0;
+  t.ctl = args.ctl;
+  t.dead_s = &sm.dead;
+  t.dead = false;
+  TeamConst ct;
+  ct.A = args.A;
+  ct.p = args.p;
+  ct.den = args.den;
+  ct.two_m = args.two_m;
+  ct.log2S = args.log2S;
+  ct.dynamic = args.dynamic;
+  ct.timing = args.timing;
+  ct.in_range = args.in_range;
+  const TeamLevel<WT> g{args.g.n, args.nnz, args.g.off, args.g.idx, args.g.w};
+  team_pass<WT, ST>(g, args.a, ct, args.lp, args.tau, args.max_iters, args.agg_lh, t, dyn, sm);
+}
+
+template <typename WT, typename ST>
+static size_t team_smem() {
+  return (size_t)TEAM_WARPS * TEAM_WSLOTS * (sizeof(typename TableVal<ST>::type) + sizeof(int32_t));
+}
+
+// Whether a cluster of nb team blocks can be resident (asked once per size).
+template <typename WT, typename ST>
+bool team_cluster_fits(int nb) {
+  static std::mutex mu;
+  static int known[TEAM_MAX_CLUSTER + 1] = {};   // 0: not asked, 1: yes, 2: no
+  if (nb < 2 || nb > TEAM_MAX_CLUSTER) return false;
+  std::lock_guard<std::mutex> lock(mu);
+  if (known[nb]) return known[nb] == 1;
+  auto k = team_pass_k<WT, ST>;
+  ensure_smem((const void *)k, team_smem<WT, ST>());
+  cudaFuncSetAttribute((const void *)k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)nb, 1, 1);
+  cfg.blockDim = dim3(TEAM_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = team_smem<WT, ST>();
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)nb;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, (const void *)k, &cfg) != cudaSuccess) n = 0;
+  (void)cudaGetLastError();
+  known[nb] = n > 0 ? 1 : 2;
+  return n > 0;
+}
+
+template <typename WT, typename ST>
+int launch_team_pass(const TeamArgs<WT> &args, int nb, int kind, cudaStream_t s) {
+  auto k = team_pass_k<WT, ST>;
+  const size_t smem = team_smem<WT, ST>();
+  ensure_smem((const void *)k, smem);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)nb, 1, 1);
+  cfg.blockDim = dim3(TEAM_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  if (kind == TEAM_CLUSTER) {
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)nb;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+  } else {
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+  }
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  note_launch();
+  if (cudaLaunchKernelEx(&cfg, k, args, kind) != cudaSuccess) return LEIDEN_ECUDA;
+  return LEIDEN_OK;
+}
+
+#define LK_TEAM_INST(WT, ST)                                                          \
+  template int launch_team_pass<WT, ST>(const TeamArgs<WT> &, int, int, cudaStream_t); \
+  template bool team_cluster_fits<WT, ST>(int);
+LK_TEAM_INST(int32_t, int64_t)
+LK_TEAM_INST(int32_t, i128)
+LK_TEAM_INST(int64_t, int64_t)
+LK_TEAM_INST(int64_t, i128)
+#undef LK_TEAM_INST
+
+}  // namespace lk
