@@ -433,10 +433,9 @@ uint64_t leiden_kernel_launches(void);
  * max_degree unbounded) spreads each row over many blocks with tables in
  * global scratch.  The tier table changes only the kernel shapes, never the
  * result: every vertex takes the same decision whichever tier processes it.
- * With the default table, DET passes whose longest row has at most 8192
- * distinct neighbours run on blocks that stay resident for the whole pass,
- * with shapes of their own; a context given another table runs the kernels
- * the table describes.
+ * With the default table, DET passes run on blocks that stay resident for the
+ * whole pass, with shapes of their own; a context given another table runs
+ * the kernels the table describes.
  * The default table is the one leiden_tiers_default returns; leiden_autotune
  * picks one per graph. */
 #define LEIDEN_MAX_TIERS 11

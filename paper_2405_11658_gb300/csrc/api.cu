@@ -617,14 +617,13 @@ int pass_body(Run &r, GraphView<WT> g, int lp, double tau, int dst, int64_t *nc_
 }
 
 // The team path (team.cuh) runs a whole pass in one launch of resident
-// blocks.  It takes every DET pass of a context with the default tier table
-// whose rows have at most TEAM_MAX_CAND distinct candidates (longer rows need
-// the multi-block hub path).  Measured against one launch per tier and
-// sub-sweep (us per sub-sweep, both sides): 27 -> 11 at 4.4e3 vertices /
-// 8.0e4 entries, 45 -> 22 at 8.3e5 / 5.7e6, 235 -> 160 at 1.2e7 / 6.9e7 (grid
-// levels): the launches, the fork to the auxiliary streams and their join
-// cost more than the sub-sweep itself on the small levels, and on the large
-// ones the tiers of a class run back to back without a tail each.
+// blocks.  It takes every DET pass of a context with the default tier table.
+// Measured against one launch per tier and sub-sweep (us per sub-sweep, both
+// sides): 27 -> 11 at 4.4e3 vertices / 8.0e4 entries, 45 -> 22 at 8.3e5 /
+// 5.7e6, 235 -> 160 at 1.2e7 / 6.9e7 (grid levels), 800 -> 620 at 8.3e5 /
+// 2.3e8 with hubs (Chung-Lu): the launches, the fork to the auxiliary streams
+// and their join cost more than the sub-sweep itself on the small levels, and
+// on the large ones the tiers of a class run back to back without a tail each.
 bool team_takes(const Run &r, int64_t n) {
   return r.o->sched == LEIDEN_DET && !r.c->tiers_set && n > 0 && n < ((int64_t)1 << 30);
 }
@@ -645,7 +644,7 @@ constexpr int64_t TEAM_BLOCK_SIZE = 2048;
 constexpr int64_t TEAM_AGG_NNZ = 5500000;
 
 // One pass on the team path; returns as pass() does, or 2 when the caller has
-// to aggregate.
+// to aggregate, or 3 when the level's hubs exceed the scratch (nothing done).
 template <typename WT>
 int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int dst, const Buckets &b,
                    int64_t *nc_out, Buckets &next, int64_t *nnz_out) {
@@ -660,6 +659,11 @@ int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int
   a.ch = c->ch; a.ch2 = c->ch2; a.processed = c->processed; a.stamp = c->stamp; a.exists = c->flag;
   a.prop_i = c->prop_i; a.prop_c = c->prop_c;
   a.err = &c->ctr[CTR_ERROR];
+  a.tkeys = c->gkeys; a.tvals = c->gvals; a.tcap = c->gcap;
+  a.hub_i = reinterpret_cast<int32_t *>(c->hub.ioff); a.hub_s = reinterpret_cast<int32_t *>(c->hub.soff);
+  a.hub_done = reinterpret_cast<int32_t *>(c->hub.tsz);
+  a.piece_i = c->hidx; a.piece_k = reinterpret_cast<int32_t *>(c->hw);
+  a.part_sc = c->hub.psc; a.part_c = c->hub.pc; a.part_kid = c->hub.pkid;
   a.hkey = c->gvals;
   a.hval = c->gvals + c->gcap / 2;
   a.cnt = c->cdist; a.cur = c->ccur; a.K2 = c->Ktmp;
@@ -701,13 +705,14 @@ int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int
     if (lp < LEIDEN_STATS_PASSES) c->stats.wide_passes |= 1u << lp;
   }
   if (rc) { check_cuda(c); return rc; }
-  std::swap(c->Sp, c->S2);
-  std::swap(c->ch, c->ch2);
   cudaMemcpyAsync(c->h_tctl, c->tctl, TEAM_CTL_HEAD, cudaMemcpyDeviceToHost, c->st);
   cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   rc = sync(c);
   if (rc) return rc;
   const TeamCtl &h = *c->h_tctl;
+  if (h.status == TEAM_TOO_BIG) return 3;
+  std::swap(c->Sp, c->S2);
+  std::swap(c->ch, c->ch2);
   if (h.abort || h.status == TEAM_NONE) {
     snprintf(c->err, sizeof(c->err), "a bounded device wait expired");
     return LEIDEN_ETIMEOUT;
@@ -774,8 +779,9 @@ int run_leiden(Run &r, const leiden_csr *g0) {
       rc = level_maxima(r, cur < 0 ? g32.off : g64.off, nv, lev);
       if (rc) return rc;
     }
-    team = team && std::min(lev.maxdeg, nv) <= TEAM_MAX_CAND && lev.maxdeg < ((int64_t)1 << 30);
+    team = team && lev.maxdeg < ((int64_t)1 << 30);
     known = false;
+    rc = 3;
     if (team) {
       Buckets next;
       rc = cur < 0 ? team_pass_host<int32_t>(r, g32, nnz_cur, lp, tau, dst, lev, &nc, next, &nnz2)
@@ -788,7 +794,8 @@ int run_leiden(Run &r, const leiden_csr *g0) {
         rc = cur < 0 ? aggregate_level<int32_t>(r, g32, dst, nc, &nnz2)
                      : aggregate_level<int64_t>(r, g64, dst, nc, &nnz2);
       }
-    } else {
+    }
+    if (rc == 3) {
       rc = cur < 0 ? pass<int32_t>(r, g32, lp, tau, dst, &nc, &nnz2)
                    : pass<int64_t>(r, g64, lp, tau, dst, &nc, &nnz2);
     }

@@ -19,7 +19,8 @@
 // scan), and equal communities meet in shared-memory atomics instead of a
 // match across the warp.  Measured (Static of a 1e4-vertex planted partition,
 // 480 sub-sweeps): 13.7 ms with one launch per tier and sub-sweep, 8.2 ms on
-// resident blocks with the tables cleared and scanned, 5.8 ms as here.
+// resident blocks with the tables cleared and scanned, 5.8 ms as here; R-MAT
+// scale 22 with hubs 123 -> 100 ms, Chung-Lu of 2.5e8 entries 290 -> 247 ms.
 #pragma once
 
 #include <limits.h>
@@ -38,22 +39,29 @@ static constexpr int TEAM_WSLOTS = 512;
 static constexpr int TEAM_SUB = 256;                     // threads of a sub-block
 static constexpr int TEAM_NSUB = TEAM_THREADS / TEAM_SUB;
 // Degree tiers: one lane per vertex, 16 lanes, a warp with one, four or eight
-// row entries per lane, a sub-block with eight, the block.
+// row entries per lane, a sub-block with eight, the block, and the whole team
+// for rows whose distinct candidates may not fit the block's table (hubs).
 static constexpr int TT_LANE = 8, TT_HALF = 16, TT_WARP1 = 32, TT_WARP4 = 128, TT_WARP8 = 256, TT_SUB = 2048;
-static constexpr int TEAM_TIERS = 7;
+static constexpr int TEAM_TIERS = 8;
 static constexpr int TEAM_MAX_KEYS = 256 * TEAM_TIERS;
 // Proposals a block keeps in shared memory per sub-sweep (more go to a list
 // of the whole team in global memory).
 static constexpr int TEAM_PROPS = 256;
 
-__device__ __forceinline__ int team_tier(int64_t deg) {
+__device__ __forceinline__ int team_tier(int64_t deg, int64_t n) {
   return deg <= TT_LANE ? 0
          : deg <= TT_HALF ? 1
          : deg <= TT_WARP1 ? 2
          : deg <= TT_WARP4 ? 3
          : deg <= TT_WARP8 ? 4
-         : deg <= TT_SUB ? 5 : 6;
+         : deg <= TT_SUB ? 5
+         : (deg < n ? deg : n) <= TEAM_MAX_CAND ? 6 : 7;
 }
+// Hubs: row entries per insert item, table slots per scan item.
+static constexpr int HUB_ITEM = 2048, HUB_SLOTS = 4096;
+// Movers with longer rows leave their re-marking to the team, in pieces of
+// this many entries.
+static constexpr int REMARK_PIECE = 1024;
 
 // Correctly rounded int128 -> double (round to nearest even) by round-to-odd
 // double rounding (Boldo and Melquiond, "When double rounding is odd", 2005):
@@ -103,6 +111,8 @@ struct TeamShared {
   int32_t h_i[TEAM_NSUB][32];
   int32_t h_n[TEAM_NSUB];
   int32_t koff[TEAM_MAX_KEYS + 1];     // class-list offsets
+  unsigned hbits[TEAM_MAX_HUBS / 32];  // hubs of the class to decide in this sub-sweep
+  int last[TEAM_NSUB];
   int flag;
   int dead;
 };
@@ -192,7 +202,7 @@ struct TeamSweep {
   unsigned par;
   uint8_t sv;
   bool spec;
-  unsigned *nover;
+  unsigned *nover, *npiece;
 };
 
 template <typename ST>
@@ -215,10 +225,14 @@ __device__ __forceinline__ void team_val_add(u64 *p, u64 w) {
 // half full; returns the slot if this call occupied it, else -1.  Equal keys
 // meet in the shared-memory atomics: combining them across the warp first
 // (match, then a walk over the peers) took longer than the conflicts.
-template <typename VT>
+// PIECE: the table takes a piece of a longer row.  An aggregated row lists its
+// communities in the order of hash32, so a piece covers a narrow range of it
+// and would pile up in one corner of the table (12 ms for a sub-sweep of R-MAT
+// scale 22's first aggregated level, 0.25 ms with a hash of its own).
+template <bool PIECE, typename VT>
 __device__ __forceinline__ int team_table_add(int32_t *keys, VT *vals, int lh, int32_t c, u64 w, u64 *err) {
   const uint32_t mask = (1u << lh) - 1u;
-  uint32_t s = hash32(c) >> (32 - lh);
+  uint32_t s = (PIECE ? (uint32_t)c * 0x85EBCA77u : hash32(c)) >> (32 - lh);
   for (uint32_t probe = 0; probe <= mask; probe++) {
     int32_t k = *(volatile int32_t *)&keys[s];
     bool fresh = false;
@@ -269,6 +283,11 @@ __device__ __forceinline__ void team_propose(const TeamArrays &a, const TeamSwee
   base = __shfl_sync(FULL_MASK, base, leader);
   if (!propose) return;
   const unsigned slot = base + __popc(m & ((1u << lane) - 1u));
+  if (!REFINE && h.deg > REMARK_PIECE) {
+    const int np = (h.deg + REMARK_PIECE - 1) / REMARK_PIECE;
+    const unsigned p0 = atomicAdd(sw.npiece, (unsigned)np);
+    for (int k = 0; k < np; k++) { a.piece_i[p0 + k] = i; a.piece_k[p0 + k] = k; }
+  }
   if (slot < TEAM_PROPS) {
     TeamProp &p = sm.prop[slot];
     p.e0 = h.e0;
@@ -404,7 +423,7 @@ __device__ __forceinline__ void team_scan_own(const TeamArrays &a, const int (&o
 
 // The row entries first, first + stride, ... (STEPS of them) of one lane: all
 // their loads, then their gathers, in flight before the first table insert.
-template <int STEPS, bool REFINE, typename WT, typename VT>
+template <int STEPS, bool REFINE, typename WT, bool PIECE = false, typename VT>
 __device__ __forceinline__ void team_insert(const TeamLevel<WT> &g, const TeamArrays &a, int32_t i, int64_t e0, int deg,
                                             int first, int stride, int32_t cbi, int32_t *keys, VT *vals, int lh,
                                             int (&own)[STEPS]) {
@@ -424,7 +443,7 @@ __device__ __forceinline__ void team_insert(const TeamLevel<WT> &g, const TeamAr
   }
 #pragma unroll
   for (int u = 0; u < STEPS; u++)
-    own[u] = own[u] != LEIDEN_EMPTY_KEY ? team_table_add(keys, vals, lh, own[u], (u64)ww[u], a.err) : -1;
+    own[u] = own[u] != LEIDEN_EMPTY_KEY ? team_table_add<PIECE>(keys, vals, lh, own[u], (u64)ww[u], a.err) : -1;
 }
 
 // G lanes per vertex (16 or 32), rows of at most G * STEPS entries, a table of
@@ -608,12 +627,277 @@ __device__ __forceinline__ int team_decide_tier(const TeamLevel<WT> &g, const Te
   return (wg + W - ((m + ch - 1) / ch) % W) % W;
 }
 
+// ---------------------------------------------------------------------------
+// Hubs: rows with more distinct candidates than the block's table holds.  A
+// hub's table is in global scratch (L2): a sub-block takes HUB_ITEM entries
+// of a row, sums them up per community in its shared table and adds the
+// distinct ones to the hub's table; after a barrier a sub-block takes
+// HUB_SLOTS slots, scores and resets them, and the sub-block that finishes a
+// hub's last slots decides.  Item and slot ranges are prefix sums over the
+// class's hubs (TeamArrays::hub_i, hub_s), made once per pass.
+// ---------------------------------------------------------------------------
+// First k in [0, m) with pre[k] > w.
+__device__ __forceinline__ int team_find(const int32_t *pre, int m, int w) {
+  int lo = 0, hi = m - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (pre[mid] > w) hi = mid; else lo = mid + 1;
+  }
+  return lo;
+}
+
+// Adds (c, w) to a hub's table of t slots at offset `at`.  32-bit values: a
+// slot is one 64-bit word, key + 1 in its low half (0: empty), the sum in its
+// high half, so both atomics meet one sector; 64-bit values: keys and values
+// apart.
+template <typename VT>
+__device__ __forceinline__ void team_hub_add(const TeamArrays &a, int64_t at, uint64_t t, int32_t c, u64 w) {
+  uint64_t s = ((uint64_t)hash32(c) * t) >> 32;
+  for (uint64_t probe = 0; probe < t; probe++) {
+    if (sizeof(VT) == 4) {
+      uint32_t *slot = reinterpret_cast<uint32_t *>(&a.tvals[at + (int64_t)s]);
+      const uint32_t key = (uint32_t)c + 1u;
+      const uint32_t old = atomicCAS(slot, 0u, key);
+      if (old == 0u || old == key) { atomicAdd(slot + 1, (uint32_t)w); return; }
+    } else {
+      const int32_t old = atomicCAS(&a.tkeys[at + (int64_t)s], LEIDEN_EMPTY_KEY, c);
+      if (old == LEIDEN_EMPTY_KEY || old == c) { atomicAdd(&a.tvals[at + (int64_t)s], w); return; }
+    }
+    s = s + 1 == t ? 0 : s + 1;
+  }
+  atomicOr(a.err, 16ull);
+}
+
+// Prefix sums of every class's hub items; false when a class has more hubs
+// than the bitmap holds or its tables exceed the scratch (the same answer in
+// every block).
+template <typename WT, typename ST>
+__device__ __forceinline__ bool team_hub_setup(const TeamLevel<WT> &g, const TeamArrays &a, int S, Team &t,
+                                               TeamShared<ST> &sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int h0 = sm.koff[7 * S], hn = sm.koff[8 * S];
+  if (h0 == hn) return true;
+  for (int s = t.rank; s < S; s += t.nb) {
+    const int p0 = sm.koff[7 * S + s], p1 = sm.koff[7 * S + s + 1];
+    int64_t ci = 0, cs = 0;
+    for (int base = p0; base < p1; base += TEAM_THREADS) {
+      const int p = base + (int)threadIdx.x;
+      int64_t vi = 0, vs = 0;
+      if (p < p1) {
+        const int32_t i = a.vlist[p];
+        const int64_t deg = g.off[i + 1] - g.off[i], cap = deg < g.n ? deg : g.n;
+        vi = (deg + HUB_ITEM - 1) / HUB_ITEM;
+        vs = (2 * cap + HUB_SLOTS - 1) / HUB_SLOTS;
+      }
+      int64_t xi = vi, xs = vs;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t yi = shfl_i64(xi, (lane - o) & 31), ys = shfl_i64(xs, (lane - o) & 31);
+        if (lane >= o) { xi += yi; xs += ys; }
+      }
+      __syncthreads();
+      if (lane == 31) { sm.red64[warp] = xi; sm.r_kid[warp] = xs; }
+      __syncthreads();
+      int64_t pi = ci, ps = cs;
+      for (int q = 0; q < TEAM_WARPS; q++) {
+        if (q < warp) { pi += sm.red64[q]; ps += sm.r_kid[q]; }
+        ci += sm.red64[q];
+        cs += sm.r_kid[q];
+      }
+      if (p < p1) {
+        a.hub_i[p - h0] = (int32_t)(pi + xi);
+        a.hub_s[p - h0] = (int32_t)(ps + xs);
+        a.hub_done[p - h0] = 0;
+      }
+    }
+    if (threadIdx.x == 0 && (p1 - p0 > TEAM_MAX_HUBS || cs * HUB_SLOTS > a.tcap || ci > INT_MAX / 2))
+      t.ctl->too_big = 1;
+  }
+  if (!t.sync()) return false;
+  return *(volatile int32_t *)&t.ctl->too_big == 0;
+}
+
+// Which hubs of the class are to be decided, into sm.hbits; whether any is.
+template <bool REFINE, typename ST>
+__device__ __forceinline__ bool team_hub_bits(const TeamArrays &a, const TeamConst &ct, const int32_t *list, int m,
+                                              TeamShared<ST> &sm) {
+  int any = 0;
+  for (int base = 0; base < m; base += TEAM_THREADS) {
+    const int k = base + (int)threadIdx.x;
+    bool act = false;
+    if (k < m) {
+      const int32_t i = list[k];
+      act = REFINE ? (a.ch[a.CB[i]] && a.C[i] == i && a.Sig[i] == a.K[i])
+                   : (!a.processed[i] && (!ct.in_range || ct.in_range[i]));
+    }
+    const unsigned mk = __ballot_sync(FULL_MASK, act);
+    if ((threadIdx.x & 31) == 0 && base + (int)threadIdx.x < m) sm.hbits[(base + (int)threadIdx.x) >> 5] = mk;
+    any |= mk != 0;
+  }
+  return __syncthreads_or(any) != 0;
+}
+
+template <bool REFINE, typename WT, typename ST>
+__device__ __forceinline__ void team_hub_insert(const TeamLevel<WT> &g, const TeamArrays &a, const Team &t,
+                                                const int32_t *list, const int32_t *pi, const int32_t *ps, int m,
+                                                int32_t *keys, typename TableVal<ST>::type *vals,
+                                                TeamShared<ST> &sm) {
+  typedef typename TableVal<ST>::type VT;
+  const int sub = threadIdx.x / TEAM_SUB, tid = threadIdx.x % TEAM_SUB;
+  const int total = pi[m - 1];
+  for (int w = sub * t.nb + t.rank; w < total; w += t.nb * TEAM_NSUB) {
+    const int k = team_find(pi, m, w);
+    if (!((sm.hbits[k >> 5] >> (k & 31)) & 1u)) continue;
+    const int32_t i = list[k];
+    const int64_t e0 = g.off[i], e1 = g.off[i + 1];
+    const int64_t c0 = e0 + (int64_t)(w - (k ? pi[k - 1] : 0)) * HUB_ITEM;
+    const int cnt = (int)(e1 - c0 < HUB_ITEM ? e1 - c0 : HUB_ITEM);
+    const int64_t at = (int64_t)(k ? ps[k - 1] : 0) * HUB_SLOTS;
+    const uint64_t ts = (uint64_t)(ps[k] - (k ? ps[k - 1] : 0)) * HUB_SLOTS;
+    const int32_t cbi = REFINE ? a.CB[i] : 0;
+    int own[8];
+    team_insert<8, REFINE, WT, true>(g, a, i, c0, cnt, tid, TEAM_SUB, cbi, keys, vals, 12, own);
+    bar_named(2 + sub, TEAM_SUB);
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      if (own[u] < 0) continue;
+      const int32_t c = keys[own[u]];
+      const u64 v = (u64)vals[own[u]];
+      keys[own[u]] = LEIDEN_EMPTY_KEY;
+      vals[own[u]] = 0;
+      team_hub_add<VT>(a, at, ts, c, v);
+    }
+    bar_named(2 + sub, TEAM_SUB);
+  }
+}
+
+template <bool REFINE, typename WT, typename ST>
+__device__ __forceinline__ void team_hub_scan(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+                                              const Team &t, const int32_t *list, const int32_t *ps, int32_t *done,
+                                              int m, const TeamSweep &sw, TeamShared<ST> &sm, TeamStat &st) {
+  typedef typename TableVal<ST>::type VT;
+  constexpr int NW = TEAM_SUB / 32;
+  const int sub = threadIdx.x / TEAM_SUB, tid = threadIdx.x % TEAM_SUB, warp = tid >> 5, lane = threadIdx.x & 31;
+  const int wabs = threadIdx.x >> 5, wbase = wabs - warp;
+  const int total = ps[m - 1];
+  for (int w = sub * t.nb + t.rank; w < total; w += t.nb * TEAM_NSUB) {
+    const int k = team_find(ps, m, w);
+    if (!((sm.hbits[k >> 5] >> (k & 31)) & 1u)) continue;
+    const int32_t i = list[k];
+    const int32_t d = a.C[i];
+    const int64_t Ki = a.K[i];
+    const ST A = (ST)ct.A, B = (ST)ct.p * (ST)Ki;
+    ST bsc = 0;
+    int32_t bc = INT32_MAX;
+    int64_t kid = 0;
+    const int64_t s0 = (int64_t)w * HUB_SLOTS + tid;
+    constexpr int Q = 4;
+    for (int x = 0; x < HUB_SLOTS; x += Q * TEAM_SUB) {
+      int32_t c[Q];
+      int64_t v[Q], sg[Q];
+#pragma unroll
+      for (int u = 0; u < Q; u++) {
+        const int64_t s = s0 + x + u * TEAM_SUB;
+        if (sizeof(VT) == 4) {
+          const u64 y = __ldcg(&a.tvals[s]);
+          c[u] = (int32_t)((uint32_t)y - 1u);   // empty: -1
+          v[u] = (int64_t)(y >> 32);
+        } else {
+          c[u] = __ldcg(&a.tkeys[s]);
+          v[u] = c[u] != LEIDEN_EMPTY_KEY ? (int64_t)__ldcg(&a.tvals[s]) : 0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < Q; u++) {
+        if (c[u] == LEIDEN_EMPTY_KEY) { sg[u] = 0; continue; }
+        const int64_t s = s0 + x + u * TEAM_SUB;
+        a.tvals[s] = 0;                         // reset for the next user of the scratch
+        if (sizeof(VT) != 4) a.tkeys[s] = LEIDEN_EMPTY_KEY;
+        sg[u] = c[u] != d ? sigma_for_score(a.Sig, c[u]) : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < Q; u++) {
+        if (c[u] == LEIDEN_EMPTY_KEY) continue;
+        st.ncand++;
+        if (c[u] == d) { kid = v[u]; continue; }
+        const ST sc = A * (ST)v[u] - B * (ST)sg[u];
+        if (team_better(sc, c[u], bsc, bc)) { bsc = sc; bc = c[u]; }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const ST osc = shfl_xor_any<ST>(bsc, o);
+      const int32_t oc = __shfl_xor_sync(FULL_MASK, bc, o);
+      kid += shfl_xor_i64(kid, o);
+      if (team_better(osc, oc, bsc, bc)) { bsc = osc; bc = oc; }
+    }
+    if (lane == 0) { sm.r_sc[wabs] = bsc; sm.r_c[wabs] = bc; sm.r_kid[wabs] = kid; }
+    bar_named(2 + sub, TEAM_SUB);
+    if (warp == 0) {
+      bsc = lane < NW ? sm.r_sc[wbase + lane] : (ST)0;
+      bc = lane < NW ? sm.r_c[wbase + lane] : INT32_MAX;
+      kid = lane < NW ? sm.r_kid[wbase + lane] : 0;
+#pragma unroll
+      for (int o = NW / 2; o > 0; o >>= 1) {
+        const ST osc = shfl_xor_any<ST>(bsc, o);
+        const int32_t oc = __shfl_xor_sync(FULL_MASK, bc, o);
+        kid += shfl_xor_i64(kid, o);
+        if (team_better(osc, oc, bsc, bc)) { bsc = osc; bc = oc; }
+      }
+      const int first = k ? ps[k - 1] : 0, items = ps[k] - first;
+      int lastone = 0;
+      if (lane == 0) {
+        a.part_sc[w] = (i128)bsc;
+        a.part_c[w] = bc;
+        a.part_kid[w] = kid;
+        __threadfence();
+        lastone = atomicAdd(&done[k], 1) == items - 1;
+      }
+      if (__shfl_sync(FULL_MASK, lastone, 0)) {
+        __threadfence();
+        // the hub's chunks are all in: reduce them and decide
+        bsc = 0;
+        bc = INT32_MAX;
+        kid = 0;
+        for (int x = lane; x < items; x += 32) {
+          const int32_t oc = __ldcg(&a.part_c[first + x]);
+          const u64 *q = reinterpret_cast<const u64 *>(&a.part_sc[first + x]);
+          const u64 lo = __ldcg(q), hi = __ldcg(q + 1);
+          const ST osc = (ST)(i128)(((unsigned __int128)hi << 64) | (unsigned __int128)lo);
+          kid += __ldcg(&a.part_kid[first + x]);
+          if (team_better(osc, oc, bsc, bc)) { bsc = osc; bc = oc; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const ST osc = shfl_xor_any<ST>(bsc, o);
+          const int32_t oc = __shfl_xor_sync(FULL_MASK, bc, o);
+          kid += shfl_xor_i64(kid, o);
+          if (team_better(osc, oc, bsc, bc)) { bsc = osc; bc = oc; }
+        }
+        TeamHead h{};
+        i128 Sx = 0;
+        bool propose = false;
+        if (lane == 0) {
+          done[k] = 0;
+          if (!REFINE) a.processed[i] = 1;   // prune: the class's hub bits are already taken
+          h = team_head(g, a, i);
+          st.scanned += h.deg;
+          st.nvert++;
+          propose = team_rule<REFINE, ST>(a, ct, Ki, h.Sd, bsc, bc, kid, &Sx);
+        }
+        team_propose<REFINE, ST>(a, sw, sm, propose, i, bc, h, Sx, st);
+      }
+    }
+    bar_named(2 + sub, TEAM_SUB);   // the r_* words are read before the next item
+  }
+}
+
 // Decisions of one colour class.  The longest rows come first, and each
 // tier's first worker follows the last one of the tier before it, so a short
 // class spreads over the team.
+// Returns false after an expired wait.
 template <bool REFINE, typename WT, typename ST>
-__device__ __forceinline__ void team_decide_class(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
-                                                  const Team &t, int s, TeamSweep sw, int32_t *keys,
+__device__ __forceinline__ bool team_decide_class(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+                                                  Team &t, int s, TeamSweep sw, int32_t *keys,
                                                   typename TableVal<ST>::type *vals, TeamShared<ST> &sm,
                                                   TeamStat &st) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -621,6 +905,16 @@ __device__ __forceinline__ void team_decide_class(const TeamLevel<WT> &g, const 
   const int32_t *ko = &sm.koff[s];   // tier q of the class: ko[q * S] .. ko[q * S + 1]
   const int nb = t.nb;
   int rot = 0;   // blocks already given a first item
+  const int m7 = ko[7 * S + 1] - ko[7 * S], hub0 = ko[7 * S] - sm.koff[7 * S];
+  bool hubs = false;
+  if (m7 > 0) {
+    hubs = team_hub_bits<REFINE, ST>(a, ct, a.vlist + ko[7 * S], m7, sm);
+    if (hubs)
+      team_hub_insert<REFINE, WT, ST>(g, a, t, a.vlist + ko[7 * S], a.hub_i + hub0, a.hub_s + hub0, m7, keys +
+                                      threadIdx.x / TEAM_SUB * (TEAM_WSLOTS * (TEAM_SUB / 32)), vals +
+                                      threadIdx.x / TEAM_SUB * (TEAM_WSLOTS * (TEAM_SUB / 32)), sm);
+    if (ko[6 * S + 1] > ko[6 * S]) __syncthreads();   // the block tier pools the sub-blocks' tables
+  }
   const int m6 = ko[6 * S + 1] - ko[6 * S];
   if (m6 > 0) {
     team_decide_group<TEAM_THREADS, REFINE, WT, ST>(g, a, ct, a.vlist + ko[6 * S], m6, t.rank, nb, 1, 0, sw, keys,
@@ -680,6 +974,11 @@ __device__ __forceinline__ void team_decide_class(const TeamLevel<WT> &g, const 
     }
     __syncwarp();
   }
+  if (hubs) {
+    if (!t.sync()) return false;
+    team_hub_scan<REFINE, WT, ST>(g, a, ct, t, a.vlist + ko[7 * S], a.hub_s + hub0, a.hub_done + hub0, m7, sw, sm, st);
+  }
+  return true;
 }
 
 // Vertex pruning: `nl` lanes re-mark entries l, l + nl, ... of a row, U of
@@ -705,7 +1004,8 @@ __device__ __forceinline__ void team_remark(const TeamLevel<WT> &g, uint8_t *pro
 // team's overflow list (nover entries).
 template <typename WT, typename ST>
 __device__ __forceinline__ void team_apply_moves(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
-                                                 const Team &t, unsigned np, unsigned nover, TeamShared<ST> &sm) {
+                                                 const Team &t, unsigned np, unsigned nover, unsigned npiece,
+                                                 TeamShared<ST> &sm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x < np) {
     const TeamProp p = sm.prop[threadIdx.x];
@@ -714,18 +1014,21 @@ __device__ __forceinline__ void team_apply_moves(const TeamLevel<WT> &g, const T
     a.C[p.i] = p.c;
     if (ct.dynamic) { a.ch[p.d] = 1; a.ch[p.c] = 1; }
   }
-  // rows of up to 64 entries: eight lanes each; up to 2048: a warp; longer
-  // ones: the block
-  constexpr int SHORT = 64, MID = 2048;
+  // rows of up to 64 entries: eight lanes each; up to REMARK_PIECE: a warp;
+  // longer ones: in pieces over the team's warps
+  constexpr int SHORT = 64;
   for (unsigned m = threadIdx.x >> 3; m < np; m += TEAM_THREADS / 8)
     if (sm.prop[m].len <= SHORT) team_remark<4>(g, a.processed, sm.prop[m].e0, sm.prop[m].len, lane & 7, 8);
   for (unsigned m = warp; m < np; m += TEAM_WARPS)
-    if (sm.prop[m].len > SHORT && sm.prop[m].len <= MID)
+    if (sm.prop[m].len > SHORT && sm.prop[m].len <= REMARK_PIECE)
       team_remark<8>(g, a.processed, sm.prop[m].e0, sm.prop[m].len, lane, 32);
-  for (unsigned m = 0; m < np; m++)
-    if (sm.prop[m].len > MID) team_remark<4>(g, a.processed, sm.prop[m].e0, sm.prop[m].len, threadIdx.x, TEAM_THREADS);
-  if (!nover) return;
   const unsigned gt = t.index(), nt = t.nb * TEAM_THREADS;
+  for (unsigned m = gt >> 5; m < npiece; m += nt >> 5) {
+    const int32_t i = a.piece_i[m];
+    const int64_t e0 = g.off[i] + (int64_t)a.piece_k[m] * REMARK_PIECE, left = g.off[i + 1] - e0;
+    team_remark<8>(g, a.processed, e0, left < REMARK_PIECE ? (int)left : REMARK_PIECE, lane, 32);
+  }
+  if (!nover) return;
   for (unsigned m = gt; m < nover; m += nt) {
     const int32_t i = a.prop_i[m], c = a.prop_c[m], d = a.C[i];
     const int64_t Ki = a.K[i];
@@ -744,7 +1047,7 @@ __device__ __forceinline__ void team_apply_moves(const TeamLevel<WT> &g, const T
     const int32_t i = a.prop_i[m];
     const int64_t e0 = g.off[i];
     const int len = (int)(g.off[i + 1] - e0);
-    if (len > SHORT) team_remark<8>(g, a.processed, e0, len, lane, 32);
+    if (len > SHORT && len <= REMARK_PIECE) team_remark<8>(g, a.processed, e0, len, lane, 32);
   }
 }
 
@@ -831,7 +1134,7 @@ __device__ __forceinline__ bool team_lists(const TeamLevel<WT> &g, const TeamArr
   const int64_t b0 = seg * t.rank < g.n ? seg * t.rank : g.n, b1 = b0 + seg < g.n ? b0 + seg : g.n;
   for (int64_t v = b0 + threadIdx.x; v < b1; v += TEAM_THREADS) {
     const int64_t deg = g.off[v + 1] - g.off[v];
-    if (deg > 0) atomicAdd(&hist[(team_tier(deg) << log2S) + det_class((int32_t)v, log2S)], 1);
+    if (deg > 0) atomicAdd(&hist[(team_tier(deg, g.n) << log2S) + det_class((int32_t)v, log2S)], 1);
   }
   __syncthreads();
   for (int k = threadIdx.x; k < nk; k += TEAM_THREADS)
@@ -872,7 +1175,7 @@ __device__ __forceinline__ bool team_lists(const TeamLevel<WT> &g, const TeamArr
   for (int64_t v = b0 + threadIdx.x; v < b1; v += TEAM_THREADS) {
     const int64_t deg = g.off[v + 1] - g.off[v];
     if (deg > 0)
-      a.vlist[atomicAdd(&hist[(team_tier(deg) << log2S) + det_class((int32_t)v, log2S)], 1)] = (int32_t)v;
+      a.vlist[atomicAdd(&hist[(team_tier(deg, g.n) << log2S) + det_class((int32_t)v, log2S)], 1)] = (int32_t)v;
   }
   return t.sync();
 }
@@ -885,7 +1188,7 @@ __device__ __forceinline__ int team_local_move(const TeamLevel<WT> &g, const Tea
   const int S = 1 << ct.log2S;
   TeamCtl *ctl = t.ctl;
   int li = 0;
-  TeamSweep sw{0, 0, true, nullptr};
+  TeamSweep sw{0, 0, true, nullptr, nullptr};
   int64_t moves = 0;
   while (li < max_iters) {
     st.S = 0;
@@ -894,10 +1197,11 @@ __device__ __forceinline__ int team_local_move(const TeamLevel<WT> &g, const Tea
       u64 t0 = 0;
       if (ct.timing && t.rank == 0 && threadIdx.x == 0) asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
       sw.nover = &ctl->nover[sw.par];
+      sw.npiece = &ctl->npiece[sw.par];
       // headers alongside the eligibility test while most listed vertices are
       // eligible or the class is too short to fill the team anyway
       sw.spec = (li == 0 && !ct.dynamic) || sm.koff[TEAM_TIERS * S] <= t.nb * TEAM_THREADS;
-      team_decide_class<false, WT, ST>(g, a, ct, t, s, sw, keys, vals, sm, st);
+      if (!team_decide_class<false, WT, ST>(g, a, ct, t, s, sw, keys, vals, sm, st)) return 0;
       if (s == S - 1) {
         // the iteration's sum of scores, one addition per block
         i128 acc = st.S;
@@ -917,7 +1221,7 @@ __device__ __forceinline__ int team_local_move(const TeamLevel<WT> &g, const Tea
         ctl->decide_ns += t1 - t0;
         ctl->subsweeps++;
       }
-      const unsigned nover = __ldcg(sw.nover);
+      const unsigned nover = __ldcg(sw.nover), npiece = __ldcg(sw.npiece);
       unsigned np = sm.nprop[sw.par];
       np = np < TEAM_PROPS ? np : TEAM_PROPS;
       if (threadIdx.x == 0) {
@@ -926,11 +1230,12 @@ __device__ __forceinline__ int team_local_move(const TeamLevel<WT> &g, const Tea
         moves += np;
         if (t.rank == 0) {
           ctl->nover[sw.par ^ 1] = 0;
+          ctl->npiece[sw.par ^ 1] = 0;
           moves += nover;
           if (s == 0) { ctl->sums[(li & 1) ^ 1][0] = 0; ctl->sums[(li & 1) ^ 1][1] = 0; }
         }
       }
-      if (np | nover) team_apply_moves<WT, ST>(g, a, ct, t, np, nover, sm);
+      if (np | nover | npiece) team_apply_moves<WT, ST>(g, a, ct, t, np, nover, npiece, sm);
       TEAM_SYNC_OR(0);
     }
     li++;
@@ -960,7 +1265,7 @@ __device__ __forceinline__ bool team_refine(const TeamLevel<WT> &g, const TeamAr
   TeamCtl *ctl = t.ctl;
   const int gt = t.index(), nt = t.nb * TEAM_THREADS;
   TeamStat st{};
-  TeamSweep sw{0, 0, true, nullptr};
+  TeamSweep sw{0, 0, true, nullptr, nullptr};
   int64_t moved = 0;
   for (int s = 0; s < S; s++, sw.par ^= 1) {
     // stamps 1..255 name the sub-sweep a vertex proposed in; a stamp only
@@ -972,7 +1277,7 @@ __device__ __forceinline__ bool team_refine(const TeamLevel<WT> &g, const TeamAr
     }
     sw.nover = &ctl->nover[sw.par];
     sw.spec = !ct.dynamic;   // every vertex starts isolated in a changed bound, but for an update's first pass
-    team_decide_class<true, WT, ST>(g, a, ct, t, s, sw, keys, vals, sm, st);
+    if (!team_decide_class<true, WT, ST>(g, a, ct, t, s, sw, keys, vals, sm, st)) return false;
     TEAM_SYNC_OR(false);
     const unsigned nover = __ldcg(sw.nover);
     unsigned np = sm.nprop[sw.par];
@@ -1031,7 +1336,7 @@ __device__ __forceinline__ bool team_aggregate(const TeamLevel<WT> &g, const Tea
   const int64_t gt = t.index(), nt = (int64_t)t.nb * TEAM_THREADS;
   const int32_t *ko = sm.koff;
   // rows of more than TT_WARP8 entries: the block each
-  for (int r = ko[5 * S] + t.rank; r < ko[7 * S]; r += t.nb) {
+  for (int r = ko[5 * S] + t.rank; r < ko[8 * S]; r += t.nb) {
     const int32_t v = a.vlist[r];
     const int64_t e0 = g.off[v], e1 = g.off[v + 1];
     const int32_t c = a.C[v];
@@ -1158,6 +1463,10 @@ __device__ __forceinline__ void team_pass(const TeamLevel<WT> &g, TeamArrays a, 
   for (int k = threadIdx.x; k < TEAM_WARPS * TEAM_WSLOTS; k += TEAM_THREADS) { keys[k] = LEIDEN_EMPTY_KEY; vals[k] = 0; }
   if (threadIdx.x < 2) sm.nprop[threadIdx.x] = 0;
   __syncthreads();
+  if (!team_hub_setup<WT, ST>(g, a, 1 << ct.log2S, t, sm)) {
+    if (!t.dead && t.rank == 0 && threadIdx.x == 0) ctl->status = TEAM_TOO_BIG;
+    return;
+  }
   const int li = team_local_move<WT, ST>(g, a, ct, tau, max_iters, t, keys, vals, sm, st);
   if (t.dead) return;
   for (int o = 16; o; o >>= 1) {

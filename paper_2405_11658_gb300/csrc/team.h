@@ -11,27 +11,33 @@ namespace lk {
 enum { TEAM_BLOCK = 0, TEAM_CLUSTER = 1, TEAM_GRID = 2 };
 // How a team pass ended: globally converged after the refinement; renumbered
 // to as many communities as vertices (aggregation would not shrink the
-// graph); renumbered only (the caller aggregates); aggregated.
-enum { TEAM_NONE = 0, TEAM_CONVERGED = 1, TEAM_NO_SHRINK = 2, TEAM_RENUMBERED = 3, TEAM_AGGREGATED = 4 };
+// graph); renumbered only (the caller aggregates); aggregated; nothing done,
+// the level's hubs exceed the scratch.
+enum { TEAM_NONE = 0, TEAM_CONVERGED = 1, TEAM_NO_SHRINK = 2, TEAM_RENUMBERED = 3, TEAM_AGGREGATED = 4, TEAM_TOO_BIG = 5 };
 
+// Distinct candidates of a vertex the block's table takes (half its slots);
+// vertices with more are hubs.  Hubs per colour class at most.
+static constexpr int64_t TEAM_MAX_CAND = 8192;
+static constexpr int TEAM_MAX_HUBS = 16384;
 static constexpr int TEAM_MAX_BLOCKS = 1024;
 static constexpr u64 TEAM_SPIN_LIMIT = 1ull << 24;   // polls of a grid barrier (several seconds)
 
 // Control words of a team, zeroed before every pass.
 struct TeamCtl {
   unsigned bar, abort;
+  unsigned npiece[2];      // row pieces the whole team re-marks, by parity
   unsigned nover[2];       // proposals beyond the blocks' own lists, by parity of the sub-sweep
   u64 sums[2][2];          // sum of S of the current / next iteration (i128)
   u64 scanned_e, scanned_v, cand, changed, rmoves;
   int64_t moves;
-  int32_t li, status;
+  int32_t li, status, too_big, pad0;
   int64_t nc, nnz2;
   u64 maxdeg, kmax;        // of the aggregated level
   u64 decide_ns, subsweeps;
   u64 stamp[4];            // globaltimer at the start and after local-moving, refinement, aggregation
   // end of the part the host reads back
   int64_t part[TEAM_MAX_BLOCKS];
-  unsigned ktot[256 * 7], kcur[256 * 7];
+  unsigned ktot[256 * 8], kcur[256 * 8];
 };
 static constexpr size_t TEAM_CTL_HEAD = offsetof(TeamCtl, part);
 
@@ -42,6 +48,16 @@ struct TeamArrays {
   uint8_t *ch, *ch2, *processed, *stamp, *exists;
   int32_t *prop_i, *prop_c;
   u64 *err;
+  // hubs: table scratch (tcap slots, empty whenever nobody uses it), prefix
+  // sums of insert and scan items, finished scan items and their results
+  int32_t *tkeys;
+  u64 *tvals;
+  int64_t tcap;
+  int32_t *hub_i, *hub_s, *hub_done, *part_c;
+  i128 *part_sc;
+  int64_t *part_kid;
+  // long rows to re-mark: mover and piece (at most 2 * nnz / REMARK_PIECE)
+  int32_t *piece_i, *piece_k;
   // aggregation: table keys and sums, row entry counts and cursors, row sums,
   // and the output graph
   u64 *hkey, *hval;
@@ -67,9 +83,6 @@ struct TeamArgs {
   const uint8_t *in_range;
   TeamCtl *ctl;
 };
-// Distinct candidates a vertex may have on the team path (its table is never
-// more than half full).
-static constexpr int64_t TEAM_MAX_CAND = 8192;
 // Launches the pass over nb blocks (one per SM at most) as `kind`.
 static constexpr int TEAM_MAX_CLUSTER = 16;
 template <typename WT, typename ST>

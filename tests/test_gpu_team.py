@@ -20,15 +20,17 @@ import paper_2405_11658_gb300 as L  # noqa: E402
 
 # one below, at and above the last degree of every tier
 EDGES = (7, 8, 9, 15, 16, 17, 31, 32, 33, 127, 128, 129, 255, 256, 257, 2047, 2048, 2049)
+HUBS = (8191, 8192, 8193, 10240, 10241, 20000)
 
 
 def tiers_graph(n, wmax, seed):
-    """A random graph with, for every degree of EDGES, three vertices of about
-    that degree: star centres over random leaves."""
+    """A random graph with, for every degree of EDGES (and, where it has the
+    vertices, of HUBS), three vertices of about that degree: star centres over
+    random leaves."""
     rng = np.random.default_rng(seed)
     us, vs = [rng.integers(0, n, 3 * n)], [rng.integers(0, n, 3 * n)]
     centre = n
-    for d in EDGES:
+    for d in EDGES + (HUBS if n >= HUBS[-1] else ()):
         for _ in range(3):
             us.append(np.full(d, centre))
             vs.append(rng.choice(n, d, replace=False))
