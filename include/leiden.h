@@ -153,8 +153,8 @@ int leiden_update(leiden_ctx *ctx, const leiden_csr *g_t,
                   double *q_out);
 
 /* Modularity (Eq. 1 at resolution gamma) of membership (DEVICE [n], labels
- * in [0, n)) on g.  q_out is HOST.  The graph and the labels are validated
- * on the device, and the verdict read, before any kernel indexes by them.
+ * in [0, n)) on g.  q_out is HOST.  The graph and the labels are validated in
+ * the pass that sums them: every index is tested before it is used.
  * Errors: LEIDEN_EINVAL (malformed graph, label out of range, bad gamma),
  * LEIDEN_ENOMEM, LEIDEN_EOVERFLOW (nnz > 2^32 or 2m >= 2^40), LEIDEN_ECUDA. */
 int leiden_modularity(leiden_ctx *ctx, const leiden_csr *g, const int32_t *membership,
@@ -235,8 +235,8 @@ int leiden_ctx_set_timing(leiden_ctx *ctx, int32_t enable);
  * the same integer arithmetic as leiden_modularity; the work is ordered on
  * cuda_stream (cudaStream_t as void*, NULL = legacy default stream), which the
  * call synchronises before writing q_out (HOST).  The graph and the labels
- * are validated, and the verdict read on the host, before any kernel indexes
- * by them; the kernels that compute the terms test every index as well.
+ * are validated in the pass that sums them: every index is tested before it
+ * is used.
  * Errors: LEIDEN_EINVAL (bad gamma, malformed graph, label out of range),
  * LEIDEN_ENOMEM (n too large), LEIDEN_EOVERFLOW (nnz > 2^32 or 2m >= 2^40),
  * LEIDEN_ECUDA. */

@@ -818,6 +818,13 @@ int run_leiden(Run &r, const leiden_csr *g0) {
   return check_cuda(c);
 }
 
+// A check found the caller's CSR malformed (flags in h_ctr[CTR_ERROR]).
+int malformed(leiden_ctx *c) {
+  snprintf(c->err, sizeof(c->err), "malformed CSR or labels (flags 0x%llx)", c->h_ctr[CTR_ERROR]);
+  cudaMemsetAsync(&c->ctr[CTR_ERROR], 0, sizeof(u64), c->st);
+  return LEIDEN_EINVAL;
+}
+
 // Device-side validation of a caller's CSR (off, idx, w); LEIDEN_EINVAL on a
 // malformed graph.  One read of the graph, so the kernels after it can index
 // by the graph's own IDs without further checks.
@@ -827,14 +834,11 @@ int validate_graph(leiden_ctx *c, const leiden_csr *g) {
   cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   int rc = sync(c);
   if (rc) return rc;
-  if (c->h_ctr[CTR_ERROR]) {
-    snprintf(c->err, sizeof(c->err), "malformed CSR (flags 0x%llx)", c->h_ctr[CTR_ERROR]);
-    cudaMemsetAsync(&c->ctr[CTR_ERROR], 0, sizeof(u64), c->st);
-    return LEIDEN_EINVAL;
-  }
-  return LEIDEN_OK;
+  return c->h_ctr[CTR_ERROR] ? malformed(c) : LEIDEN_OK;
 }
 
+// Checks the arguments and the graph and takes K (row sums, into K0) and 2m
+// in the same pass over the graph.
 int setup_run(leiden_ctx *c, const leiden_csr *g, const leiden_opts *o, Run &r) {
   r.c = c;
   r.o = o;
@@ -843,23 +847,22 @@ int setup_run(leiden_ctx *c, const leiden_csr *g, const leiden_opts *o, Run &r) 
   if (rc) return rc;
   rc = check_graph(c, g);
   if (rc) return rc;
-  rc = validate_graph(c, g);
+  cudaMemsetAsync(&c->ctr[CTR_ERROR], 0, sizeof(u64), c->st);
+  launch_row_sums(GraphView<int32_t>{g->n, g->off, g->idx, g->w}, g->nnz, c->K0, &c->ctr[CTR_SCRATCH0],
+                  &c->ctr[CTR_ERROR], c->st);
+  cudaMemcpyAsync(c->h_ctr, c->ctr, CTR_COUNT * sizeof(u64), cudaMemcpyDeviceToHost, c->st);
+  rc = sync(c);
   if (rc) return rc;
+  if (c->h_ctr[CTR_ERROR]) return malformed(c);
+  r.two_m = (int64_t)c->h_ctr[CTR_SCRATCH0 + 3];
+  r.A = r.two_m * r.q;
   r.N = g->n;
   return LEIDEN_OK;
 }
 
-int finish_two_m(leiden_ctx *c, Run &r, const leiden_csr *g) {
-  // 2m = total CSR weight of G^t, from its row sums (K0)
-  cudaMemsetAsync(&c->ctr[CTR_SCRATCH0], 0, sizeof(u64), c->st);
-  launch_sum_i64(c->K0, g->n, &c->ctr[CTR_SCRATCH0], c->st);
-  cudaMemcpyAsync(&c->h_ctr[CTR_SCRATCH0], &c->ctr[CTR_SCRATCH0], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
-  int rc = sync(c);
-  if (rc) return rc;
-  r.two_m = (int64_t)c->h_ctr[CTR_SCRATCH0];
-  if (r.two_m < 0 || r.two_m >= ((int64_t)1 << 40)) return LEIDEN_EOVERFLOW;
-  r.A = r.two_m * r.q;
-  return LEIDEN_OK;
+// Every 2m a run accepts (its products stay within 128 bits).
+int check_two_m(const Run &r) {
+  return r.two_m < 0 || r.two_m >= ((int64_t)1 << 40) ? LEIDEN_EOVERFLOW : LEIDEN_OK;
 }
 
 // The u64 accumulators of Eq. 1 cannot wrap while nnz <= 2^32 (each weight is
@@ -867,20 +870,25 @@ int finish_two_m(leiden_ctx *c, Run &r, const leiden_csr *g) {
 // while 2m < 2^40 (the bound every run checks).
 constexpr int64_t kModMaxNnz = (int64_t)1 << 32;
 
-int modularity_of(leiden_ctx *c, const leiden_csr *g, const int32_t *C, int64_t p, int64_t q, double *q_out) {
-  if (g->nnz > kModMaxNnz) return LEIDEN_EOVERFLOW;
+// Modularity of C on g; `unchecked`: the caller's graph and labels have not
+// been validated yet (a bad one gets LEIDEN_EINVAL).
+int modularity_of(leiden_ctx *c, const leiden_csr *g, const int32_t *C, int64_t p, int64_t q, bool unchecked,
+                  double *q_out) {
+  if (!unchecked && g->nnz > kModMaxNnz) return LEIDEN_EOVERFLOW;
   GraphView<int32_t> gv{g->n, g->off, g->idx, g->w};
   launch_modularity_terms(gv, g->nnz, C, c->Ktmp, &c->ctr[CTR_SCRATCH0], &c->ctr[CTR_ERROR], c->st);
   cudaMemcpyAsync(&c->h_ctr[CTR_SCRATCH0], &c->ctr[CTR_SCRATCH0], 4 * sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   int rc = sync(c);
   if (rc) return rc;
+  if (c->h_ctr[CTR_ERROR] && unchecked) return malformed(c);
   if (c->h_ctr[CTR_ERROR]) {
     // the callers validated the graph and the labels first, so this is an
     // internal inconsistency; the kernels skipped every bad index
     cudaMemsetAsync(&c->ctr[CTR_ERROR], 0, sizeof(u64), c->st);
     return check_dev_flags(c, c->h_ctr[CTR_ERROR]);
   }
+  if (g->nnz > kModMaxNnz) return LEIDEN_EOVERFLOW;
   const int64_t inside = (int64_t)c->h_ctr[CTR_SCRATCH0];
   const i128 sq = read_i128(&c->h_ctr[CTR_SCRATCH0 + 1]);
   const int64_t two_m = (int64_t)c->h_ctr[CTR_SCRATCH0 + 3];
@@ -1157,9 +1165,7 @@ int leiden_static(leiden_ctx *c, const leiden_csr *g, const leiden_opts *o, int3
   if (rc) return rc;
   reset_stats(c);
   const int64_t n = g->n;
-  GraphView<int32_t> gv{n, g->off, g->idx, g->w};
-  launch_row_sums(gv, c->K0, c->st);
-  rc = finish_two_m(c, r, g);
+  rc = check_two_m(r);
   if (rc) return rc;
   // Static: C' = identity, K' = K, Sigma' = K, every community changed,
   // every vertex affected and in range
@@ -1177,7 +1183,7 @@ int leiden_static(leiden_ctx *c, const leiden_csr *g, const leiden_opts *o, int3
   rc = sync(c);
   if (rc) return rc;
   if (q_out) {
-    rc = modularity_of(c, g, membership_out, r.p, r.q, q_out);
+    rc = modularity_of(c, g, membership_out, r.p, r.q, false, q_out);
     if (rc) return rc;
   }
   finish_timing(c);
@@ -1220,9 +1226,7 @@ int leiden_update(leiden_ctx *c, const leiden_csr *g, const int32_t *prior_membe
     return LEIDEN_EINVAL;
   }
 
-  GraphView<int32_t> gv{n, g->off, g->idx, g->w};
-  launch_row_sums(gv, c->K0, c->st);  // K^t of G^t, also the source of 2m
-  rc = finish_two_m(c, r, g);
+  rc = check_two_m(r);
   if (rc) return rc;
   // Alg. update: K^t, Sigma^t from the auxiliary information, or recomputed
   if (prior_K) {
@@ -1275,7 +1279,7 @@ int leiden_update(leiden_ctx *c, const leiden_csr *g, const int32_t *prior_membe
   rc = sync(c);
   if (rc) return rc;
   if (q_out) {
-    rc = modularity_of(c, g, membership_out, r.p, r.q, q_out);
+    rc = modularity_of(c, g, membership_out, r.p, r.q, false, q_out);
     if (rc) return rc;
   }
   finish_timing(c);
@@ -1289,21 +1293,12 @@ int leiden_modularity(leiden_ctx *c, const leiden_csr *g, const int32_t *members
   int rc = check_graph(c, g);
   if (rc) return rc;
   if (g->n > 0 && !membership) return LEIDEN_EINVAL;
-  rc = validate_graph(c, g);
-  if (rc) return rc;
-  cudaMemsetAsync(&c->ctr[CTR_ERROR], 0, sizeof(u64), c->st);
-  launch_check_range(membership, g->n, g->n, &c->ctr[CTR_ERROR], c->st);
-  cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
-  rc = sync(c);
-  if (rc) return rc;
-  if (c->h_ctr[CTR_ERROR]) {
-    cudaMemsetAsync(&c->ctr[CTR_ERROR], 0, sizeof(u64), c->st);
-    return LEIDEN_EINVAL;
-  }
   int64_t p, q;
   rc = gamma_ratio(gamma, &p, &q);
   if (rc) return rc;
-  return modularity_of(c, g, membership, p, q, q_out);
+  cudaMemsetAsync(&c->ctr[CTR_ERROR], 0, sizeof(u64), c->st);
+  // the terms kernel tests every index before it uses it
+  return modularity_of(c, g, membership, p, q, true, q_out);
 }
 
 int leiden_apply_batch(leiden_ctx *c, const leiden_csr *g, const leiden_edges *del, const leiden_edges *ins,

@@ -241,14 +241,14 @@ void exclusive_scan(const TI *in, int64_t *out, int64_t n, int64_t *tmp, cudaStr
 int64_t scan_tmp_elems(int64_t n);
 
 // misc.cu
-template <typename WT>
-void launch_row_sums(GraphView<WT> g, int64_t *K, cudaStream_t s);
+// One pass that checks a CSR of nnz entries (a malformed one sets 512 in *err;
+// nothing outside the arrays is touched) and writes K; acc[3] = 2m.
+void launch_row_sums(GraphView<int32_t> g, int64_t nnz, int64_t *K, u64 *acc, u64 *err, cudaStream_t s);
 void launch_iota(int32_t *a, int64_t n, cudaStream_t s);
 void launch_fill_u8(uint8_t *a, uint8_t v, int64_t n, cudaStream_t s);
 void launch_copy_i64(int64_t *dst, const int64_t *src, int64_t n, cudaStream_t s);
 void launch_invert_u8(uint8_t *dst, const uint8_t *src, int64_t n, cudaStream_t s);
 void launch_clear_left(int64_t *Sig, int64_t n, cudaStream_t s);
-void launch_sum_i64(const int64_t *a, int64_t n, u64 *out, cudaStream_t s);
 void launch_subset_renumber(int64_t n, int32_t *C, const int64_t *Sig, int64_t *Sig2,
                             const uint8_t *ch, uint8_t *ch2, int32_t *rep, cudaStream_t s);
 void launch_break(int64_t n, int32_t *C, const int64_t *K, int64_t *Sig, const uint8_t *ch,
@@ -260,11 +260,9 @@ void launch_lookup(int64_t n, int32_t *Ctop, const int32_t *Cp, cudaStream_t s);
 void launch_canonical(int64_t n, const int32_t *C, int32_t *out, int32_t *minv, uint8_t *flag,
                       int64_t *scanned, int64_t *tmp, cudaStream_t s);
 // Eq. 1 terms of membership C on g (nnz entries): acc[0] internal weight,
-// acc[1..2] sum of Sigma_c^2 (i128), acc[3] 2m.  Bounds-checked: a bad row,
-// label or column ID is skipped and sets 512 in *err; nothing runs when *err
-// is already set.
-template <typename WT>
-void launch_modularity_terms(GraphView<WT> g, int64_t nnz, const int32_t *C, int64_t *Sig_tmp, u64 *acc,
+// acc[1..2] sum of Sigma_c^2 (i128), acc[3] 2m.  Checks as launch_row_sums,
+// and the labels against [0, n).
+void launch_modularity_terms(GraphView<int32_t> g, int64_t nnz, const int32_t *C, int64_t *Sig_tmp, u64 *acc,
                              u64 *err, cudaStream_t s);
 void launch_update_weights(int64_t count, const int32_t *src, const int32_t *dst,
                            const int32_t *w, int sign, const int32_t *Cprev, int64_t *K,

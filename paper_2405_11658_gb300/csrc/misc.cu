@@ -20,26 +20,176 @@ static inline unsigned grid_for(int64_t n, int threads, int64_t cap = 1 << 20) {
 #define GRID_STRIDE(i, n) \
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += (int64_t)gridDim.x * blockDim.x)
 
-// K_i = sum of the row (self-loop included once), warp per vertex.
-template <typename WT>
-__global__ void row_sums_k(GraphView<WT> g, int64_t *K) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = w0; i < g.n; i += nw) {
-    int64_t s = 0;
-    for (int64_t e = g.off[i] + lane; e < g.off[i + 1]; e += 32) s += (int64_t)g.w[e];
-    for (int o = 16; o; o >>= 1) s += shfl_xor_i64(s, o);
-    if (lane == 0) K[i] = s;
+// ---------------------------------------------------------------------------
+// One pass over a CSR that checks it and sums its rows (K_i, self-loop
+// included once, and 2m) or takes the terms of Eq. 1.
+//
+// Bound by the stream of idx and w (8 bytes an entry) and, for Eq. 1, by the
+// gathers of C[j] from L2.  A warp takes `ch` consecutive items of the merged
+// sequence of entries and row ends (entry e of row i is item e + i), found by
+// a 32-way search of the row offsets, so heavy rows, runs of empty rows and
+// ordinary ones all split evenly: with the rows dealt out instead, the block
+// with R-MAT scale 22's first rows took 4.8 ms, the whole pass takes 1.0
+// ms here (3.4 ms with a warp and an atomic per row).  G lanes share a short
+// row (2 where rows have up to 8 entries on average, else 8), four entries per
+// lane in flight; longer pieces take the whole warp.  32 rows' totals meet
+// per community before they reach Sigma: neighbouring vertices often share
+// one, and an atomic per vertex queued on a few addresses.
+//
+// The offsets and labels are checked by check_graph_rows_k; this kernel tests
+// every index before it uses it all the same -- the row bounds against
+// [0, nnz], the labels and column IDs against [0, n) -- so a malformed input
+// can never make it read or write outside the arrays: an offending row or
+// entry is skipped and sets 512 in *err, as does a weight that is not
+// positive.  K and Sigma are zero on entry.
+// ---------------------------------------------------------------------------
+static constexpr int ROWS_THREADS = 256, ROWS_WARPS = ROWS_THREADS / 32;
+template <int G, bool MOD>
+__global__ void __launch_bounds__(ROWS_THREADS) rows_k(GraphView<int32_t> g, int64_t nnz, const int32_t *C, int64_t *K,
+                                                       int64_t *Sig, u64 *acc, u64 *err, int64_t ch) {
+  __shared__ int64_t sbuf[32];
+  __shared__ u64 wscr[ROWS_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t inside = 0, total = 0;
+  bool bad = false;
+  // entries first, first + step, ... < e1 of a row of community ci
+  auto part = [&](int64_t first, int64_t e1, int64_t step, int32_t ci) -> int64_t {
+    int64_t k = 0;
+    for (int64_t e = first; e < e1; e += 4 * step) {
+      int32_t j[4], w[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const bool in = e + u * step < e1;
+        j[u] = in ? g.idx[e + u * step] : 0;
+        w[u] = in ? g.w[e + u * step] : 0;
+        if (in && (j[u] < 0 || (int64_t)j[u] >= g.n || w[u] <= 0)) { bad = true; w[u] = 0; j[u] = 0; }
+      }
+      if (MOD) {
+        int32_t cj[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) cj[u] = w[u] ? C[j[u]] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+          if (cj[u] == ci) inside += w[u];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; u++) k += w[u];
+    }
+    return k;
+  };
+  const int64_t items = g.n + nnz;
+  for (int64_t d0 = ((int64_t)warp * gridDim.x + blockIdx.x) * ch; d0 < items;
+       d0 += (int64_t)ROWS_WARPS * gridDim.x * ch) {   // uniform per warp
+    const int64_t d1 = d0 + ch < items ? d0 + ch : items;
+    // last row r with off[r] + r <= d0
+    int64_t r0 = 0, len = g.n;
+    while (len > 1) {
+      const int64_t step = (len + 31) / 32, r = r0 + lane * step;
+      const unsigned m = __ballot_sync(FULL_MASK, lane * step < len && g.off[r] + r <= d0);
+      const int k = m ? 31 - __clz(m) : 0;
+      len = len - k * step < step ? len - k * step : step;
+      r0 += k * step;
+    }
+    int64_t windows = ch / 32 + 2;   // rows of the piece at most, 32 at a time
+    for (int64_t rb = r0; rb < g.n && windows > 0; rb += 32, windows--) {
+      const int64_t i = rb + lane;
+      int64_t e0 = 0, e1 = 0;
+      int32_t ci = -1;
+      bool mine = false, whole = false;
+      if (i < g.n) {
+        const int64_t a = g.off[i], b = g.off[i + 1];
+        mine = a + i < d1;
+        if (mine) {
+          if (MOD) ci = C[i];
+          if (a < 0 || b < a || b > nnz || (MOD && (ci < 0 || (int64_t)ci >= g.n))) {
+            bad = true;
+            ci = -1;
+          } else {
+            e0 = a + i >= d0 ? a : d0 - i;
+            e1 = b + i <= d1 ? b : d1 - i;
+            if (e1 < e0) e1 = e0;
+            whole = e0 == a && e1 == b;
+          }
+        }
+      }
+      if (!__any_sync(FULL_MASK, mine)) break;
+      const int64_t n_i = e1 - e0;
+      int64_t Ki = 0;
+      // short pieces, 32 / G at a time
+#pragma unroll 1
+      for (int it = 0; it < G; it++) {
+        const int src = it * (32 / G) + lane / G;
+        const int64_t a = shfl_i64(e0, src), b = shfl_i64(e1, src);
+        const int32_t c = __shfl_sync(FULL_MASK, ci, src);
+        int64_t k = b - a <= 16 * G ? part(a + lane % G, b, G, c) : 0;
+#pragma unroll
+        for (int o = G / 2; o; o >>= 1) k += shfl_xor_i64(k, o);
+        // row it * (32 / G) + q was summed by the lanes from q * G on
+        const int64_t v = shfl_i64(k, (lane % (32 / G)) * G);
+        if (lane / (32 / G) == it) Ki = v;
+      }
+      for (unsigned m = __ballot_sync(FULL_MASK, n_i > 16 * G); m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        int64_t k = part(shfl_i64(e0, src) + lane, shfl_i64(e1, src), 32, __shfl_sync(FULL_MASK, ci, src));
+        for (int o = 16; o; o >>= 1) k += shfl_xor_i64(k, o);
+        if (lane == src) Ki = k;
+      }
+      total += Ki;
+      if (MOD) {
+        u64 sum = 0;
+        if (warp_combine((unsigned long long)(uint32_t)ci, ci >= 0 && Ki != 0, (u64)Ki, &sum, wscr[warp]))
+          atomicAdd((u64 *)&Sig[ci], sum);
+      } else if (Ki != 0) {
+        if (whole) K[i] = Ki;
+        else atomic_add_i64(&K[i], Ki);   // a row shared with the neighbouring pieces
+      }
+    }
   }
+  if (bad) atomicOr(err, 512ull);
+  if (MOD) {
+    inside = block_sum_i64(inside, sbuf);
+    if (threadIdx.x == 0 && inside) atomicAdd(&acc[0], (u64)inside);
+  }
+  total = block_sum_i64(total, sbuf);
+  if (threadIdx.x == 0 && total) atomicAdd(&acc[3], (u64)total);
 }
-template <typename WT>
-void launch_row_sums(GraphView<WT> g, int64_t *K, cudaStream_t s) {
+
+// Row offsets: off[0] = 0, off[n] = nnz, non-decreasing; labels (if any) in
+// [0, n).  Sets *err on violation.
+__global__ void check_graph_rows_k(int64_t n, int64_t nnz, const int64_t *off, const int32_t *C, u64 *err) {
+  bool bad = blockIdx.x == 0 && threadIdx.x == 0 && (off[0] != 0 || off[n] != nnz);
+  GRID_STRIDE(i, n) {
+    const int64_t a = off[i], b = off[i + 1];
+    if (a > b || a < 0 || b > nnz) bad = true;
+    if (C && (C[i] < 0 || (int64_t)C[i] >= n)) bad = true;
+  }
+  if (bad) atomicOr(err, 128ull);
+}
+
+template <bool MOD>
+static void launch_rows(GraphView<int32_t> g, int64_t nnz, const int32_t *C, int64_t *K, int64_t *Sig, u64 *acc,
+                        u64 *err, cudaStream_t s) {
+  LK_COUNTED check_graph_rows_k<<<grid_for(g.n > 0 ? g.n : 1, 256, 152 * 32), 256, 0, s>>>(g.n, nnz, g.off, C, err);
   if (g.n <= 0) return;
-  LK_COUNTED row_sums_k<WT><<<grid_for(g.n * 32, 256, 152 * 64), 256, 0, s>>>(g, K);
+  auto k2 = rows_k<2, MOD>;
+  auto k8 = rows_k<8, MOD>;
+  const bool two = nnz <= 8 * g.n;
+  const int64_t cap = resident_blocks(two ? (const void *)k2 : (const void *)k8, ROWS_THREADS, 0, 152);
+  // pieces of 256 .. 2048 items, small ones where the graph is too short to
+  // give every resident warp one of the longer
+  int64_t ch = (g.n + nnz) / (cap * ROWS_WARPS);
+  ch = ch < 256 ? 256 : ch > 2048 ? 2048 : ch;
+  int64_t blocks = ((g.n + nnz + ch - 1) / ch + ROWS_WARPS - 1) / ROWS_WARPS;
+  if (blocks > cap) blocks = cap;
+  if (two) LK_COUNTED k2<<<(unsigned)blocks, ROWS_THREADS, 0, s>>>(g, nnz, C, K, Sig, acc, err, ch);
+  else LK_COUNTED k8<<<(unsigned)blocks, ROWS_THREADS, 0, s>>>(g, nnz, C, K, Sig, acc, err, ch);
 }
-template void launch_row_sums<int32_t>(GraphView<int32_t>, int64_t *, cudaStream_t);
-template void launch_row_sums<int64_t>(GraphView<int64_t>, int64_t *, cudaStream_t);
+
+void launch_row_sums(GraphView<int32_t> g, int64_t nnz, int64_t *K, u64 *acc, u64 *err, cudaStream_t s) {
+  cudaMemsetAsync(acc, 0, 4 * sizeof(u64), s);
+  if (g.n > 0) cudaMemsetAsync(K, 0, (size_t)g.n * sizeof(int64_t), s);
+  launch_rows<false>(g, nnz, nullptr, K, nullptr, acc, err, s);
+}
 
 __global__ void iota_k(int32_t *a, int64_t n) { GRID_STRIDE(i, n) a[i] = (int32_t)i; }
 void launch_iota(int32_t *a, int64_t n, cudaStream_t s) {
@@ -61,17 +211,6 @@ void launch_clear_left(int64_t *Sig, int64_t n, cudaStream_t s) {
 }
 void launch_invert_u8(uint8_t *dst, const uint8_t *src, int64_t n, cudaStream_t s) {
   if (n > 0) LK_COUNTED invert_u8_k<<<grid_for(n, 256), 256, 0, s>>>(dst, src, n);
-}
-
-__global__ void sum_i64_k(const int64_t *a, int64_t n, u64 *out) {
-  __shared__ int64_t sbuf[32];
-  int64_t s = 0;
-  GRID_STRIDE(i, n) s += a[i];
-  s = block_sum_i64(s, sbuf);
-  if (threadIdx.x == 0 && s) atomicAdd(out, (u64)s);
-}
-void launch_sum_i64(const int64_t *a, int64_t n, u64 *out, cudaStream_t s) {
-  if (n > 0) LK_COUNTED sum_i64_k<<<grid_for(n, 256, 152 * 8), 256, 0, s>>>(a, n, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -182,55 +321,8 @@ void launch_canonical(int64_t n, const int32_t *C, int32_t *out, int32_t *minv, 
   LK_COUNTED canon_out_k<<<g, 256, 0, s>>>(n, C, minv, scanned, out);
 }
 
-// ---------------------------------------------------------------------------
 // Eq. 1 terms: acc[0] = sum of internal weight (sum_c sigma_c), acc[1..2] =
 // sum_c Sigma_c^2 (i128), acc[3] = 2m.
-//
-// Every index is tested before it is used -- the row bounds against [0, nnz],
-// the labels and column IDs against [0, n) -- so a malformed input can never
-// make these kernels read or write outside the arrays, whatever the caller
-// has or has not validated: an offending row or entry is skipped and sets
-// 512 in *err.  A kernel that finds *err already set (an earlier check on
-// the same stream failed) does nothing.
-// ---------------------------------------------------------------------------
-template <typename WT>
-__global__ void mod_rows_k(GraphView<WT> g, int64_t nnz, const int32_t *C, int64_t *Sig, u64 *acc,
-                           u64 *err) {
-  __shared__ int64_t sbuf[32];
-  __shared__ int s_skip;
-  // one reading for the whole block, so no thread skips the barriers below
-  // while another waits at them
-  if (threadIdx.x == 0) s_skip = *(volatile u64 *)err != 0;
-  __syncthreads();
-  if (s_skip) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int64_t inside = 0, total = 0;
-  bool bad = false;
-  for (int64_t i = w0; i < g.n; i += nw) {
-    const int64_t e0 = g.off[i], e1 = g.off[i + 1];
-    const int32_t ci = C[i];
-    if (e0 < 0 || e1 < e0 || e1 > nnz || ci < 0 || (int64_t)ci >= g.n) { bad = true; continue; }
-    int64_t k = 0;
-    for (int64_t e = e0 + lane; e < e1; e += 32) {
-      const int64_t w = (int64_t)g.w[e];
-      const int32_t j = g.idx[e];
-      if (j < 0 || (int64_t)j >= g.n) { bad = true; continue; }
-      k += w;
-      if (C[j] == ci) inside += w;
-    }
-    for (int o = 16; o; o >>= 1) k += shfl_xor_i64(k, o);
-    if (lane == 0 && k) { atomic_add_i64(&Sig[ci], k); total += k; }
-  }
-  if (bad) atomicOr(err, 512ull);
-  inside = block_sum_i64(inside, sbuf);
-  total = block_sum_i64(total, sbuf);
-  if (threadIdx.x == 0) {
-    if (inside) atomicAdd(&acc[0], (u64)inside);
-    if (total) atomicAdd(&acc[3], (u64)total);
-  }
-}
 __global__ void mod_sq_k(int64_t n, const int64_t *Sig, u64 *acc) {
   __shared__ i128 sbuf[32];
   i128 s = 0;
@@ -238,19 +330,13 @@ __global__ void mod_sq_k(int64_t n, const int64_t *Sig, u64 *acc) {
   s = block_sum_i128(s, sbuf);
   if (threadIdx.x == 0 && s != 0) atomic_add_i128(&acc[1], s);
 }
-template <typename WT>
-void launch_modularity_terms(GraphView<WT> g, int64_t nnz, const int32_t *C, int64_t *Sig_tmp, u64 *acc,
+void launch_modularity_terms(GraphView<int32_t> g, int64_t nnz, const int32_t *C, int64_t *Sig_tmp, u64 *acc,
                              u64 *err, cudaStream_t s) {
   cudaMemsetAsync(acc, 0, 4 * sizeof(u64), s);
-  if (g.n <= 0) return;
-  cudaMemsetAsync(Sig_tmp, 0, (size_t)g.n * sizeof(int64_t), s);
-  LK_COUNTED mod_rows_k<WT><<<grid_for(g.n * 32, 256, 152 * 32), 256, 0, s>>>(g, nnz, C, Sig_tmp, acc, err);
-  LK_COUNTED mod_sq_k<<<grid_for(g.n, 256, 152 * 8), 256, 0, s>>>(g.n, Sig_tmp, acc);
+  if (g.n > 0) cudaMemsetAsync(Sig_tmp, 0, (size_t)g.n * sizeof(int64_t), s);
+  launch_rows<true>(g, nnz, C, nullptr, Sig_tmp, acc, err, s);
+  if (g.n > 0) LK_COUNTED mod_sq_k<<<grid_for(g.n, 256, 152 * 8), 256, 0, s>>>(g.n, Sig_tmp, acc);
 }
-template void launch_modularity_terms<int32_t>(GraphView<int32_t>, int64_t, const int32_t *, int64_t *, u64 *,
-                                               u64 *, cudaStream_t);
-template void launch_modularity_terms<int64_t>(GraphView<int64_t>, int64_t, const int32_t *, int64_t *, u64 *,
-                                               u64 *, cudaStream_t);
 
 // Sigma[c] = sum of K over members of c (Sigma zeroed first).
 __global__ void sigma_from_k(int64_t n, const int32_t *C, const int64_t *K, int64_t *Sig) {
@@ -312,19 +398,12 @@ void launch_mark_df(int64_t count, const int32_t *src, const int32_t *dst, const
 
 // A CSR is well formed: off[0] = 0, off[n] = nnz, offsets non-decreasing,
 // column IDs in [0, n), weights > 0.  Sets *err on violation.
-__global__ void check_graph_rows_k(int64_t n, int64_t nnz, const int64_t *off, u64 *err) {
-  GRID_STRIDE(i, n) {
-    const int64_t a = off[i], b = off[i + 1];
-    if (a > b || a < 0 || b > nnz) atomicOr(err, 128ull);
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && (off[0] != 0 || off[n] != nnz)) atomicOr(err, 128ull);
-}
 __global__ void check_graph_entries_k(int64_t n, int64_t nnz, const int32_t *idx, const int32_t *w, u64 *err) {
   GRID_STRIDE(e, nnz) if (idx[e] < 0 || idx[e] >= n || w[e] <= 0) atomicOr(err, 256ull);
 }
 void launch_check_graph(int64_t n, int64_t nnz, const int64_t *off, const int32_t *idx, const int32_t *w,
                         u64 *err, cudaStream_t s) {
-  LK_COUNTED check_graph_rows_k<<<grid_for(n > 0 ? n : 1, 256), 256, 0, s>>>(n, nnz, off, err);
+  LK_COUNTED check_graph_rows_k<<<grid_for(n > 0 ? n : 1, 256, 152 * 32), 256, 0, s>>>(n, nnz, off, nullptr, err);
   if (nnz > 0) LK_COUNTED check_graph_entries_k<<<grid_for(nnz, 256, 152 * 32), 256, 0, s>>>(n, nnz, idx, w, err);
 }
 

@@ -75,16 +75,9 @@ extern "C" int leiden_modularity_noalloc(const leiden_csr *g, const int32_t *mem
   unsigned long long *acc = scr + LEIDEN_NOALLOC_MAX_N;  // [0..3] terms, [8] error flag
   unsigned long long h[9] = {0};
   // The array keeps the previous call's contents: clear what must start at 0.
-  // Validate the graph and the labels, and read the verdict on the host,
-  // before any kernel indexes by them.
+  // The terms kernel tests every index before it uses it (a bad one is skipped
+  // and flagged), so the checks and the terms take one pass and one wait.
   cudaMemsetAsync(acc + 8, 0, sizeof(unsigned long long), s);
-  lk::launch_check_graph(g->n, g->nnz, g->off, g->idx, g->w, acc + 8, s);
-  lk::launch_check_range(membership, g->n, g->n, acc + 8, s);
-  cudaMemcpyAsync(&h[8], acc + 8, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
-  if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return LEIDEN_ECUDA;
-  if (h[8]) return LEIDEN_EINVAL;
-  // The terms kernels test every index themselves as well (a bad one is
-  // skipped and flagged), so no access depends on the order above.
   lk::GraphView<int32_t> gv{g->n, g->off, g->idx, g->w};
   lk::launch_modularity_terms(gv, g->nnz, membership, sig, acc, acc + 8, s);  // zeroes sig[0..n), acc[0..3]
   cudaMemcpyAsync(h, acc, 9 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
