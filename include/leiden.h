@@ -248,27 +248,29 @@ int leiden_modularity_noalloc(const leiden_csr *g, const int32_t *membership, do
  * Many small graphs in one persistent launch.
  *
  * leiden_batch_run takes up to max_graphs graphs at once and runs, for each,
- * the whole of Alg. leiden (every pass) inside one thread block: one kernel
- * launch for the batch, whose blocks take graphs from a device-side queue
- * (largest first) until none is left, with no host synchronisation between
- * phases.  The launch, together with the upload of the graph descriptors and
- * the download of the results, is captured once into a CUDA graph and
- * replayed for every later batch.  Same arithmetic and DET schedule as
- * leiden_static / leiden_update: for each graph the membership, modularity
- * and per-pass statistics are bit-identical to those calls.  Meant for graphs
- * small enough that one thread block per graph keeps the GPU busy; larger
- * graphs belong to a leiden_ctx.  ND, DS and DF updates recompute K^t and
- * Sigma^t from G^t and C^{t-1} (Alg. update with no auxiliary input).
+ * the whole of Alg. leiden (every pass) inside one thread block or one
+ * thread-block cluster (the largest graphs of the run, while SMs are to
+ * spare): one kernel launch for the batch, whose blocks take graphs from a
+ * device-side queue (largest first) until none is left, with no host
+ * synchronisation between phases.  The launch, together with the upload of
+ * the graph descriptors and the download of the results, is captured into a
+ * CUDA graph (one per cluster size) and replayed for later batches.  Same
+ * arithmetic and DET schedule as leiden_static / leiden_update: for each graph
+ * the membership, modularity and per-pass statistics are bit-identical to
+ * those calls.  Meant for graphs small enough that a block or a cluster per
+ * graph keeps the GPU busy; larger graphs belong to a leiden_ctx.  ND, DS and
+ * DF updates recompute K^t and Sigma^t from G^t and C^{t-1} (Alg. update with
+ * no auxiliary input).
  * ------------------------------------------------------------------------- */
 typedef struct leiden_batch leiden_batch;
 
 /* Creates a batch workspace bound to a stream (cudaStream_t as void*, NULL =
  * legacy default stream) for up to max_graphs graphs per run with at most
  * max_total_n vertices and max_total_nnz CSR entries summed over the run's
- * graphs (about 300 B per vertex plus 36 B per entry).  `threads` is the
- * block size of the persistent kernel (128..512, multiple of 32; 0 = 512)
- * and blocks_per_sm the number of blocks per SM it is launched with (1..4;
- * 0 = 1).  Errors: LEIDEN_EINVAL, LEIDEN_ENOMEM, LEIDEN_ECUDA. */
+ * graphs (about 100 B per vertex plus 60 B per entry).  `threads` (128..512,
+ * multiple of 32; 0) and blocks_per_sm (1..4; 0) are checked and otherwise
+ * without effect: the kernel has one shape, chosen for the SMs it runs on.
+ * Errors: LEIDEN_EINVAL, LEIDEN_ENOMEM, LEIDEN_ECUDA. */
 int leiden_batch_create(leiden_batch **out, void *cuda_stream, int32_t max_graphs, int64_t max_total_n,
                         int64_t max_total_nnz, int32_t threads, int32_t blocks_per_sm);
 

@@ -487,7 +487,7 @@ STATIC = 0
 
 class Batch:
     """A ``leiden_batch``: many small graphs per call, each run whole by one
-    thread block of one persistent, CUDA-graph-captured launch."""
+    thread block or one cluster of one persistent, CUDA-graph-captured launch."""
 
     def __init__(self, max_graphs: int, max_total_n: int, max_total_nnz: int, threads: int = 0,
                  blocks_per_sm: int = 0, stream=None):

@@ -681,9 +681,8 @@ int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int
   ta.in_range = lp == 0 ? r.in_range0 : nullptr;
   // aggregation table: at most two thirds full, keys and sums in the two
   // halves of the scratch values (zero whenever nobody uses them)
-  int lh = 10;
-  while (((int64_t)1 << lh) < nnz + nnz / 2) lh++;
-  ta.agg_lh = (!c->agg_uniform && nnz <= TEAM_AGG_NNZ && ((int64_t)2 << lh) <= c->gcap) ? lh : 0;
+  const int64_t slots = nnz + nnz / 2 + 64;
+  ta.agg_slots = (!c->agg_uniform && nnz <= TEAM_AGG_NNZ && 2 * slots <= c->gcap) ? slots : 0;
   ta.ctl = c->tctl;
   cudaMemsetAsync(c->tctl, 0, sizeof(TeamCtl), c->st);
   int64_t nb = std::min<int64_t>(c->sms, (nnz + g.n + TEAM_BLOCK_SIZE - 1) / TEAM_BLOCK_SIZE);

@@ -5,14 +5,18 @@
 
 #include <stdint.h>
 
+#include <cuda_runtime.h>
+
 #include "leiden.h"
 
 namespace lk {
 
 struct SmallHeader {
   int32_t count;     // jobs in this run
-  uint32_t next;     // queue head (0 at launch)
-  int64_t pad[7];
+  int32_t wide;      // jobs [0, wide) are run by whole clusters
+  uint32_t next;     // queue head of the clusters (0 at launch)
+  uint32_t next1;    // queue head of the single blocks (wide at launch)
+  int64_t pad[6];
 };
 
 struct SmallJob {
@@ -52,12 +56,15 @@ struct SmallResult {
 // 256-byte aligned).  n vertices and nnz CSR entries of the input graph bound
 // every level (aggregation never grows a graph).
 struct SmallLayout {
-  int64_t Ctop, Cp, CB, rep, vl, pi, pc, cv, longl, gkeys, idxA, idxB, hidx;
-  int64_t Kp, Sp, S2, scn, coff, ccur, hoff, cdist, offA, offB, wA, wB, hw;
-  int64_t pS;
+  int64_t Ctop, Cp, CB, rep, vl, pi, pc, idxA, idxB;
+  int64_t Kp, Sp, S2, cnt, cur, K2, offA, offB, wA, wB;
   int64_t ch, ch2, proc, stamp, flag;
-  int64_t gvals;
-  int log2T;         // slots of the global table: 2^log2T >= 2 n
+  int64_t table;     // aggregation keys and sums; before that the hubs' tables
+  int64_t slots;     // aggregation slots (keys, then as many sums)
+  int64_t piece_i, piece_k;
+  // graphs with more than TEAM_MAX_CAND vertices only (0 elements otherwise)
+  int64_t tkeys, hub_i, hub_s, hub_done, part_c, part_kid, part_sc;
+  int64_t tcap;      // hub table slots
   int64_t total;
 };
 
@@ -65,10 +72,6 @@ __host__ __device__ inline SmallLayout small_layout(int64_t n, int64_t nnz) {
   SmallLayout L{};
   const int64_t nv = n > 0 ? n : 1;
   const int64_t ne = nnz > 0 ? nnz : 1;
-  int lt = 6;
-  while (((int64_t)1 << lt) < 2 * nv) lt++;
-  L.log2T = lt;
-  const int64_t T = (int64_t)1 << lt;
   int64_t at = 0;
   auto put = [&](int64_t bytes) {
     const int64_t o = at;
@@ -76,15 +79,25 @@ __host__ __device__ inline SmallLayout small_layout(int64_t n, int64_t nnz) {
     return o;
   };
   L.Ctop = put(nv * 4); L.Cp = put(nv * 4); L.CB = put(nv * 4); L.rep = put(nv * 4); L.vl = put(nv * 4);
-  L.pi = put(nv * 4); L.pc = put(nv * 4); L.cv = put(nv * 4); L.longl = put(nv * 4); L.gkeys = put(T * 4);
-  L.idxA = put(ne * 4); L.idxB = put(ne * 4); L.hidx = put(ne * 4);
-  L.Kp = put(nv * 8); L.Sp = put(nv * 8); L.S2 = put(nv * 8); L.scn = put((nv + 1) * 8);
-  L.coff = put((nv + 1) * 8); L.ccur = put(nv * 8); L.hoff = put((nv + 1) * 8); L.cdist = put((nv + 1) * 8);
+  L.pi = put(nv * 4); L.pc = put(nv * 4);
+  L.idxA = put(ne * 4); L.idxB = put(ne * 4);
+  L.Kp = put(nv * 8); L.Sp = put(nv * 8); L.S2 = put(nv * 8);
+  L.cnt = put(nv * 8); L.cur = put(nv * 8); L.K2 = put(nv * 8);
   L.offA = put((nv + 1) * 8); L.offB = put((nv + 1) * 8);
-  L.wA = put(ne * 8); L.wB = put(ne * 8); L.hw = put(ne * 8);
-  L.pS = put(nv * 16);
+  L.wA = put(ne * 8); L.wB = put(ne * 8);
   L.ch = put(nv); L.ch2 = put(nv); L.proc = put(nv); L.stamp = put(nv); L.flag = put(nv);
-  L.gvals = put(T * 8);
+  L.slots = ne + ne / 2 + 64;
+  L.table = put(L.slots * 16);
+  // a mover's row of more than 1024 entries in pieces of 1024
+  L.piece_i = put((ne / 512 + 16) * 4); L.piece_k = put((ne / 512 + 16) * 4);
+  // hubs: a class's tables hold twice its hubs' entries, each table rounded up
+  // to 4096 slots, so the table's 3 nnz words are enough for all of them
+  const bool hubs = n > 8192;
+  L.tcap = hubs ? 2 * L.slots : 0;
+  const int64_t nh = hubs ? ne / 8192 + 16 : 0, np = hubs ? L.tcap / 4096 + 16 : 0;
+  L.tkeys = put(L.tcap * 4);
+  L.hub_i = put(nh * 4); L.hub_s = put(nh * 4); L.hub_done = put(nh * 4);
+  L.part_c = put(np * 4); L.part_kid = put(np * 8); L.part_sc = put(np * 16);
   L.total = at;
   return L;
 }
@@ -93,13 +106,19 @@ __host__ __device__ inline SmallLayout small_layout(int64_t n, int64_t nnz) {
 // a workspace for sum(n) vertices and sum(nnz) entries over g graphs holds
 // every batch within those totals.
 __host__ __device__ inline int64_t small_layout_bound(int64_t n, int64_t nnz, int64_t graphs) {
-  // per vertex: 9 x 4 + 10 x 8 + 16 + 5 bytes, the global table < 4 n slots
-  // of 12 bytes; per entry 3 x (4 + 8); per graph 35 arrays of alignment
-  // slack, the one-element minimum of empty graphs and the 64-slot table
-  return n * (36 + 80 + 16 + 5 + 48) + nnz * 36 + graphs * (35 * 256 + 1024 + 64 * 12 + 64);
+  // per vertex: 7 x 4 + 8 x 8 + 5 bytes; per entry 2 x (4 + 8), 1.5 x 16 for
+  // the table, 3 x 4 for the hubs' keys and below 1 for the pieces and hub
+  // items; per graph 32 arrays of alignment slack and the fixed extras
+  return n * 97 + nnz * 61 + graphs * (34 * 256 + 8192);
 }
 
-size_t small_dyn_smem(int threads);
-__global__ void small_leiden_k(SmallHeader *hdr, const SmallJob *jobs, SmallOpts o, SmallResult *results);
+// Threads of a block, blocks of a cluster at most.
+static constexpr int SMALL_MAX_CLUSTER = 16;
+struct SmallCtl;
+size_t small_ctl_bytes(int blocks);
+// Enqueues the kernel: `blocks` blocks in clusters of `cluster`; jobs before
+// hdr->wide are run by whole clusters, the others by single blocks.
+int launch_small(SmallHeader *hdr, const SmallJob *jobs, const SmallOpts &o, SmallResult *results, SmallCtl *ctl,
+                 int blocks, int cluster, cudaStream_t s);
 
 }  // namespace lk

@@ -190,6 +190,16 @@ struct TeamConst {
   const uint8_t *in_range;
 };
 
+// A value kept in the block's shared memory and read again at every use, so
+// that it takes no register between uses.  The batch kernel holds its arrays
+// this way; a context's arrays are kernel parameters, which cost none either.
+template <typename T>
+struct Held {
+  T v;
+  __device__ __forceinline__ operator T() const { return *(const volatile T *)&v; }
+  __device__ __forceinline__ void operator=(T x) { v = x; }
+};
+
 // Running sums of a thread: statistics and the scores of its moves.
 struct TeamStat {
   int64_t scanned, nvert, ncand;
@@ -250,8 +260,8 @@ __device__ __forceinline__ int team_table_add(int32_t *keys, VT *vals, int lh, i
   return -1;
 }
 
-template <bool REFINE>
-__device__ __forceinline__ bool team_eligible(const TeamArrays &a, const TeamConst &ct, int32_t i) {
+template <bool REFINE, typename AR, typename CT>
+__device__ __forceinline__ bool team_eligible(const AR &a, const CT &ct, int32_t i) {
   if (!REFINE) {
     if (a.processed[i]) return false;
     a.processed[i] = 1;                               // prune
@@ -261,8 +271,8 @@ __device__ __forceinline__ bool team_eligible(const TeamArrays &a, const TeamCon
 }
 
 // The move rule for vertex i (one lane): Eq. 2 scaled, strictly better only.
-template <bool REFINE, typename ST>
-__device__ __forceinline__ bool team_rule(const TeamArrays &a, const TeamConst &ct, int64_t Ki, int64_t Sd, ST bsc,
+template <bool REFINE, typename ST, typename AR, typename CT>
+__device__ __forceinline__ bool team_rule(const AR &a, const CT &ct, int64_t Ki, int64_t Sd, ST bsc,
                                           int32_t bc, int64_t kid, i128 *S) {
   if (bc == INT32_MAX) return false;
   *S = (i128)bsc - (i128)ct.A * kid - (i128)ct.p * Ki * (Ki - Sd);
@@ -272,8 +282,8 @@ __device__ __forceinline__ bool team_rule(const TeamArrays &a, const TeamConst &
 
 // Appends the proposals of a warp (whole warp calls) to the block's list, or
 // to the team's when that is full, and adds up their scores.
-template <bool REFINE, typename ST>
-__device__ __forceinline__ void team_propose(const TeamArrays &a, const TeamSweep &sw, TeamShared<ST> &sm, bool propose,
+template <bool REFINE, typename ST, typename AR>
+__device__ __forceinline__ void team_propose(const AR &a, const TeamSweep &sw, TeamShared<ST> &sm, bool propose,
                                              int32_t i, int32_t c, const TeamHead &h, i128 S, TeamStat &st) {
   const unsigned m = __ballot_sync(FULL_MASK, propose);
   if (!m) return;
@@ -306,8 +316,8 @@ __device__ __forceinline__ void team_propose(const TeamArrays &a, const TeamSwee
 }
 
 // Header of vertex i, and of a refinement its bound.
-template <typename WT>
-__device__ __forceinline__ TeamHead team_head(const TeamLevel<WT> &g, const TeamArrays &a, int32_t i) {
+template <typename GL, typename AR>
+__device__ __forceinline__ TeamHead team_head(const GL &g, const AR &a, int32_t i) {
   TeamHead h;
   h.e0 = g.off[i];
   h.deg = (int32_t)(g.off[i + 1] - h.e0);
@@ -328,8 +338,8 @@ __device__ __forceinline__ TeamHead team_shfl(const TeamHead &h, int src) {
 
 // One lane per vertex: the row (at most TT_LANE entries) in registers, equal
 // communities merged into their first occurrence.
-template <bool REFINE, typename WT, typename ST>
-__device__ __forceinline__ void team_decide_lane(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+template <bool REFINE, typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ void team_decide_lane(const GL &g, const AR &a, const CT &ct,
                                                  int32_t i, bool act, const TeamSweep &sw, TeamShared<ST> &sm,
                                                  TeamStat &st) {
   typedef typename TableVal<ST>::type VT;
@@ -392,8 +402,8 @@ __device__ __forceinline__ void team_decide_lane(const TeamLevel<WT> &g, const T
 
 // Best candidate among the slots this lane occupied (own[u] >= 0), which are
 // reset as they are read: the table is empty again once every lane is done.
-template <int STEPS, typename ST>
-__device__ __forceinline__ void team_scan_own(const TeamArrays &a, const int (&own)[STEPS], int32_t *keys,
+template <int STEPS, typename ST, typename AR>
+__device__ __forceinline__ void team_scan_own(const AR &a, const int (&own)[STEPS], int32_t *keys,
                                               typename TableVal<ST>::type *vals, int32_t d, ST A, ST B, ST &bsc,
                                               int32_t &bc, int64_t &kid, TeamStat &st) {
   constexpr int Q = STEPS < 4 ? STEPS : 4;   // Sigma' gathers in flight
@@ -423,8 +433,8 @@ __device__ __forceinline__ void team_scan_own(const TeamArrays &a, const int (&o
 
 // The row entries first, first + stride, ... (STEPS of them) of one lane: all
 // their loads, then their gathers, in flight before the first table insert.
-template <int STEPS, bool REFINE, typename WT, bool PIECE = false, typename VT>
-__device__ __forceinline__ void team_insert(const TeamLevel<WT> &g, const TeamArrays &a, int32_t i, int64_t e0, int deg,
+template <int STEPS, bool REFINE, typename WT, bool PIECE = false, typename VT, typename GL, typename AR>
+__device__ __forceinline__ void team_insert(const GL &g, const AR &a, int32_t i, int64_t e0, int deg,
                                             int first, int stride, int32_t cbi, int32_t *keys, VT *vals, int lh,
                                             int (&own)[STEPS]) {
   VT ww[STEPS];
@@ -449,8 +459,8 @@ __device__ __forceinline__ void team_insert(const TeamLevel<WT> &g, const TeamAr
 // G lanes per vertex (16 or 32), rows of at most G * STEPS entries, a table of
 // twice as many slots per group.  The whole warp calls; i < 0 marks an idle
 // group.
-template <int G, int STEPS, bool REFINE, typename WT, typename ST>
-__device__ __forceinline__ void team_decide_warp(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+template <int G, int STEPS, bool REFINE, typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ void team_decide_warp(const GL &g, const AR &a, const CT &ct,
                                                  int32_t i, const TeamHead &h, const TeamSweep &sw, int32_t *keys,
                                                  typename TableVal<ST>::type *vals, TeamShared<ST> &sm, TeamStat &st) {
   constexpr int LH = G * STEPS == 16 ? 5 : G * STEPS == 32 ? 6 : G * STEPS == 128 ? 8 : 9;
@@ -487,8 +497,8 @@ __device__ __forceinline__ void team_decide_warp(const TeamLevel<WT> &g, const T
 // listed vertices first, first + step, ... of list[0 .. m).  Warp 0 of the
 // group stages 32 listed vertices at once and keeps the eligible ones.  `bar`
 // is the group's named barrier, q its staging slot.
-template <int GT, bool REFINE, typename WT, typename ST>
-__device__ __forceinline__ void team_decide_group(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+template <int GT, bool REFINE, typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ void team_decide_group(const GL &g, const AR &a, const CT &ct,
                                                   const int32_t *list, int m, int first, int step, int bar, int q,
                                                   const TeamSweep &sw, int32_t *keys,
                                                   typename TableVal<ST>::type *vals, TeamShared<ST> &sm,
@@ -586,8 +596,8 @@ __device__ __forceinline__ void team_decide_group(const TeamLevel<WT> &g, const 
 // The vertices of one warp-per-vertex tier (list[0 .. m)): `ch` consecutive
 // listed vertices per warp and step, as few as spread the list over the team.
 // wg is the warp's place in the tier's order; returns it for the next tier.
-template <int G, int STEPS, bool REFINE, typename WT, typename ST>
-__device__ __forceinline__ int team_decide_tier(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+template <int G, int STEPS, bool REFINE, typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ int team_decide_tier(const GL &g, const AR &a, const CT &ct,
                                                 const int32_t *list, int m, int wg, int W, const TeamSweep &sw,
                                                 int32_t *keys, typename TableVal<ST>::type *vals, TeamShared<ST> &sm,
                                                 TeamStat &st) {
@@ -650,8 +660,8 @@ __device__ __forceinline__ int team_find(const int32_t *pre, int m, int w) {
 // slot is one 64-bit word, key + 1 in its low half (0: empty), the sum in its
 // high half, so both atomics meet one sector; 64-bit values: keys and values
 // apart.
-template <typename VT>
-__device__ __forceinline__ void team_hub_add(const TeamArrays &a, int64_t at, uint64_t t, int32_t c, u64 w) {
+template <typename VT, typename AR>
+__device__ __forceinline__ void team_hub_add(const AR &a, int64_t at, uint64_t t, int32_t c, u64 w) {
   uint64_t s = ((uint64_t)hash32(c) * t) >> 32;
   for (uint64_t probe = 0; probe < t; probe++) {
     if (sizeof(VT) == 4) {
@@ -671,8 +681,8 @@ __device__ __forceinline__ void team_hub_add(const TeamArrays &a, int64_t at, ui
 // Prefix sums of every class's hub items; false when a class has more hubs
 // than the bitmap holds or its tables exceed the scratch (the same answer in
 // every block).
-template <typename WT, typename ST>
-__device__ __forceinline__ bool team_hub_setup(const TeamLevel<WT> &g, const TeamArrays &a, int S, Team &t,
+template <typename WT, typename ST, typename GL, typename AR>
+__device__ __forceinline__ bool team_hub_setup(const GL &g, const AR &a, int S, Team &t,
                                                TeamShared<ST> &sm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h0 = sm.koff[7 * S], hn = sm.koff[8 * S];
@@ -717,8 +727,8 @@ __device__ __forceinline__ bool team_hub_setup(const TeamLevel<WT> &g, const Tea
 }
 
 // Which hubs of the class are to be decided, into sm.hbits; whether any is.
-template <bool REFINE, typename ST>
-__device__ __forceinline__ bool team_hub_bits(const TeamArrays &a, const TeamConst &ct, const int32_t *list, int m,
+template <bool REFINE, typename ST, typename AR, typename CT>
+__device__ __forceinline__ bool team_hub_bits(const AR &a, const CT &ct, const int32_t *list, int m,
                                               TeamShared<ST> &sm) {
   int any = 0;
   for (int base = 0; base < m; base += TEAM_THREADS) {
@@ -736,8 +746,8 @@ __device__ __forceinline__ bool team_hub_bits(const TeamArrays &a, const TeamCon
   return __syncthreads_or(any) != 0;
 }
 
-template <bool REFINE, typename WT, typename ST>
-__device__ __forceinline__ void team_hub_insert(const TeamLevel<WT> &g, const TeamArrays &a, const Team &t,
+template <bool REFINE, typename WT, typename ST, typename GL, typename AR>
+__device__ __forceinline__ void team_hub_insert(const GL &g, const AR &a, const Team &t,
                                                 const int32_t *list, const int32_t *pi, const int32_t *ps, int m,
                                                 int32_t *keys, typename TableVal<ST>::type *vals,
                                                 TeamShared<ST> &sm) {
@@ -770,8 +780,8 @@ __device__ __forceinline__ void team_hub_insert(const TeamLevel<WT> &g, const Te
   }
 }
 
-template <bool REFINE, typename WT, typename ST>
-__device__ __forceinline__ void team_hub_scan(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+template <bool REFINE, typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ void team_hub_scan(const GL &g, const AR &a, const CT &ct,
                                               const Team &t, const int32_t *list, const int32_t *ps, int32_t *done,
                                               int m, const TeamSweep &sw, TeamShared<ST> &sm, TeamStat &st) {
   typedef typename TableVal<ST>::type VT;
@@ -895,8 +905,8 @@ __device__ __forceinline__ void team_hub_scan(const TeamLevel<WT> &g, const Team
 // tier's first worker follows the last one of the tier before it, so a short
 // class spreads over the team.
 // Returns false after an expired wait.
-template <bool REFINE, typename WT, typename ST>
-__device__ __forceinline__ bool team_decide_class(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+template <bool REFINE, typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ bool team_decide_class(const GL &g, const AR &a, const CT &ct,
                                                   Team &t, int s, TeamSweep sw, int32_t *keys,
                                                   typename TableVal<ST>::type *vals, TeamShared<ST> &sm,
                                                   TeamStat &st) {
@@ -984,8 +994,8 @@ __device__ __forceinline__ bool team_decide_class(const TeamLevel<WT> &g, const 
 // Vertex pruning: `nl` lanes re-mark entries l, l + nl, ... of a row, U of
 // them in flight.  Most neighbours of a mover are unprocessed already:
 // reading the flag first spares the random byte store.
-template <int U, typename WT>
-__device__ __forceinline__ void team_remark(const TeamLevel<WT> &g, uint8_t *processed, int64_t e0, int len, int l,
+template <int U, typename GL>
+__device__ __forceinline__ void team_remark(const GL &g, uint8_t *processed, int64_t e0, int len, int l,
                                             int nl) {
   for (int x = l; x < len; x += nl * U) {
     int32_t j[U];
@@ -1002,8 +1012,8 @@ __device__ __forceinline__ void team_remark(const TeamLevel<WT> &g, uint8_t *pro
 
 // Commits of a local-moving sub-sweep: the block's own proposals, then the
 // team's overflow list (nover entries).
-template <typename WT, typename ST>
-__device__ __forceinline__ void team_apply_moves(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+template <typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ void team_apply_moves(const GL &g, const AR &a, const CT &ct,
                                                  const Team &t, unsigned np, unsigned nover, unsigned npiece,
                                                  TeamShared<ST> &sm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1124,8 +1134,8 @@ __device__ __forceinline__ int64_t team_scan(int64_t n, Team &t, TeamShared<ST> 
 // Vertex lists by (tier, colour class) in a.vlist, offsets in sm.koff (key =
 // tier * S + class); vertices without entries are left out.  hist: shared
 // words for the block's counts (the table area, free here).
-template <typename WT, typename ST>
-__device__ __forceinline__ bool team_lists(const TeamLevel<WT> &g, const TeamArrays &a, int log2S, Team &t,
+template <typename WT, typename ST, typename GL, typename AR>
+__device__ __forceinline__ bool team_lists(const GL &g, const AR &a, int log2S, Team &t,
                                            int32_t *hist, TeamShared<ST> &sm) {
   const int nk = (1 << log2S) * TEAM_TIERS;
   for (int k = threadIdx.x; k < nk; k += TEAM_THREADS) hist[k] = 0;
@@ -1181,8 +1191,8 @@ __device__ __forceinline__ bool team_lists(const TeamLevel<WT> &g, const TeamArr
 }
 
 // Alg. leidenlm; returns l_i (0 after an expired wait).
-template <typename WT, typename ST>
-__device__ __forceinline__ int team_local_move(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct,
+template <typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ int team_local_move(const GL &g, const AR &a, const CT &ct,
                                                double tau, int max_iters, Team &t, int32_t *keys,
                                                typename TableVal<ST>::type *vals, TeamShared<ST> &sm, TeamStat &st) {
   const int S = 1 << ct.log2S;
@@ -1258,8 +1268,8 @@ __device__ __forceinline__ int team_local_move(const TeamLevel<WT> &g, const Tea
 }
 
 // Alg. leidenre: one sweep, one sub-sweep per colour class.  stamp is zero.
-template <typename WT, typename ST>
-__device__ __forceinline__ bool team_refine(const TeamLevel<WT> &g, const TeamArrays &a, const TeamConst &ct, Team &t,
+template <typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ bool team_refine(const GL &g, const AR &a, const CT &ct, Team &t,
                                             int32_t *keys, typename TableVal<ST>::type *vals, TeamShared<ST> &sm) {
   const int S = 1 << ct.log2S;
   TeamCtl *ctl = t.ctl;
@@ -1305,21 +1315,21 @@ __device__ __forceinline__ bool team_refine(const TeamLevel<WT> &g, const TeamAr
   return true;
 }
 
-// Insert of one ((c, d), w) into the aggregation's global table of H slots
-// (2^lh): key c * 2^32 + d, plus one.  The first insert of a pair counts it
+// Insert of one ((c, d), w) into the aggregation's global table of H slots:
+// key c * 2^32 + d, plus one.  The first insert of a pair counts it
 // as an entry of c's row.
-__device__ __forceinline__ void team_agg_add(const TeamArrays &a, int lh, int32_t c, int32_t d, u64 w) {
+template <typename AR>
+__device__ __forceinline__ void team_agg_add(const AR &a, u64 H, int32_t c, int32_t d, u64 w) {
   const u64 key = (((u64)(uint32_t)c << 32) | (uint32_t)d) + 1ull;
-  const u64 mask = ((u64)1 << lh) - 1ull;
-  u64 s = (key * 0x9E3779B97F4A7C15ull) >> (64 - lh);
-  for (u64 probe = 0; probe <= mask; probe++) {
+  u64 s = __umul64hi(key * 0x9E3779B97F4A7C15ull, H);
+  for (u64 probe = 0; probe < H; probe++) {
     u64 k = *(volatile u64 *)&a.hkey[s];
     if (k == 0) {
       k = atomicCAS(&a.hkey[s], 0ull, key);
       if (k == 0) atomicAdd((u64 *)&a.cnt[c], 1ull);
     }
     if (k == 0 || k == key) { atomicAdd(&a.hval[s], w); return; }
-    s = (s + 1) & mask;
+    s = s + 1 == H ? 0 : s + 1;
   }
   atomicOr(a.err, 16ull);
 }
@@ -1329,8 +1339,8 @@ __device__ __forceinline__ void team_agg_add(const TeamArrays &a, int lh, int32_
 // the team as evenly as small ones; the pairs then go to their rows.
 // Writes off2, idx2, w2, K'' = row sums, and the level state of the next
 // pass.  cnt and K2 are zero on entry; the table is empty on entry and exit.
-template <typename WT, typename ST>
-__device__ __forceinline__ bool team_aggregate(const TeamLevel<WT> &g, const TeamArrays &a, int64_t nc, int lh, int S, Team &t,
+template <typename WT, typename ST, typename GL, typename AR>
+__device__ __forceinline__ bool team_aggregate(const GL &g, const AR &a, int64_t nc, u64 H, int S, Team &t,
                                                u64 (*wscr)[32], TeamShared<ST> &sm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t gt = t.index(), nt = (int64_t)t.nb * TEAM_THREADS;
@@ -1348,7 +1358,7 @@ __device__ __forceinline__ bool team_aggregate(const TeamLevel<WT> &g, const Tea
       const u64 w = in ? (u64)(int64_t)g.w[e] : 0;
       rs += w;
       u64 sum = 0;
-      if (warp_combine((unsigned long long)(uint32_t)d, in, w, &sum, wscr[warp])) team_agg_add(a, lh, c, d, sum);
+      if (warp_combine((unsigned long long)(uint32_t)d, in, w, &sum, wscr[warp])) team_agg_add(a, H, c, d, sum);
     }
     for (int o = 16; o; o >>= 1) rs += (u64)shfl_xor_i64((int64_t)rs, o);
     if (lane == 0 && rs) atomicAdd((u64 *)&a.K2[c], rs);
@@ -1367,7 +1377,7 @@ __device__ __forceinline__ bool team_aggregate(const TeamLevel<WT> &g, const Tea
       const u64 w = in ? (u64)(int64_t)g.w[e0 + x + lane] : 0;
       rs += w;
       u64 sum = 0;
-      if (warp_combine((unsigned long long)(uint32_t)d, in, w, &sum, wscr[warp])) team_agg_add(a, lh, c, d, sum);
+      if (warp_combine((unsigned long long)(uint32_t)d, in, w, &sum, wscr[warp])) team_agg_add(a, H, c, d, sum);
     }
     for (int o = 16; o; o >>= 1) rs += (u64)shfl_xor_i64((int64_t)rs, o);
     if (lane == 0 && rs) atomicAdd((u64 *)&a.K2[c], rs);
@@ -1394,7 +1404,7 @@ __device__ __forceinline__ bool team_aggregate(const TeamLevel<WT> &g, const Tea
       rs += w;
       u64 sum = 0;
       const unsigned long long key = ((unsigned long long)(uint32_t)c << 32) | (uint32_t)d;
-      if (warp_combine(key, in, w, &sum, wscr[warp])) team_agg_add(a, lh, c, d, sum);
+      if (warp_combine(key, in, w, &sum, wscr[warp])) team_agg_add(a, H, c, d, sum);
     }
 #pragma unroll
     for (int o = 4; o; o >>= 1) rs += (u64)shfl_xor_i64((int64_t)rs, o);
@@ -1424,8 +1434,7 @@ __device__ __forceinline__ bool team_aggregate(const TeamLevel<WT> &g, const Tea
   }
   TEAM_SYNC_OR(false);
   // the pairs to their rows, the table empty again
-  const int64_t H = (int64_t)1 << lh;
-  for (int64_t s = gt; s < H; s += nt) {
+  for (int64_t s = gt; s < (int64_t)H; s += nt) {
     const u64 k = __ldcg(&a.hkey[s]);
     if (!k) continue;
     const u64 v = __ldcg(&a.hval[s]);
@@ -1439,10 +1448,13 @@ __device__ __forceinline__ bool team_aggregate(const TeamLevel<WT> &g, const Tea
   return true;
 }
 
-// One whole pass.  See TeamArgs for what it reads and leaves behind.
-template <typename WT, typename ST>
-__device__ __forceinline__ void team_pass(const TeamLevel<WT> &g, TeamArrays a, const TeamConst &ct, int lp, double tau,
-                                          int max_iters, int agg_lh, Team &t, unsigned char *dyn, TeamShared<ST> &sm) {
+// One whole pass.  See TeamArgs for what it reads and leaves behind.  SHARED:
+// the array table is one copy in the block's shared memory (else each thread
+// has its own).
+template <bool SHARED, typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ void team_pass(const GL &g, AR &a, const CT &ct, int lp, double tau,
+                                          int max_iters, int64_t agg_slots, Team &t, unsigned char *dyn,
+                                          TeamShared<ST> &sm) {
   typedef typename TableVal<ST>::type VT;
   VT *vals = reinterpret_cast<VT *>(dyn);
   int32_t *keys = reinterpret_cast<int32_t *>(vals + TEAM_WARPS * TEAM_WSLOTS);
@@ -1505,8 +1517,11 @@ __device__ __forceinline__ void team_pass(const TeamLevel<WT> &g, TeamArrays a, 
     a.ch2[r] = a.ch[c];
   }
   TEAM_SYNC_OR();
-  { int64_t *x = a.Sig; a.Sig = a.Sig2; a.Sig2 = x; }
-  { uint8_t *x = a.ch; a.ch = a.ch2; a.ch2 = x; }
+  if (!SHARED || threadIdx.x == 0) {
+    { int64_t *x = a.Sig; a.Sig = a.Sig2; a.Sig2 = x; }
+    { uint8_t *x = a.ch; a.ch = a.ch2; a.ch2 = x; }
+  }
+  if (SHARED) __syncthreads();
   for (int64_t i = gt; i < n; i += nt) {
     const int32_t c = a.rep[a.C[i]];
     a.CB[i] = c;
@@ -1535,7 +1550,7 @@ __device__ __forceinline__ void team_pass(const TeamLevel<WT> &g, TeamArrays a, 
       [&](int64_t c, int64_t pre) { a.rep[c] = (int32_t)pre; });
   if (t.dead) return;
   if (t.rank == 0 && threadIdx.x == 0) ctl->nc = nc;
-  const bool agg = agg_lh > 0 && nc != n;
+  const bool agg = agg_slots > 0 && nc != n;
   TEAM_SYNC_OR();
   for (int64_t i = gt; i < n; i += nt) {
     const int32_t c = a.rep[a.C[i]];
@@ -1548,7 +1563,7 @@ __device__ __forceinline__ void team_pass(const TeamLevel<WT> &g, TeamArrays a, 
     return;
   }
   TEAM_SYNC_OR();
-  if (!team_aggregate<WT, ST>(g, a, nc, agg_lh, 1 << ct.log2S, t, reinterpret_cast<u64(*)[32]>(dyn), sm)) return;
+  if (!team_aggregate<WT, ST>(g, a, nc, (u64)agg_slots, 1 << ct.log2S, t, reinterpret_cast<u64(*)[32]>(dyn), sm)) return;
   // the next level: K' = Sigma' = row sums, C' = identity, everything
   // unprocessed, every community changed (C, K, Sig were read last before
   // the barriers of the aggregation)

@@ -70,7 +70,7 @@ struct TeamArrays {
 // One pass on a level graph of WT weights with scores of ST.  Reads the level
 // (off, idx, w), K', Sigma', C', processed, changed flags (and the DS range);
 // leaves the renumbered C' also in CB for the dendrogram lookup and, when it
-// aggregates (agg_lh > 0), the next level's graph and its initial state.
+// aggregates (agg_slots > 0), the next level's graph and its initial state.
 // Sig / Sig2 and ch / ch2 have changed places when it returns.
 template <typename WT>
 struct TeamArgs {
@@ -79,7 +79,8 @@ struct TeamArgs {
   TeamArrays a;
   int64_t A, p, two_m;
   double den, tau;
-  int log2S, dynamic, timing, lp, max_iters, agg_lh;
+  int log2S, dynamic, timing, lp, max_iters;
+  int64_t agg_slots;       // aggregation table (0: the caller aggregates)
   const uint8_t *in_range;
   TeamCtl *ctl;
 };

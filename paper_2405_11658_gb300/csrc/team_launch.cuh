@@ -1,4 +1,8 @@
-// team.cu -- the cooperative launch of a team pass (team.cuh) for a context.
+// team_launch.cuh -- the launch of a team pass (team.cuh) for a context.  Each
+// weight type and score width is instantiated in a file of its own
+// (team_*.cu), because one kernel takes the compiler a good twenty seconds.
+#pragma once
+
 #include <mutex>
 
 #include "team.cuh"
@@ -29,7 +33,8 @@ __global__ void __launch_bounds__(TEAM_THREADS, 1) team_pass_k(TeamArgs<WT> args
   ct.timing = args.timing;
   ct.in_range = args.in_range;
   const TeamLevel<WT> g{args.g.n, args.nnz, args.g.off, args.g.idx, args.g.w};
-  team_pass<WT, ST>(g, args.a, ct, args.lp, args.tau, args.max_iters, args.agg_lh, t, dyn, sm);
+  TeamArrays a = args.a;
+  team_pass<false, WT, ST>(g, a, ct, args.lp, args.tau, args.max_iters, args.agg_slots, t, dyn, sm);
 }
 
 template <typename WT, typename ST>
@@ -92,14 +97,5 @@ int launch_team_pass(const TeamArgs<WT> &args, int nb, int kind, cudaStream_t s)
   if (cudaLaunchKernelEx(&cfg, k, args, kind) != cudaSuccess) return LEIDEN_ECUDA;
   return LEIDEN_OK;
 }
-
-#define LK_TEAM_INST(WT, ST)                                                          \
-  template int launch_team_pass<WT, ST>(const TeamArgs<WT> &, int, int, cudaStream_t); \
-  template bool team_cluster_fits<WT, ST>(int);
-LK_TEAM_INST(int32_t, int64_t)
-LK_TEAM_INST(int32_t, i128)
-LK_TEAM_INST(int64_t, int64_t)
-LK_TEAM_INST(int64_t, i128)
-#undef LK_TEAM_INST
 
 }  // namespace lk

@@ -105,3 +105,35 @@ def test_same_result_as_the_multi_kernel_path():
                  "move_scanned_vertices", "move_bytes"):
         assert sa[name] == sb[name], name
     assert la < lb / 5   # the two paths really differ
+
+
+@pytest.mark.parametrize("count", [1, 7, 20, 45, 90, 160])
+def test_batch_cluster_sizes(count):
+    # clusters of 16, 8, 4, 2 blocks for the largest graphs, single blocks for
+    # the others: each graph as on a context
+    sizes = [int(20 + 6000 * 0.96 ** k) for k in range(count)]
+    graphs = [S.erdos_renyi(n, 8 / n, n, wmax=3) if n < 400 else S.planted_partition(n, max(2, n // 300), 0.02, 5 / n, n)
+              for n in sizes]
+    with L.Context(max_n=8192, max_nnz=1 << 19) as ctx, \
+            L.Batch(max_graphs=count, max_total_n=sum(len(g[0]) for g in graphs),
+                    max_total_nnz=sum(len(g[1]) for g in graphs)) as batch:
+        gs = [L.Graph.from_numpy(*g) for g in graphs]
+        outs, res = batch.run([{"graph": g} for g in gs])
+        for g, out, r in zip(gs, outs, res):
+            memb, q = ctx.static(g)
+            st = ctx.stats()
+            assert r["status"] == 0 and torch.equal(out, memb) and r["q"] == q
+            for name in ("passes", "iters", "nv", "nnz", "moves", "refine_moves", "changed0"):
+                assert r[name] == st[name], name
+
+
+@pytest.mark.parametrize("opts", [{"det_subsets": 1}, {"gamma": 1153434 / 1048576, "det_subsets": 1}, {}])
+def test_batch_with_hub_rows(opts):
+    # more than 8192 distinct candidates: the hub tables of the batch workspace
+    g = tiers_graph(30000, 1 << 12, 4)
+    ref = O.static(*g, O.LeidenOpts(**opts))
+    with L.Batch(max_graphs=3, max_total_n=3 * len(g[0]), max_total_nnz=3 * len(g[1])) as batch:
+        G = L.Graph.from_numpy(*g)
+        outs, res = batch.run([{"graph": G}] * 3, L.Opts(**opts))
+        for out, r in zip(outs, res):
+            assert r["status"] == 0 and np.array_equal(out.cpu().numpy(), ref.membership) and r["q"] == ref.q
