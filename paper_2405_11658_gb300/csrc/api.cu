@@ -1327,6 +1327,12 @@ int leiden_apply_batch(leiden_ctx *c, const leiden_csr *g, const leiden_edges *d
   w.bits = reinterpret_cast<uint32_t *>(scratch + ((U + 15) & ~(int64_t)15));
   w.tflag = c->flag; w.tpos = c->cdist; w.trow = c->cv;
   w.newdeg = c->ctdeg;
+  w.big = c->clist;
+  // a long row has more than 256 entries or records, of which there are at
+  // most max_nnz each: two pieces per 256 of either fit the level buffer
+  w.pt = c->gidx[1];
+  w.pp = reinterpret_cast<int32_t *>(c->gw[1]);
+  w.counts = &c->ctr[CTR_SCRATCH0];
   w.scan_tmp = c->scan_tmp;
   w.err = &c->ctr[CTR_ERROR];
   rc = apply_batch(g->n, g->off, g->idx, g->w, nd, nd ? del->src : nullptr, nd ? del->dst : nullptr,

@@ -178,17 +178,59 @@ __global__ void ba_touched_flag_k(int64_t n, const int64_t *cnt, uint8_t *tflag)
 __global__ void ba_touched_list_k(int64_t n, const uint8_t *tflag, const int64_t *tpos, int32_t *trow) {
   DSTRIDE(u, n) if (tflag[u]) trow[tpos[u]] = (int32_t)u;
 }
-// One thread per touched row: sort the row's updates by target (insertion
-// sort: a row gets few), merge equal targets, classify each against the old
-// row and record the exclusive prefix counts of removed and new entries.
-// Writes the compacted records to the front of the row's list, their count to
-// nrec[u] and the new row length to newdeg[u].
+// Rows with more updates than this are sorted and classified by a block.
+static constexpr int BA_ROW_SERIAL = 16;
+// Touched rows with more old entries or records than this are merged in pieces
+// of BA_PIECE by a warp each.
+static constexpr int BA_LONG = 256, BA_PIECE = 512;
+
+// The merge pieces of a long row: the old entries and the records
+// p * BA_PIECE .. of each.
+__device__ __forceinline__ void ba_pieces(int64_t t, int64_t old, int64_t nr, int32_t *pt, int32_t *pp, u64 *npiece) {
+  const int64_t m = old > nr ? old : nr;
+  if (m <= BA_LONG) return;
+  const int64_t c = (m + BA_PIECE - 1) / BA_PIECE;
+  const u64 at = atomicAdd(npiece, (u64)c);
+  for (int64_t k = 0; k < c; k++) { pt[at + k] = (int32_t)t; pp[at + k] = (int32_t)k; }
+}
+
+// What a target's updates (dels of weight dw, insertions summing to iw) make
+// of the row's entry at f: kind and new weight; false for an invalid deletion.
+__device__ __forceinline__ bool ba_classify(int32_t tgt, int dels, int64_t dw, int64_t iw, int64_t a0, int64_t a1,
+                                            const int32_t *idx, const int32_t *w, uint8_t *kind, int64_t *nw,
+                                            u64 *err) {
+  if (dels > 1) { atomicOr(err, 4ull); return false; }       // duplicate deletion
+  const int64_t f = row_find(idx, a0, a1, tgt);
+  const bool exists = f < a1 && idx[f] == tgt;
+  if (dels && (!exists || (int64_t)w[f] != dw)) { atomicOr(err, 2ull); return false; }  // missing edge / weight
+  if (exists) {
+    if (dels && iw == 0) { *kind = UPD_REMOVED; *nw = 0; }
+    else { *kind = UPD_REWEIGHT; *nw = dels ? iw : (int64_t)w[f] + iw; }
+  } else {
+    *kind = UPD_NEW; *nw = iw;
+  }
+  if (*nw > INT32_MAX) { atomicOr(err, 1024ull); *nw = INT32_MAX; }  // weight beyond int32
+  return true;
+}
+
+// One thread per touched row with few updates: sort them by target (insertion
+// sort), merge equal targets, classify each against the old row and record the
+// exclusive prefix counts of removed and new entries.  Writes the compacted
+// records to the front of the row's list, their count to nrec[u] and the new
+// row length to newdeg[u].  Rows with more updates go to the block kernel
+// below (heavy rows draw a share of the deletions): one thread's sort and its
+// chain of binary searches held the whole kernel up.
 __global__ void ba_row_k(int64_t T, const int32_t *trow, const int64_t *uoff, int32_t *ut, int32_t *uw,
                          uint8_t *uk, int32_t *Rp, int32_t *Np, int64_t *nrec, const int64_t *off,
-                         const int32_t *idx, const int32_t *w, int64_t *newdeg, u64 *err) {
+                         const int32_t *idx, const int32_t *w, int64_t *newdeg, int32_t *big, int32_t *pt, int32_t *pp,
+                         u64 *counts, u64 *err) {
   DSTRIDE(t, T) {
     const int32_t u = trow[t];
     const int64_t b = uoff[u], e = uoff[u + 1];
+    if (e - b > BA_ROW_SERIAL) {
+      big[atomicAdd(&counts[0], 1ull)] = (int32_t)t;
+      continue;
+    }
     for (int64_t x = b + 1; x < e; x++) {
       const int32_t kv = ut[x], kw = uw[x];
       int64_t y = x - 1;
@@ -200,24 +242,13 @@ __global__ void ba_row_k(int64_t T, const int32_t *trow, const int64_t *uoff, in
     int64_t q = b;
     for (int64_t x = b; x < e;) {
       const int32_t tgt = ut[x];
-      int64_t dw = 0, iw = 0;
+      int64_t dw = 0, iw = 0, nw;
       int dels = 0;
+      uint8_t kind;
       for (; x < e && ut[x] == tgt; x++) {
         if (uw[x] < 0) { dels++; dw = -(int64_t)uw[x]; } else { iw += uw[x]; }
       }
-      if (dels > 1) { atomicOr(err, 4ull); continue; }       // duplicate deletion
-      const int64_t f = row_find(idx, a0, a1, tgt);
-      const bool exists = f < a1 && idx[f] == tgt;
-      if (dels && (!exists || (int64_t)w[f] != dw)) { atomicOr(err, 2ull); continue; }  // missing edge / weight
-      uint8_t kind;
-      int64_t nw;
-      if (exists) {
-        if (dels && iw == 0) { kind = UPD_REMOVED; nw = 0; }
-        else { kind = UPD_REWEIGHT; nw = dels ? iw : (int64_t)w[f] + iw; }
-      } else {
-        kind = UPD_NEW; nw = iw;
-      }
-      if (nw > INT32_MAX) { atomicOr(err, 1024ull); nw = INT32_MAX; }  // weight beyond int32
+      if (!ba_classify(tgt, dels, dw, iw, a0, a1, idx, w, &kind, &nw, err)) continue;
       ut[q] = tgt; uw[q] = (int32_t)nw; uk[q] = kind; Rp[q] = R; Np[q] = N;
       R += kind == UPD_REMOVED;
       N += kind == UPD_NEW;
@@ -225,6 +256,122 @@ __global__ void ba_row_k(int64_t T, const int32_t *trow, const int64_t *uoff, in
     }
     nrec[u] = q - b;
     newdeg[u] = (a1 - a0) - R + N;
+    ba_pieces(t, a1 - a0, q - b, pt, pp, &counts[1]);
+  }
+}
+
+// A block per row with many updates: bitonic sort of (target, weight) pairs
+// (every comparator puts the smaller one at the lower index, so the missing
+// elements up to the next power of two count as largest and are skipped), in
+// shared memory up to BA_SORT pairs; then one thread per distinct target
+// classifies it, and block-wide prefix sums place the records.
+static constexpr int BA_BIG_THREADS = 256, BA_SORT = 4096;
+template <typename GET, typename PUT>
+__device__ __forceinline__ void ba_bitonic(int64_t n, GET get, PUT put) {
+  int64_t P = 1;
+  while (P < n) P <<= 1;
+  auto exchange = [&](int64_t i, int64_t j) {
+    if (j >= n) return;
+    const u64 x = get(i), y = get(j);
+    if (y < x) { put(i, y); put(j, x); }
+  };
+  for (int64_t k = 2; k <= P; k <<= 1) {
+    for (int64_t q = threadIdx.x; q < P / 2; q += BA_BIG_THREADS) {   // mirrored halves of each run of k
+      const int64_t r = q / (k / 2), o = q % (k / 2);
+      exchange(r * k + o, r * k + k - 1 - o);
+    }
+    __syncthreads();
+    for (int64_t h = k >> 2; h > 0; h >>= 1) {
+      for (int64_t q = threadIdx.x; q < P / 2; q += BA_BIG_THREADS) {
+        const int64_t i = (q / h) * 2 * h + q % h;
+        exchange(i, i + h);
+      }
+      __syncthreads();
+    }
+  }
+}
+__global__ void __launch_bounds__(BA_BIG_THREADS) ba_row_big_k(const int32_t *trow, const int64_t *uoff, int32_t *ut,
+                                                               int32_t *uw, uint8_t *uk, int32_t *Rp, int32_t *Np,
+                                                               int64_t *nrec, const int64_t *off, const int32_t *idx,
+                                                               const int32_t *w, int64_t *newdeg, const int32_t *big,
+                                                               int32_t *pt, int32_t *pp, u64 *counts, u64 *err) {
+  __shared__ u64 buf[BA_SORT];
+  __shared__ int wsum[3][BA_BIG_THREADS / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t nbig = (int64_t)counts[0];
+  for (int64_t bi = blockIdx.x; bi < nbig; bi += gridDim.x) {
+    const int32_t t = big[bi], u = trow[t];
+    const int64_t b = uoff[u], n = uoff[u + 1] - b;
+    const int64_t a0 = off[u], a1 = off[u + 1];
+    auto pair = [&](int64_t x) { return ((u64)(uint32_t)ut[b + x] << 32) | (uint32_t)uw[b + x]; };
+    if (n <= BA_SORT) {
+      for (int64_t x = threadIdx.x; x < n; x += BA_BIG_THREADS) buf[x] = pair(x);
+      __syncthreads();
+      ba_bitonic(n, [&](int64_t x) { return buf[x]; }, [&](int64_t x, u64 v) { buf[x] = v; });
+      for (int64_t x = threadIdx.x; x < n; x += BA_BIG_THREADS) {
+        ut[b + x] = (int32_t)(buf[x] >> 32);
+        uw[b + x] = (int32_t)(uint32_t)buf[x];
+      }
+      __syncthreads();
+    } else {
+      ba_bitonic(n, pair, [&](int64_t x, u64 v) {
+        ut[b + x] = (int32_t)(v >> 32);
+        uw[b + x] = (int32_t)(uint32_t)v;
+      });
+    }
+    // records, a tile of the sorted updates at a time; a tile's records land
+    // at or before its own positions, after every thread has read its updates
+    int64_t q = 0;
+    int R = 0, N = 0;
+    for (int64_t x0 = 0; x0 < n; x0 += BA_BIG_THREADS) {
+      const int64_t x = x0 + threadIdx.x;
+      const int32_t tgt = x < n ? ut[b + x] : -1;
+      // the update before the tile may have been overwritten by a record, but
+      // a record there has the last target before it or an earlier one
+      const bool first = x < n && (x == 0 || (threadIdx.x ? ut[b + x - 1] : (int32_t)wsum[2][0]) != tgt);
+      bool rec = false;
+      uint8_t kind = 0;
+      int64_t nw = 0;
+      if (first) {
+        int64_t dw = 0, iw = 0;
+        int dels = 0;
+        for (int64_t y = x; y < n && ut[b + y] == tgt; y++) {
+          const int32_t v = uw[b + y];
+          if (v < 0) { dels++; dw = -(int64_t)v; } else { iw += v; }
+        }
+        rec = ba_classify(tgt, dels, dw, iw, a0, a1, idx, w, &kind, &nw, err);
+      }
+      const int32_t lastt = x0 + BA_BIG_THREADS <= n ? ut[b + x0 + BA_BIG_THREADS - 1] : -1;
+      const unsigned mq = __ballot_sync(FULL_MASK, rec), mr = __ballot_sync(FULL_MASK, rec && kind == UPD_REMOVED),
+                     mn = __ballot_sync(FULL_MASK, rec && kind == UPD_NEW), below = (1u << lane) - 1u;
+      __syncthreads();   // every update of the tile is read; wsum[2][0] too
+      if (lane == 0) { wsum[0][warp] = __popc(mq) | (__popc(mr) << 10) | (__popc(mn) << 20); }
+      if (threadIdx.x == 0) wsum[2][0] = lastt;
+      __syncthreads();
+      int pre = 0, tot = 0;
+      for (int k = 0; k < BA_BIG_THREADS / 32; k++) {
+        if (k < warp) pre += wsum[0][k];
+        tot += wsum[0][k];
+      }
+      if (rec) {
+        const int64_t at = b + q + (pre & 1023) + __popc(mq & below);
+        ut[at] = tgt;
+        uw[at] = (int32_t)nw;
+        uk[at] = kind;
+        Rp[at] = R + ((pre >> 10) & 1023) + __popc(mr & below);
+        Np[at] = N + (pre >> 20) + __popc(mn & below);
+      }
+      q += tot & 1023;
+      R += (tot >> 10) & 1023;
+      N += tot >> 20;
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+      nrec[u] = q;
+      newdeg[u] = (a1 - a0) - R + N;
+      ba_pieces(t, a1 - a0, q, pt, pp, &counts[1]);
+    }
+    __syncthreads();
   }
 }
 // Row starts as a bitmap over the entries (for the sortedness check of the
@@ -276,10 +423,57 @@ __global__ void ba_copy_k(int64_t nnz, int64_t T, const int32_t *trow, const int
     }
   }
 }
-// BA_MERGE_LANES lanes per touched row (most touched rows are short, so a
-// whole warp per row would leave most lanes idle): every surviving old entry
-// goes to its rank among the new row (its position less the removed entries
-// before it plus the new ones before it), every new entry likewise.
+// Old entries and records [l0, l1) of a touched row, `G` lanes: every surviving
+// old entry goes to its rank among the new row (its position less the removed
+// entries before it plus the new ones before it), every new entry likewise.
+template <int G>
+__device__ __forceinline__ void ba_merge_part(int lane, int64_t l0, int64_t l1, int64_t a0, int64_t a1, int64_t p0,
+                                              int64_t nr, int64_t o0, int64_t len, const int32_t *ut, const int32_t *uw,
+                                              const uint8_t *uk, const int32_t *Rp, const int32_t *Np,
+                                              const int32_t *idx, const int32_t *w, int32_t *idx2, int32_t *w2,
+                                              u64 *err) {
+  const int64_t e1 = a0 + l1 < a1 ? a0 + l1 : a1;
+  for (int64_t a = a0 + l0 + lane; a < e1; a += G) {
+    const int32_t x = idx[a];
+    if (a > a0 && idx[a - 1] >= x) { atomicOr(err, 8ull); continue; }
+    int64_t lo = 0, hi = nr;                                 // first record with target >= x
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (ut[p0 + mid] < x) lo = mid + 1; else hi = mid;
+    }
+    int64_t rb, nb;
+    if (lo < nr) { rb = Rp[p0 + lo]; nb = Np[p0 + lo]; }
+    else if (nr > 0) {                                       // after every record
+      const int64_t l = p0 + nr - 1;
+      rb = Rp[l] + (uk[l] == UPD_REMOVED);
+      nb = Np[l] + (uk[l] == UPD_NEW);
+    } else { rb = 0; nb = 0; }
+    int32_t wt = w[a];
+    if (lo < nr && ut[p0 + lo] == x) {
+      if (uk[p0 + lo] == UPD_REMOVED) continue;
+      wt = uw[p0 + lo];
+    }
+    const int64_t pos = (a - a0) - rb + nb;
+    if (pos < 0 || pos >= len) { atomicOr(err, 8ull); continue; }
+    idx2[o0 + pos] = x;
+    w2[o0 + pos] = wt;
+  }
+  const int64_t q1 = l1 < nr ? l1 : nr;
+  for (int64_t q = l0 + lane; q < q1; q += G) {
+    if (uk[p0 + q] != UPD_NEW) continue;
+    const int32_t y = ut[p0 + q];
+    const int64_t pos = (row_find(idx, a0, a1, y) - a0) - Rp[p0 + q] + Np[p0 + q];
+    if (pos < 0 || pos >= len) { atomicOr(err, 8ull); continue; }
+    idx2[o0 + pos] = y;
+    w2[o0 + pos] = uw[p0 + q];
+  }
+}
+
+// Rows of up to BA_LONG old entries and records: BA_MERGE_LANES lanes per row
+// (most touched rows are short, so a whole warp per row would leave most lanes
+// idle).  Longer rows: a warp per piece; with eight lanes on a whole heavy row
+// the last rows held the kernel up (1e-2 |E| on a Chung-Lu graph of 6.25e7
+// entries: 1.52 ms, both kernels 0.39 ms).
 static constexpr int BA_MERGE_LANES = 8;
 __global__ void ba_merge_k(int64_t T, const int32_t *trow, const int64_t *uoff, const int64_t *nrec,
                            const int32_t *ut, const int32_t *uw, const uint8_t *uk, const int32_t *Rp,
@@ -292,41 +486,27 @@ __global__ void ba_merge_k(int64_t T, const int32_t *trow, const int64_t *uoff, 
   for (int64_t t = wid; t < T; t += nwarps) {
     const int32_t u = trow[t];
     const int64_t a0 = off[u], a1 = off[u + 1];
-    const int64_t p0 = uoff[u], nr = nrec[u];
-    const int64_t o0 = off2[u], len = off2[u + 1] - o0;
-    for (int64_t a = a0 + lane; a < a1; a += G) {
-      const int32_t x = idx[a];
-      if (a > a0 && idx[a - 1] >= x) { atomicOr(err, 8ull); continue; }
-      int64_t lo = 0, hi = nr;                                 // first record with target >= x
-      while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (ut[p0 + mid] < x) lo = mid + 1; else hi = mid;
-      }
-      int64_t rb, nb;
-      if (lo < nr) { rb = Rp[p0 + lo]; nb = Np[p0 + lo]; }
-      else if (nr > 0) {                                       // after every record
-        const int64_t l = p0 + nr - 1;
-        rb = Rp[l] + (uk[l] == UPD_REMOVED);
-        nb = Np[l] + (uk[l] == UPD_NEW);
-      } else { rb = 0; nb = 0; }
-      int32_t wt = w[a];
-      if (lo < nr && ut[p0 + lo] == x) {
-        if (uk[p0 + lo] == UPD_REMOVED) continue;
-        wt = uw[p0 + lo];
-      }
-      const int64_t pos = (a - a0) - rb + nb;
-      if (pos < 0 || pos >= len) { atomicOr(err, 8ull); continue; }
-      idx2[o0 + pos] = x;
-      w2[o0 + pos] = wt;
-    }
-    for (int64_t q = lane; q < nr; q += G) {
-      if (uk[p0 + q] != UPD_NEW) continue;
-      const int32_t y = ut[p0 + q];
-      const int64_t pos = (row_find(idx, a0, a1, y) - a0) - Rp[p0 + q] + Np[p0 + q];
-      if (pos < 0 || pos >= len) { atomicOr(err, 8ull); continue; }
-      idx2[o0 + pos] = y;
-      w2[o0 + pos] = uw[p0 + q];
-    }
+    const int64_t nr = nrec[u];
+    if (a1 - a0 > BA_LONG || nr > BA_LONG) continue;
+    const int64_t o0 = off2[u];
+    ba_merge_part<G>(lane, 0, BA_LONG, a0, a1, uoff[u], nr, o0, off2[u + 1] - o0, ut, uw, uk, Rp, Np, idx, w, idx2, w2,
+                     err);
+  }
+}
+__global__ void ba_merge_pieces_k(const u64 *counts, const int32_t *pt, const int32_t *pp, const int32_t *trow,
+                                  const int64_t *uoff, const int64_t *nrec, const int32_t *ut, const int32_t *uw,
+                                  const uint8_t *uk, const int32_t *Rp, const int32_t *Np, const int64_t *off,
+                                  const int32_t *idx, const int32_t *w, const int64_t *off2, int32_t *idx2,
+                                  int32_t *w2, u64 *err) {
+  const int lane = threadIdx.x & 31;
+  const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int64_t np = (int64_t)counts[1];
+  for (int64_t k = wid; k < np; k += nwarps) {
+    const int32_t u = trow[pt[k]];
+    const int64_t l0 = (int64_t)pp[k] * BA_PIECE, o0 = off2[u];
+    ba_merge_part<32>(lane, l0, l0 + BA_PIECE, off[u], off[u + 1], uoff[u], nrec[u], o0, off2[u + 1] - o0, ut, uw, uk,
+                      Rp, Np, idx, w, idx2, w2, err);
   }
 }
 
@@ -361,9 +541,16 @@ int apply_batch(int64_t n, const int64_t *off, const int32_t *idx, const int32_t
   if (cudaStreamSynchronize(s) != cudaSuccess) return LEIDEN_ECUDA;
   // new row lengths: the old ones, then the touched rows' own
   if (n > 0) LK_COUNTED ba_deg_k<<<gridd(n, 256), 256, 0, s>>>(n, off, wk.newdeg);
-  if (T > 0)
+  if (T > 0) {
+    cudaMemsetAsync(wk.counts, 0, 2 * sizeof(u64), s);
     LK_COUNTED ba_row_k<<<gridd(T, 128), 128, 0, s>>>(T, wk.trow, wk.uoff, wk.ut, wk.uw, wk.uk, wk.Rp, wk.Np, wk.cnt,
-                                                      off, idx, w, wk.newdeg, wk.err);
+                                                      off, idx, w, wk.newdeg, wk.big, wk.pt, wk.pp, wk.counts, wk.err);
+    // a row with more than BA_ROW_SERIAL updates needs that many in the batch
+    if (2 * (nd + ni) > BA_ROW_SERIAL)
+      LK_COUNTED ba_row_big_k<<<gridd(2 * (nd + ni) / BA_ROW_SERIAL, 1, 152 * 6), BA_BIG_THREADS, 0, s>>>(
+          wk.trow, wk.uoff, wk.ut, wk.uw, wk.uk, wk.Rp, wk.Np, wk.cnt, off, idx, w, wk.newdeg, wk.big, wk.pt, wk.pp,
+          wk.counts, wk.err);
+  }
   exclusive_scan<int64_t>(wk.newdeg, off_out, n, wk.scan_tmp, s);
   int64_t nnz2 = 0;
   cudaMemcpyAsync(&nnz2, off_out + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
@@ -379,10 +566,13 @@ int apply_batch(int64_t n, const int64_t *off, const int32_t *idx, const int32_t
     LK_COUNTED ba_copy_k<<<gridd(tiles * 32, 256, 152 * 64), 256, 0, s>>>(nnz, T, wk.trow, off, off_out, idx, w,
                                                                          wk.bits, nnz2, idx_out, w_out, wk.err);
   }
-  if (T > 0)
-    LK_COUNTED ba_merge_k<<<gridd(T * BA_MERGE_LANES, 256, 152 * 32), 256, 0, s>>>(T, wk.trow, wk.uoff, wk.cnt, wk.ut, wk.uw,
-                                                                      wk.uk, wk.Rp, wk.Np, off, idx, w, off_out,
-                                                                      idx_out, w_out, wk.err);
+  if (T > 0) {
+    LK_COUNTED ba_merge_k<<<gridd(T * BA_MERGE_LANES, 256, 152 * 32), 256, 0, s>>>(
+        T, wk.trow, wk.uoff, wk.cnt, wk.ut, wk.uw, wk.uk, wk.Rp, wk.Np, off, idx, w, off_out, idx_out, w_out, wk.err);
+    LK_COUNTED ba_merge_pieces_k<<<152 * 8, 256, 0, s>>>(wk.counts, wk.pt, wk.pp, wk.trow, wk.uoff, wk.cnt, wk.ut,
+                                                         wk.uw, wk.uk, wk.Rp, wk.Np, off, idx, w, off_out, idx_out,
+                                                         w_out, wk.err);
+  }
   cudaMemcpyAsync(&herr, wk.err, sizeof(u64), cudaMemcpyDeviceToHost, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return LEIDEN_ECUDA;
   if (herr) return LEIDEN_EINVAL;

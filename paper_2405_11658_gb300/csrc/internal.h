@@ -335,6 +335,9 @@ struct BatchWork {
   int64_t *tpos;     // [n+1] their exclusive scan
   int32_t *trow;     // [n] touched rows in increasing order
   int64_t *newdeg;   // [n+1]
+  int32_t *big;      // [n] rows with many updates
+  int32_t *pt, *pp;  // [(nnz + 2*(nd+ni)) / 256 + ...] merge pieces of long rows: touched row, piece
+  u64 *counts;       // [2] rows in big, pieces
   uint32_t *bits;    // [nnz/32 + 1] row starts
   int64_t *scan_tmp;
   u64 *err;

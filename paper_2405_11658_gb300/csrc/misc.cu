@@ -398,13 +398,23 @@ void launch_mark_df(int64_t count, const int32_t *src, const int32_t *dst, const
 
 // A CSR is well formed: off[0] = 0, off[n] = nnz, offsets non-decreasing,
 // column IDs in [0, n), weights > 0.  Sets *err on violation.
-__global__ void check_graph_entries_k(int64_t n, int64_t nnz, const int32_t *idx, const int32_t *w, u64 *err) {
-  GRID_STRIDE(e, nnz) if (idx[e] < 0 || idx[e] >= n || w[e] <= 0) atomicOr(err, 256ull);
+// Four entries a load where both arrays start on 16 bytes (vec), else one.
+__global__ void check_graph_entries_k(int64_t n, int64_t nnz, const int32_t *idx, const int32_t *w, int vec, u64 *err) {
+  bool bad = false;
+  const int64_t nv = vec ? nnz / 4 : 0;
+  GRID_STRIDE(v, nv) {
+    const int4 j = reinterpret_cast<const int4 *>(idx)[v], x = reinterpret_cast<const int4 *>(w)[v];
+    bad |= (int64_t)(uint32_t)j.x >= n || (int64_t)(uint32_t)j.y >= n || (int64_t)(uint32_t)j.z >= n ||
+           (int64_t)(uint32_t)j.w >= n || x.x <= 0 || x.y <= 0 || x.z <= 0 || x.w <= 0;
+  }
+  GRID_STRIDE(q, nnz - 4 * nv) bad |= (int64_t)(uint32_t)idx[4 * nv + q] >= n || w[4 * nv + q] <= 0;
+  if (bad) atomicOr(err, 256ull);
 }
 void launch_check_graph(int64_t n, int64_t nnz, const int64_t *off, const int32_t *idx, const int32_t *w,
                         u64 *err, cudaStream_t s) {
   LK_COUNTED check_graph_rows_k<<<grid_for(n > 0 ? n : 1, 256, 152 * 32), 256, 0, s>>>(n, nnz, off, nullptr, err);
-  if (nnz > 0) LK_COUNTED check_graph_entries_k<<<grid_for(nnz, 256, 152 * 32), 256, 0, s>>>(n, nnz, idx, w, err);
+  const int vec = (((uintptr_t)idx | (uintptr_t)w) & 15) == 0;
+  if (nnz > 0) LK_COUNTED check_graph_entries_k<<<grid_for(nnz, 256, 152 * 32), 256, 0, s>>>(n, nnz, idx, w, vec, err);
 }
 
 // Labels in [0, hi); sets *err on violation.

@@ -87,10 +87,11 @@ def test_malformed_inputs_are_refused(fault):
         lab[5] = -1
     g = L.Graph.from_numpy(off, idx, w)
     t = torch.from_numpy(lab).cuda()
-    with L.Context(max_n=n, max_nnz=len(idx)) as ctx:
+    with L.Context(max_n=n, max_nnz=len(idx) + 8) as ctx:
         calls = [lambda: ctx.modularity(g, t), lambda: L.modularity_noalloc(g, t)]
         if not fault.startswith("label"):
             calls.append(lambda: ctx.static(g))
+            calls.append(lambda: ctx.apply_batch(g, None, L.Edges.from_numpy(([0], [n - 1], [1]))))
         calls.append(lambda: ctx.update(g, t, None, None, "DF"))
         for call in calls:
             with pytest.raises(L.LeidenError) as e:
@@ -98,3 +99,61 @@ def test_malformed_inputs_are_refused(fault):
             assert e.value.code == -1
         good = S.rmat(11, 8, seed=4)
         assert np.array_equal(ctx.static(L.Graph.from_numpy(*good))[0].cpu().numpy(), O.static(*good).membership)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_batch_application_reads_any_alignment(shift):
+    # entry arrays that start 4, 8 or 12 bytes past a 16-byte boundary
+    off, idx, w = S.chung_lu(3000, 15000, 2.1, 1, 4, seed=5)
+    big_i = torch.zeros(len(idx) + 8, dtype=torch.int32, device="cuda")
+    big_w = torch.zeros(len(idx) + 8, dtype=torch.int32, device="cuda")
+    big_i[shift:shift + len(idx)] = torch.from_numpy(idx).cuda()
+    big_w[shift:shift + len(idx)] = torch.from_numpy(w).cuda()
+    g = L.Graph(torch.from_numpy(off).cuda(), big_i[shift:shift + len(idx)], big_w[shift:shift + len(idx)])
+    dels, ins = S.random_batch(off, idx, w, 200, seed=6)
+    want = O.apply_batch(off, idx, w, dels, ins)
+    with L.Context(max_n=g.n, max_nnz=g.nnz + 1024) as ctx:
+        got = ctx.apply_batch(g, L.Edges.from_numpy(dels), L.Edges.from_numpy(ins))
+    for a, b in zip((got.off, got.idx, got.w), want):
+        assert np.array_equal(a.cpu().numpy(), b)
+
+
+def heavy_batch(n, hub_deg, hub_ins, hub_dels, seed, repeats=1):
+    """A graph whose vertex 0 has hub_deg neighbours, and a batch that inserts
+    hub_ins edges at it (each listed `repeats` times) and deletes hub_dels."""
+    rng = np.random.default_rng(seed)
+    nb = rng.choice(np.arange(1, n), hub_deg + hub_ins, replace=False)
+    u = np.concatenate([np.zeros(hub_deg, np.int64), rng.integers(1, n, 2 * n)])
+    v = np.concatenate([nb[:hub_deg], rng.integers(1, n, 2 * n)])
+    g = S.edges_to_csr(n, u, v, rng.integers(1, 9, len(u)))
+    off, idx, w = g
+    pick = rng.choice(off[1], hub_dels, replace=False)
+    dels = (np.zeros(hub_dels, np.int32), idx[pick], w[pick])
+    # new neighbours, repeats of them, and some of the old ones reweighted
+    t = np.concatenate([np.repeat(nb[hub_deg:], repeats), np.setdiff1d(idx[:off[1]], idx[pick])[:hub_ins // 3]])
+    t = rng.permutation(t).astype(np.int32)
+    ins = (np.zeros(len(t), np.int32), t, rng.integers(1, 5, len(t)).astype(np.int32))
+    return g, dels, ins
+
+
+@pytest.mark.parametrize("hub_deg,hub_ins,hub_dels,repeats", [
+    (40, 8, 4, 1), (40, 16, 1, 1), (40, 17, 0, 1),              # around the serial limit of 16 updates
+    (256, 3, 0, 1), (257, 3, 3, 1), (300, 255, 40, 1), (300, 257, 40, 2),   # around one merge piece
+    (512, 1, 0, 1), (513, 200, 100, 3), (1024, 255, 1, 1),
+    (6000, 3000, 1000, 1), (6000, 3000, 1096, 1), (9000, 4000, 2000, 2),    # around the shared-memory sort
+])
+def test_batches_on_a_heavy_row(hub_deg, hub_ins, hub_dels, repeats):
+    g, dels, ins = heavy_batch(20000, hub_deg, hub_ins, hub_dels, 7, repeats)
+    want = O.apply_batch(*g, dels, ins)
+    with L.Context(max_n=20000, max_nnz=len(g[1]) + 4 * len(ins[0]) + 2 * len(dels[0])) as ctx:
+        got = ctx.apply_batch(L.Graph.from_numpy(*g), L.Edges.from_numpy(dels), L.Edges.from_numpy(ins))
+        for a, b in zip((got.off, got.idx, got.w), want):
+            assert np.array_equal(a.cpu().numpy(), b)
+        # refused as before: a deletion listed twice, one of a wrong weight
+        if hub_dels >= 2:
+            twice = tuple(np.concatenate([x, x[:1]]) for x in dels)
+            wrong = (dels[0], dels[1], dels[2] + 1)
+            for bad in (twice, wrong):
+                with pytest.raises(L.LeidenError) as e:
+                    ctx.apply_batch(L.Graph.from_numpy(*g), L.Edges.from_numpy(bad), L.Edges.from_numpy(ins))
+                assert e.value.code == -1
