@@ -7,8 +7,8 @@
 // 3. per community, scanCommunities with self = true over every member row
 //    into a hashtable of (neighbour community d, summed weight); the entries
 //    land in the community's hole range and cdist[c] counts them.  Work is
-//    bucketed by total degree: a warp with a shared table, a block with a
-//    shared table, or, for the largest communities, their entries split by
+//    bucketed by total degree: eight lanes or a warp with a shared table, a
+//    block with a shared table, or, for the largest communities, their entries split by
 //    target into shared-memory-sized buckets hashed by many blocks (the load
 //    imbalance of selective refinement, Sec. 4.4);
 // 4. exclusive scan of cdist gives the compact super-vertex offsets; a copy
@@ -122,37 +122,6 @@ __device__ __forceinline__ void walk_segments(const GraphView<WT> &g, const int3
   }
 }
 
-// The warp walks the rows of members cv[m0 .. m1) as one flattened range:
-// each batch of 32 members is prefix-summed across the lanes, and every lane
-// finds the member of its entry by a binary search over the shuffled sums.
-// Every loop that contains a shuffle is uniform across the warp.
-template <typename WT>
-__device__ __forceinline__ void warp_rows_into_table(const GraphView<WT> &g, const int32_t *C,
-                                                     const int32_t *cv, int64_t m0, int64_t m1,
-                                                     int64_t mstep, int32_t *keys, u64 *vals,
-                                                     uint32_t mask, int sh, u64 *err, u64 *scratch) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t mb = m0; mb < m1; mb += mstep) {
-    const int64_t m = mb + lane;
-    int64_t start = 0, deg = 0;
-    if (m < m1) {
-      const int32_t v = cv[m];
-      start = g.off[v];
-      deg = g.off[v + 1] - start;
-    }
-    int64_t incl = deg;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int64_t y = shfl_i64(incl, (lane - o) & 31);
-      if (lane >= o) incl += y;
-    }
-    const int64_t total = shfl_i64(incl, 31);
-    walk_segments(g, C, start, deg, incl, total, err, [&](int32_t c, u64 wv, bool act, int64_t) {
-      u64 sum = 0;
-      if (warp_combine((unsigned long long)(uint32_t)c, act, wv, &sum, scratch)) tadd(keys, vals, mask, sh, c, sum, err);
-    });
-  }
-}
-
 // Emit the occupied slots of a table into [base, ...), warp-cooperative;
 // returns (count, weight sum) in lane 0 of each participating warp via the
 // shared counters.
@@ -177,37 +146,134 @@ __device__ __forceinline__ void warp_emit(const int32_t *keys, const u64 *vals, 
   if (lane == 0 && ws) atomicAdd((u64 *)wsum, (u64)ws);
 }
 
-// Warp tier: one warp per community, table of 2^LOG2H shared slots.
-template <int LOG2H, typename WT>
-__global__ void __launch_bounds__(256) agg_warp_k(GraphView<WT> g, const int32_t *C, const int32_t *list,
-                                                  int64_t nlist, const int64_t *coff, const int64_t *hoff,
-                                                  const int32_t *cv, int32_t *hidx, int64_t *hw,
-                                                  int64_t *cdist, int64_t *Kout, u64 *err) {
-  constexpr int H = 1 << LOG2H;
+// Adds w to a table value as two 32-bit words, the carry passed on by the adder
+// that wrapped the low one (a 64-bit shared-memory atomic is a
+// compare-and-swap loop).
+__device__ __forceinline__ void agg_val_add(u64 *p, u64 w) {
+  uint32_t *h = reinterpret_cast<uint32_t *>(p);
+  const uint32_t lo = (uint32_t)w;
+  const uint32_t old = atomicAdd(&h[0], lo);
+  const uint32_t hi = (uint32_t)(w >> 32) + (old + lo < old ? 1u : 0u);
+  if (hi) atomicAdd(&h[1], hi);
+}
+
+// Group tiers: G lanes per community (8 or 32), total degree at most half the
+// table of 2^LOG2H shared slots.  The members' rows are walked as one flat
+// range: G members at a time, their degrees prefix-summed across the group,
+// each lane finding the member of its entry by a binary search over the
+// shuffled sums, AGG_UNROLL entries per lane in flight.  The lane that
+// occupies a slot lists it, and the group emits and resets the listed slots,
+// so a community costs its entries and not its table.
+//
+// Bound by the chain member -> row -> entry -> C'[j] of a short community;
+// hence four communities a warp where they have up to 64 entries.  First
+// aggregation of a 6.25e6-vertex grid (mean total degree 8): 3.02 ms with a
+// warp and a cleared, scanned 128-slot table per community, 0.45 ms here; a
+// 6.25e7-entry Chung-Lu graph's communities of up to 384 entries 2.29 ms then,
+// of up to 512 entries 0.73 ms now.
+template <int G, int LOG2H, typename WT>
+__global__ void __launch_bounds__(256) agg_group_k(GraphView<WT> g, const int32_t *C, const int32_t *list,
+                                                   int64_t nlist, const int64_t *coff, const int64_t *hoff,
+                                                   const int32_t *cv, int32_t *hidx, int64_t *hw, int64_t *cdist,
+                                                   int64_t *Kout, u64 *err) {
+  constexpr int H = 1 << LOG2H, GPB = 256 / G;
   extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-  u64 *vals = reinterpret_cast<u64 *>(smem) + (size_t)warp * H;
-  int32_t *keys = reinterpret_cast<int32_t *>(reinterpret_cast<u64 *>(smem) + (size_t)wpb * H) + (size_t)warp * H;
-  __shared__ unsigned long long s_cnt[8];
-  __shared__ int64_t s_ws[8];
-  __shared__ u64 wscratch[8][32];
-  const int64_t w0 = (int64_t)blockIdx.x * wpb + warp, nw = (int64_t)gridDim.x * wpb;
-  for (int64_t li = w0; li < nlist; li += nw) {
+  const int grp = threadIdx.x / G, gl = threadIdx.x % G;
+  u64 *vals = reinterpret_cast<u64 *>(smem) + (size_t)grp * H;
+  int32_t *keys = reinterpret_cast<int32_t *>(reinterpret_cast<u64 *>(smem) + (size_t)GPB * H) + (size_t)grp * H;
+  uint16_t *used = reinterpret_cast<uint16_t *>(reinterpret_cast<int32_t *>(reinterpret_cast<u64 *>(smem) +
+                                                                             (size_t)GPB * H) +
+                                                (size_t)GPB * H) + (size_t)grp * (H / 2);
+  __shared__ int s_cnt[GPB];
+  const unsigned gm = G == 32 ? FULL_MASK : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+  for (int s = gl; s < H; s += G) { keys[s] = LEIDEN_EMPTY_KEY; vals[s] = 0; }
+  if (gl == 0) s_cnt[grp] = 0;
+  __syncwarp(gm);
+  for (int64_t li = (int64_t)blockIdx.x * GPB + grp; li < nlist; li += (int64_t)gridDim.x * GPB) {
     const int32_t c = list[li];
-    // table sized for this community: 2^lh >= 2 * total degree, lh <= LOG2H
-    const int64_t td = hoff[c + 1] - hoff[c];
-    int lh = 1;
-    while (lh < LOG2H && ((int64_t)1 << lh) < 2 * td) lh++;
-    const int Hc = 1 << lh;
-    for (int s = lane; s < Hc; s += 32) { keys[s] = LEIDEN_EMPTY_KEY; vals[s] = 0; }
-    if (lane == 0) { s_cnt[warp] = 0; s_ws[warp] = 0; }
-    __syncwarp();
-    warp_rows_into_table(g, C, cv, coff[c], coff[c + 1], 32, keys, vals, Hc - 1, 32 - lh, err, wscratch[warp]);
-    __syncwarp();
-    warp_emit(keys, vals, Hc, 0, 32, hidx, hw, hoff[c], &s_cnt[warp], &s_ws[warp]);
-    __syncwarp();
-    if (lane == 0) { cdist[c] = (int64_t)s_cnt[warp]; Kout[c] = s_ws[warp]; }
-    __syncwarp();
+    const int64_t m0 = coff[c], m1 = coff[c + 1], out = hoff[c];
+    for (int64_t mb = m0; mb < m1; mb += G) {
+      int64_t rs = 0;
+      int deg = 0;
+      if (mb + gl < m1) {
+        const int32_t v = cv[mb + gl];
+        rs = g.off[v];
+        deg = (int)(g.off[v + 1] - rs);
+      }
+      int incl = deg;
+#pragma unroll
+      for (int o = 1; o < G; o <<= 1) {
+        const int y = __shfl_up_sync(gm, incl, o, G);
+        if (gl >= o) incl += y;
+      }
+      const int total = __shfl_sync(gm, incl, G - 1, G);
+      rs -= incl - deg;   // row start less the member's place in the flat range
+      for (int t0 = 0; t0 < total; t0 += G * AGG_UNROLL) {
+        int32_t cc[AGG_UNROLL];
+        int64_t wv[AGG_UNROLL];
+#pragma unroll
+        for (int u = 0; u < AGG_UNROLL; u++) {
+          const int t = t0 + u * G + gl;
+          int k = 0;   // first lane whose inclusive sum exceeds t
+#pragma unroll
+          for (int b = G / 2; b; b >>= 1)
+            if (__shfl_sync(gm, incl, k + b - 1, G) <= t) k += b;
+          const int64_t e = (int64_t)__shfl_sync(gm, (long long)rs, k, G) + t;
+          cc[u] = t < total ? g.idx[e] : -1;
+          wv[u] = t < total ? (int64_t)g.w[e] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < AGG_UNROLL; u++) {
+          if (cc[u] == -1) continue;
+          if ((uint32_t)cc[u] >= (uint32_t)g.n) { atomicOr(err, 64ull); cc[u] = -1; }
+          else cc[u] = C[cc[u]];
+        }
+#pragma unroll
+        for (int u = 0; u < AGG_UNROLL; u++) {
+          const int32_t d = cc[u];
+          if (d < 0) continue;
+          uint32_t s = hash32(d) >> (32 - LOG2H);
+          bool done = false;
+          for (int probe = 0; probe < H; probe++) {
+            int32_t k = *(volatile int32_t *)&keys[s];
+            bool fresh = false;
+            if (k == LEIDEN_EMPTY_KEY) {
+              k = atomicCAS(&keys[s], LEIDEN_EMPTY_KEY, d);
+              fresh = k == LEIDEN_EMPTY_KEY;
+            }
+            if (fresh || k == d) {
+              agg_val_add(&vals[s], (u64)wv[u]);
+              if (fresh) used[atomicAdd(&s_cnt[grp], 1)] = (uint16_t)s;
+              done = true;
+              break;
+            }
+            s = (s + 1) & (H - 1);
+          }
+          if (!done) atomicOr(err, 16ull);
+        }
+      }
+    }
+    __syncwarp(gm);
+    const int n = s_cnt[grp];
+    int64_t ks = 0;
+    for (int k = gl; k < n; k += G) {
+      const uint32_t s = used[k];
+      const int64_t v = (int64_t)vals[s];
+      hidx[out + k] = keys[s];
+      hw[out + k] = v;
+      keys[s] = LEIDEN_EMPTY_KEY;
+      vals[s] = 0;
+      ks += v;
+    }
+#pragma unroll
+    for (int o = G / 2; o; o >>= 1) ks += (int64_t)__shfl_xor_sync(gm, (long long)ks, o, G);
+    __syncwarp(gm);
+    if (gl == 0) {
+      cdist[c] = n;
+      Kout[c] = ks;
+      s_cnt[grp] = 0;
+    }
+    __syncwarp(gm);
   }
 }
 
@@ -765,8 +831,8 @@ __global__ void agg_compact_win_k(const int32_t *list, int64_t nlist, const int6
   }
 }
 
-// Communities by total degree: a warp with a small or a larger shared table,
-// a block, or the bucketed multi-block path for giant ones -- the GPU form of
+// Communities by total degree: eight lanes or a warp with a shared table, a
+// block, or the bucketed multi-block path for giant ones -- the GPU form of
 // the paper's Optimized Aggregation (Sec. 4.4), which keeps one large
 // unrefined community from holding up a worker.  uniform = 1 sends every
 // community through the multi-block path instead (one method for all sizes,
@@ -776,8 +842,10 @@ static TierTable agg_tiers(int uniform) {
   int k = 0;
   tt.t[k++] = {TIER_SKIP, 0, 0, 0, 0};
   if (!uniform) {
-    tt.t[k++] = {TIER_GROUP, 48, 32, 7, 256};     // warp, 128 slots
-    tt.t[k++] = {TIER_GROUP, 384, 32, 10, 128};   // warp, 1024 slots
+    tt.t[k++] = {TIER_GROUP, 16, 8, 5, 256};      // 8 lanes, 32 slots
+    tt.t[k++] = {TIER_GROUP, 64, 8, 7, 256};      // 8 lanes, 128 slots
+    tt.t[k++] = {TIER_GROUP, 256, 32, 9, 256};    // warp, 512 slots
+    tt.t[k++] = {TIER_GROUP, 512, 32, 10, 256};   // warp, 1024 slots
     tt.t[k++] = {TIER_BLOCK, 2048, 0, 12, 256};   // block, 4096 slots (48 KB: 4 blocks per SM)
   }
   tt.t[k++] = {TIER_GLOBAL, INT64_MAX, 0, 0, 256};
@@ -815,17 +883,19 @@ int aggregate(GraphView<WT> g, const int32_t *C, int64_t nc, int64_t *off2, int3
     const int64_t nl = koff[t + 1] - koff[t];
     if (nl <= 0) continue;
     if (T.kind == TIER_GROUP) {
-      const size_t smem = (size_t)(T.threads / 32) * (1u << T.log2H) * 12;
-      const unsigned blocks = gridn(nl * 32, T.threads, (int64_t)wk.sms * 16);
-      if (T.log2H == 7) {
-        LK_COUNTED agg_warp_k<7, WT><<<blocks, T.threads, smem, s>>>(g, C, list, nl, wk.coff, wk.hoff, wk.cv, wk.hidx,
-                                                          wk.hw, wk.cdist, Kout, err);
-      } else {
-        auto k = agg_warp_k<10, WT>;
+      // per group: table (12 bytes a slot) and the list of its occupied slots
+      const size_t smem = (size_t)(256 / T.G) * (1u << T.log2H) * 13;
+      auto launch = [&](auto k) {
         ensure_smem((const void *)k, smem);
-        LK_COUNTED k<<<blocks, T.threads, smem, s>>>(g, C, list, nl, wk.coff, wk.hoff, wk.cv, wk.hidx, wk.hw,
-                                          wk.cdist, Kout, err);
-      }
+        const int64_t cap = resident_blocks((const void *)k, 256, smem, wk.sms);
+        const int64_t need = (nl * T.G + 255) / 256;
+        LK_COUNTED k<<<(unsigned)(need < cap ? need : cap), 256, smem, s>>>(g, C, list, nl, wk.coff, wk.hoff, wk.cv,
+                                                                            wk.hidx, wk.hw, wk.cdist, Kout, err);
+      };
+      if (T.log2H == 5) launch(agg_group_k<8, 5, WT>);
+      else if (T.log2H == 7) launch(agg_group_k<8, 7, WT>);
+      else if (T.log2H == 9) launch(agg_group_k<32, 9, WT>);
+      else launch(agg_group_k<32, 10, WT>);
     } else if (T.kind == TIER_BLOCK) {
       // table, member batch (16 bytes a thread), combine scratch (256 bytes a warp)
       const size_t smem = (size_t)(1u << T.log2H) * 12 + (size_t)T.threads * 16 + (size_t)(T.threads / 32) * 256;

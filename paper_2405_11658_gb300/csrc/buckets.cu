@@ -39,18 +39,23 @@ __global__ void __launch_bounds__(BK_THREADS) bucket_count_k(const int64_t *off,
     blockhist[(int64_t)k * gridDim.x + blockIdx.x] = hist[k];
 }
 
+// 32-bit cursors within the block's run of a key: most vertices of a block
+// share a key, and 64-bit shared-memory atomics are compare-and-swap loops
+// (350 us at 2.5e6 communities, 28 us with 32-bit ones).
 __global__ void __launch_bounds__(BK_THREADS) bucket_scatter_k(const int64_t *off, int64_t n, int log2S,
                                                                TierMax tm, int nkeys,
                                                                const int64_t *scanned, int32_t *list) {
-  extern __shared__ int64_t cur[];
-  for (int k = threadIdx.x; k < nkeys; k += blockDim.x)
-    cur[k] = scanned[(int64_t)k * gridDim.x + blockIdx.x];
+  extern __shared__ int64_t base_s[];
+  unsigned *cur = reinterpret_cast<unsigned *>(base_s + nkeys);
+  for (int k = threadIdx.x; k < nkeys; k += blockDim.x) {
+    base_s[k] = scanned[(int64_t)k * gridDim.x + blockIdx.x];
+    cur[k] = 0;
+  }
   __syncthreads();
   const int64_t base = (int64_t)blockIdx.x * BK_CHUNK;
   for (int64_t v = base + threadIdx.x; v < n && v < base + BK_CHUNK; v += blockDim.x) {
     const int key = det_class((int32_t)v, log2S) * tm.n + tier_of(off[v + 1] - off[v], tm);
-    const int64_t pos = (int64_t)atomicAdd((u64 *)&cur[key], 1ull);
-    list[pos] = (int32_t)v;
+    list[base_s[key] + atomicAdd(&cur[key], 1u)] = (int32_t)v;
   }
 }
 
@@ -75,7 +80,7 @@ void launch_buckets(const int64_t *off, int64_t n, int log2S, const TierTable &t
   LK_COUNTED bucket_count_k<<<(unsigned)nb, BK_THREADS, nkeys * sizeof(int32_t), s>>>(off, n, log2S, tm, nkeys,
                                                                           blockhist);
   exclusive_scan<int32_t>(blockhist, scanned, nb * nkeys, scan_tmp, s);
-  LK_COUNTED bucket_scatter_k<<<(unsigned)nb, BK_THREADS, nkeys * sizeof(int64_t), s>>>(off, n, log2S, tm, nkeys,
+  LK_COUNTED bucket_scatter_k<<<(unsigned)nb, BK_THREADS, nkeys * (sizeof(int64_t) + sizeof(unsigned)), s>>>(off, n, log2S, tm, nkeys,
                                                                             scanned, list);
   LK_COUNTED bucket_koff_k<<<1, 256, 0, s>>>(scanned, nkeys, nb, koff_dev);
 }

@@ -137,3 +137,26 @@ def test_batch_with_hub_rows(opts):
         outs, res = batch.run([{"graph": G}] * 3, L.Opts(**opts))
         for out, r in zip(outs, res):
             assert r["status"] == 0 and np.array_equal(out.cpu().numpy(), ref.membership) and r["q"] == ref.q
+
+
+@pytest.mark.parametrize("size", [2, 4, 5, 8, 9, 16, 17, 23, 24, 45, 46, 60])
+def test_aggregation_tier_edges(size):
+    # cliques joined in a ring: communities of total degree size * (size - 1)
+    # + 2, on both sides of the aggregation tiers' limits 16, 64, 256, 512 and
+    # 2048 (a context with a tier table of its own aggregates through them)
+    a, b = np.triu_indices(size, 1)
+    count = 300
+    base = np.arange(count) * size
+    u, v = (base[:, None] + a).ravel(), (base[:, None] + b).ravel()
+    g = S.edges_to_csr(count * size, np.concatenate([u, base + size - 1]), np.concatenate([v, np.roll(base, -1)]),
+                       np.random.default_rng(size).integers(1, 1 << (22 if size < 40 else 18), len(u) + count))  # 2m < 2^40
+    ref = O.static(*g, O.LeidenOpts())
+    tiers = L.default_tiers()
+    tiers[0]["threads"] = 128
+    with L.Context(max_n=count * size, max_nnz=len(g[1])) as ctx:
+        ctx.set_tiers(tiers)
+        memb, q = ctx.static(L.Graph.from_numpy(*g))
+        st = ctx.stats()
+    assert np.array_equal(memb.cpu().numpy(), ref.membership) and q == ref.q
+    for name in ("iters", "nv", "nnz", "moves", "refine_moves"):
+        assert st[name][:ref.stats["passes"]] == ref.stats[name], name
