@@ -119,22 +119,26 @@ int capture(leiden_batch *b, const SmallOpts &so, int k) {
   return LEIDEN_OK;
 }
 
-// Clusters of 2^k blocks for the largest `*wide` of the graphs, single blocks
-// for the others.  A cluster of c blocks for w graphs leaves sms - w c blocks
-// for the other count - w, so w = (sms - count) / (c - 1) keeps every graph on
-// SMs of its own; the largest c that still covers a third of the graphs (their
-// sizes differ, and the largest ones finish last).  64 graphs of 1e3..1e4
-// vertices: single blocks 28.4 ms, clusters of 2 for all 19.7, of 4 for the
-// 20 largest 18.3, of 4 for all 20.0, of 8 for the 20 largest 26.9.
-int cluster_log2(int count, int sms, int64_t largest, int32_t *wide) {
+// Clusters of 2^k blocks for the largest `*wide` of the graphs (sizes: their
+// vertices + entries, largest first), single blocks for the others.  A cluster
+// of c blocks for w graphs leaves sms - w c blocks for the other count - w, so
+// w = (sms - count) / (c - 1) keeps every graph on SMs of its own; the largest
+// c that still covers a third of the graphs (their sizes differ, and the
+// largest ones finish last).  A graph below 6144 c is not worth the cluster's
+// barriers, about 1 us each against the block's 0.05: with clusters of 4 for
+// graphs of 1e3 vertices (1.1e4) a batch took 15% longer than with one 512-
+// thread block each.  64 graphs of 1e3..1e4 vertices (1.1e4 .. 1.1e5): single
+// blocks 28.4 ms, clusters of 2 for all 19.7, of 4 for the 20 largest 18.3, of
+// 4 for all 20.0, of 8 for the 20 largest 26.9.
+int cluster_log2(int count, int sms, const std::vector<int64_t> &sizes, int32_t *wide) {
+  *wide = 0;
   for (int k = 4; k > 0; k--) {
     const int c = 1 << k;
     const int w = std::min(count, std::max(0, (sms - count) / (c - 1)));
-    if (3 * w < count || largest < (int64_t)1024 * c) continue;
-    *wide = w;
+    if (3 * w < count || sizes[0] < (int64_t)6144 * c) continue;
+    while (*wide < w && sizes[*wide] >= (int64_t)3072 * c) ++*wide;
     return k;
   }
-  *wide = 0;
   return 0;
 }
 
@@ -223,9 +227,9 @@ extern "C" int leiden_batch_run(leiden_batch *b, int32_t count, const leiden_bat
   SmallJob *jobs = reinterpret_cast<SmallJob *>(b->h_desc + sizeof(SmallHeader));
   memset(hdr, 0, sizeof(SmallHeader));
   hdr->count = count;
-  int64_t largest = 0;
-  if (count) largest = items[order[0]].g.nnz + items[order[0]].g.n;
-  const int lc = cluster_log2(count, b->sms, largest, &hdr->wide);
+  std::vector<int64_t> sizes(count);
+  for (int k = 0; k < count; k++) sizes[k] = items[order[k]].g.nnz + items[order[k]].g.n;
+  const int lc = cluster_log2(count, b->sms, sizes, &hdr->wide);
   hdr->next = 0;
   hdr->next1 = (uint32_t)hdr->wide;
   int64_t at = 0;

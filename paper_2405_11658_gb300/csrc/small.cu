@@ -15,8 +15,7 @@
 // barriers, and with fewer graphs than SMs the others would be idle anyway.
 // 64 graphs of 1e3..1e4 vertices, half of them updates: 50 ms with a 512-
 // thread block per graph, tables cleared per vertex and 128-bit scores
-// throughout, 28 ms on single team blocks, 18 ms with clusters for the
-// largest.
+// throughout, 14 ms as here.
 #include <limits.h>
 
 #include <mutex>
@@ -84,20 +83,25 @@ struct SmallLevel {
     n = n_; nnz = nnz_; off = off_; idx = idx_; w = w_;
   }
 };
-struct SmallState {
-  SmallArrays a;
-  SmallConst ct;
-  SmallLevel<int64_t> g;
-};
-
 // Workspace of one graph, carved from its slice of the batch arena.
 struct WS {
   int32_t *Ctop, *idx[2];
   int64_t *off[2], *w[2];
   int64_t slots;
 };
+struct SmallState {
+  SmallArrays a;
+  SmallConst ct;
+  SmallLevel<int64_t> g;
+  WS w;
+  // the pass at hand: its number, level buffer (-1: the input), sizes, largest
+  // K', tolerance and score width
+  int lp, cur, narrow;
+  int64_t nv, nnz, kmax;
+  double tau;
+};
 
-// Carves the slice; one thread of the block writes the array table.
+// Carves the slice (one thread of the block).
 __device__ __forceinline__ void carve_ws(char *base, int64_t n, int64_t nnz, u64 *err, WS &w, SmallArrays &a) {
   const SmallLayout L = small_layout(n, nnz);
   w.Ctop = (int32_t *)(base + L.Ctop);
@@ -108,7 +112,6 @@ __device__ __forceinline__ void carve_ws(char *base, int64_t n, int64_t nnz, u64
   w.w[0] = (int64_t *)(base + L.wA);
   w.w[1] = (int64_t *)(base + L.wB);
   w.slots = L.slots;
-  if (threadIdx.x) return;
   a.C = (int32_t *)(base + L.Cp);
   a.CB = (int32_t *)(base + L.CB);
   a.rep = (int32_t *)(base + L.rep);
@@ -244,20 +247,33 @@ extern __shared__ __align__(16) unsigned char small_dyn[];
 __device__ __forceinline__ SmallState &small_state() { return *reinterpret_cast<SmallState *>(small_dyn + kState); }
 
 
-// One pass with the level's score width, a function of its own per width
-// (inlined into one body they spill and take minutes to compile).
-template <typename ST>
-__device__ __noinline__ void small_pass(int lp, double tau, int max_iters, int64_t slots, Team *t) {
-  Team tt = *t;
+// The pass at hand of state: clears the control words, points the arrays at the
+// level and its output, picks the score width.
+__device__ __forceinline__ void small_next(const SmallJob &j, const SmallOpts &o, const Team &t, SmallCtl *ctl) {
   SmallState &s = small_state();
-  team_pass<true, int64_t, ST>(s.g, s.a, s.ct, lp, tau, max_iters, slots, tt, small_dyn,
-                               *reinterpret_cast<TeamShared<ST> *>(small_dyn + kTables));
-  t->dead = tt.dead;
+  unsigned *z = reinterpret_cast<unsigned *>(&ctl->t);
+  for (unsigned k = (unsigned)t.index(); k < sizeof(TeamCtl) / 4; k += (unsigned)(t.nb * TEAM_THREADS)) z[k] = 0;
+  if (threadIdx.x == 0) {
+    const int cur = s.cur, dst = cur < 0 ? 0 : 1 - cur;
+    s.a.off2 = s.w.off[dst];
+    s.a.idx2 = s.w.idx[dst];
+    s.a.w2 = s.w.w[dst];
+    if (cur < 0) s.g.set(j.n, j.nnz, j.off, j.idx, s.w.w[1]);
+    else s.g.set(s.nv, s.nnz, s.w.off[cur], s.w.idx[cur], s.w.w[cur]);
+    // 64-bit scores while every product stays below 2^62 (see narrow_scores)
+    const int64_t pq = o.p > o.q ? o.p : o.q, two_m = s.ct.two_m;
+    s.narrow = !LK_FORCE_WIDE_SCORES && s.kmax < ((int64_t)1 << 31) &&
+               (i128)s.kmax * two_m * pq < ((i128)1 << 62);
+  }
 }
 
-// The whole of Alg. leiden for one job.
-__device__ __noinline__ void run_job(const SmallJob &j, const SmallOpts &o, SmallResult *res, Team t, SmallCtl *ctl) {
-  WideShared &sm = *reinterpret_cast<WideShared *>(small_dyn + kTables);
+// Everything before the first pass of a job; false when there is none (bad
+// input, or a result without passes).  The functions around the passes are not
+// inlined: the passes, inlined once each into the kernel, then have its
+// registers to themselves (as functions of their own they spilled twice as
+// much: 64 graphs of 1e3..1e4 vertices 16.6 ms, 14.1 so).
+__device__ __noinline__ bool small_setup(const SmallJob &j, const SmallOpts &o, SmallResult *res, Team t,
+                                         SmallCtl *ctl) {
   const int64_t N = j.n, gt = t.index(), nt = (int64_t)t.nb * TEAM_THREADS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wg = warp * t.nb + t.rank, W = t.nb * TEAM_WARPS;
@@ -269,17 +285,17 @@ __device__ __noinline__ void run_job(const SmallJob &j, const SmallOpts &o, Smal
     res->changed0 = 0;
     ctl->err = ctl->two_m = ctl->kmax = ctl->inside = ctl->sq[0] = ctl->sq[1] = ctl->affected = 0;
   }
-  TEAM_SYNC_OR();
+  TEAM_SYNC_OR(false);
   check_job(j, t, &ctl->err);
-  TEAM_SYNC_OR();
+  TEAM_SYNC_OR(false);
   if (*(volatile u64 *)&ctl->err) {
     if (lead) res->status = LEIDEN_EINVAL;
-    return;
+    return false;
   }
-  WS w;
   SmallState &state = small_state();
-  carve_ws(j.ws, N, j.nnz, &ctl->err, w, state.a);
+  if (threadIdx.x == 0) carve_ws(j.ws, N, j.nnz, &ctl->err, state.w, state.a);
   __syncthreads();
+  const WS &w = state.w;
   const SmallArrays &a0 = state.a;
   const bool upd = j.mode != LEIDEN_STATIC;
   // K = row sums of G^t; 2m = their total
@@ -307,11 +323,11 @@ __device__ __noinline__ void run_job(const SmallJob &j, const SmallOpts &o, Smal
     a0.ch[i] = upd ? (o.refine_all_first_pass ? 1 : 0) : 1;
     a0.processed[i] = (upd && j.mode == LEIDEN_DF) ? 1 : 0;
   }
-  TEAM_SYNC_OR();
+  TEAM_SYNC_OR(false);
   const int64_t two_m = (int64_t)__ldcg(&ctl->two_m);
   if (two_m < 0 || two_m >= ((int64_t)1 << 40)) {
     if (lead) res->status = LEIDEN_EOVERFLOW;
-    return;
+    return false;
   }
   if (threadIdx.x == 0) {
     SmallConst &ct = state.ct;
@@ -339,84 +355,92 @@ __device__ __noinline__ void run_job(const SmallJob &j, const SmallOpts &o, Smal
       if (same && !o.refine_all_first_pass) a0.ch[j.prior[u]] = 1;                       // changedCommunities
       if (j.mode == LEIDEN_DF && same == del) { a0.processed[u] = 0; a0.processed[v] = 0; }  // Alg. frontier
     }
-    TEAM_SYNC_OR();
+    TEAM_SYNC_OR(false);
     if (j.mode == LEIDEN_DS) {
-      if (!mark_ds(j, a0, state.ct, t)) return;
-      TEAM_SYNC_OR();
+      if (!mark_ds(j, a0, state.ct, t)) return false;
+      TEAM_SYNC_OR(false);
     }
     u64 k = 0;
     for (int64_t i = gt; i < N; i += nt) k += a0.processed[i] == 0;
     for (int s = 16; s; s >>= 1) k += (u64)shfl_xor_i64((int64_t)k, s);
     if (lane == 0 && k) atomicAdd(&ctl->affected, k);
-    TEAM_SYNC_OR();
+    TEAM_SYNC_OR(false);
     if (lead) res->affected0 = (int64_t)__ldcg(&ctl->affected);
   } else {
     if (lead) res->affected0 = N;
-    TEAM_SYNC_OR();
+    TEAM_SYNC_OR(false);
   }
 
-  double tau = o.tol;
-  int cur = -1;  // -1: the input graph; 0 / 1: level buffers
-  int64_t nv = N, nnz_cur = j.nnz;
-  int64_t kmax = (int64_t)__ldcg(&ctl->kmax);
-  const int64_t pq = o.p > o.q ? o.p : o.q;
-  for (int lp = 0; lp < o.max_passes; lp++) {
-    // the pass's control words
-    {
-      unsigned *z = reinterpret_cast<unsigned *>(&ctl->t);
-      for (unsigned k = (unsigned)gt; k < sizeof(TeamCtl) / 4; k += (unsigned)nt) z[k] = 0;
-    }
-    const int dst = cur < 0 ? 0 : 1 - cur;
-    if (threadIdx.x == 0) {
-      state.a.off2 = dst ? w.off[1] : w.off[0];
-      state.a.idx2 = dst ? w.idx[1] : w.idx[0];
-      state.a.w2 = dst ? w.w[1] : w.w[0];
-      if (cur < 0) state.g.set(N, j.nnz, j.off, j.idx, w.w[1]);
-      else state.g.set(nv, nnz_cur, cur ? w.off[1] : w.off[0], cur ? w.idx[1] : w.idx[0], cur ? w.w[1] : w.w[0]);
-    }
-    // 64-bit scores while every product stays below 2^62 (see narrow_scores)
-    const bool narrow = !LK_FORCE_WIDE_SCORES && kmax < ((int64_t)1 << 31) &&
-                        (i128)kmax * two_m * pq < ((i128)1 << 62);
-    TEAM_SYNC_OR();
-    if (nv == 0) {
-      // an empty graph: one pass over nothing
-      if (lead && lp < LEIDEN_STATS_PASSES) {
-        res->passes = lp + 1;
-        res->iters[lp] = 1;
-        res->nv[lp] = res->nnz[lp] = res->moves[lp] = res->refine_moves[lp] = 0;
-      }
-      break;
-    }
-    if (narrow) small_pass<int64_t>(lp, tau, o.max_iters, w.slots, &t);
-    else small_pass<i128>(lp, tau, o.max_iters, w.slots, &t);
-    TEAM_SYNC_OR();
-    const volatile TeamCtl &h = ctl->t;
-    const int status = h.status;
-    if (lead && lp < LEIDEN_STATS_PASSES) {
-      if (lp == 0) res->changed0 = (int64_t)h.changed;
-      res->nnz[lp] = nnz_cur;
-      res->passes = lp + 1;
-      res->iters[lp] = h.li;
-      res->nv[lp] = nv;
-      res->moves[lp] = h.moves;
-      res->refine_moves[lp] = (int64_t)h.rmoves;
-    }
-    if (threadIdx.x == 0) {
-      state.ct.dynamic = 0;
-      state.ct.in_range = (const uint8_t *)nullptr;
-    }
-    if (status != TEAM_AGGREGATED) {
-      if (status != TEAM_CONVERGED && status != TEAM_NO_SHRINK && lead) atomicOr(&ctl->err, 2048ull);
-      break;
-    }
-    for (int64_t v = gt; v < N; v += nt) w.Ctop[v] = a0.CB[w.Ctop[v]];   // dendrogram lookup
-    cur = dst;
-    nv = h.nc;
-    nnz_cur = h.nnz2;
-    kmax = (int64_t)h.kmax;
-    tau /= o.tol_drop;
-    TEAM_SYNC_OR();   // the control words are read before the next pass clears them
+  if (threadIdx.x == 0) {
+    state.lp = 0;
+    state.cur = -1;
+    state.nv = N;
+    state.nnz = j.nnz;
+    state.kmax = (int64_t)__ldcg(&ctl->kmax);
+    state.tau = o.tol;
   }
+  __syncthreads();
+  if (N == 0 && lead) {   // an empty graph: one pass over nothing
+    res->passes = 1;
+    res->iters[0] = 1;
+    res->nv[0] = res->nnz[0] = res->moves[0] = res->refine_moves[0] = 0;
+  }
+  if (N > 0) small_next(j, o, t, ctl);
+  t.sync();
+  return N > 0;
+}
+
+// After a pass: its statistics, the dendrogram lookup and the next pass; false
+// when it was the last one.
+__device__ __noinline__ bool small_after(const SmallJob &j, const SmallOpts &o, SmallResult *res, Team t,
+                                         SmallCtl *ctl) {
+  SmallState &s = small_state();
+  const bool lead = t.rank == 0 && threadIdx.x == 0;
+  const volatile TeamCtl &h = ctl->t;
+  const int status = h.status, lp = s.lp;
+  if (lead && lp < LEIDEN_STATS_PASSES) {
+    if (lp == 0) res->changed0 = (int64_t)h.changed;
+    res->nnz[lp] = s.nnz;
+    res->passes = lp + 1;
+    res->iters[lp] = h.li;
+    res->nv[lp] = s.nv;
+    res->moves[lp] = h.moves;
+    res->refine_moves[lp] = (int64_t)h.rmoves;
+  }
+  if (status != TEAM_AGGREGATED) {
+    if (status != TEAM_CONVERGED && status != TEAM_NO_SHRINK && lead) atomicOr(&ctl->err, 2048ull);
+    return false;
+  }
+  for (int64_t v = t.index(); v < j.n; v += (int64_t)t.nb * TEAM_THREADS)
+    s.w.Ctop[v] = s.a.CB[s.w.Ctop[v]];
+  const int64_t nv = h.nc, nnz = h.nnz2, kmax = (int64_t)h.kmax;
+  t.sync();   // the control words are read before they are cleared
+  if (threadIdx.x == 0) {
+    s.cur = s.cur < 0 ? 0 : 1 - s.cur;
+    s.nv = nv;
+    s.nnz = nnz;
+    s.kmax = kmax;
+    s.tau /= o.tol_drop;
+    s.lp = lp + 1;
+    s.ct.dynamic = 0;
+    s.ct.in_range = (const uint8_t *)nullptr;
+  }
+  __syncthreads();
+  if (lp + 1 >= o.max_passes) return false;
+  small_next(j, o, t, ctl);
+  t.sync();
+  return true;
+}
+
+// The returned membership and the terms of its modularity.
+__device__ __noinline__ void small_finish(const SmallJob &j, SmallResult *res, Team t, SmallCtl *ctl) {
+  WideShared &sm = *reinterpret_cast<WideShared *>(small_dyn + kTables);
+  SmallState &state = small_state();
+  const WS &w = state.w;
+  const int64_t N = j.n, gt = t.index(), nt = (int64_t)t.nb * TEAM_THREADS, two_m = state.ct.two_m;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wg = warp * t.nb + t.rank, W = t.nb * TEAM_WARPS;
+  const bool lead = t.rank == 0 && threadIdx.x == 0;
   TEAM_SYNC_OR();
   // last lookup, then canonical labels: communities numbered by their
   // smallest member
@@ -515,7 +539,23 @@ __global__ void __launch_bounds__(TEAM_THREADS, 1) small_leiden_k(SmallHeader *h
       ctl = &ctls[blockIdx.x];
       continue;
     }
-    run_job(jobs[k], o, &results[jobs[k].result], t, ctl);
+    const SmallJob &j = jobs[k];
+    SmallResult *res = &results[j.result];
+    if (small_setup(j, o, res, t, ctl)) {
+      SmallState &s = small_state();
+      do {
+        if (s.narrow)
+          team_pass<true, int64_t, int64_t>(s.g, s.a, s.ct, s.lp, s.tau, o.max_iters, s.w.slots, t, small_dyn,
+                                            *reinterpret_cast<TeamShared<int64_t> *>(small_dyn + kTables));
+        else
+          team_pass<true, int64_t, i128>(s.g, s.a, s.ct, s.lp, s.tau, o.max_iters, s.w.slots, t, small_dyn,
+                                         *reinterpret_cast<TeamShared<i128> *>(small_dyn + kTables));
+        t.sync();
+      } while (small_after(j, o, res, t, ctl));
+      small_finish(j, res, t, ctl);
+    } else if (j.n == 0 && *(volatile u64 *)&ctl->err == 0) {
+      small_finish(j, res, t, ctl);
+    }
     t.sync();   // a job may end early, in every block alike; its words are done with
   }
 }
