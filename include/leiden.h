@@ -201,7 +201,8 @@ typedef struct {
   double t_agg_ms[LEIDEN_STATS_PASSES];
   double t_pass_ms[LEIDEN_STATS_PASSES];
   /* the same decide-kernel figures for the first pass alone (the first-pass
-   * local-moving phase; in a profiler it is the NVTX range local_move_pass0) */
+   * local-moving phase; in a profiler it is the NVTX range local_move_pass0,
+   * or resident_pass0 for the whole pass when it runs in one launch) */
   double move0_kernel_ms;
   int64_t move0_kernel_launches;
   double move0_bytes;

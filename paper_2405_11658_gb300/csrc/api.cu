@@ -108,20 +108,31 @@ namespace {
 
 constexpr int MAX_KEYS = 256 * MAX_TIERS;
 
-int dalloc(leiden_ctx *c, void **p, size_t bytes) {
-  if (bytes == 0) bytes = 16;
-  if (cudaMalloc(p, bytes) != cudaSuccess) {
+// The workspace is one device allocation: dal notes an array, alloc_all makes
+// the allocation and points the arrays into it.  About seventy allocations
+// took over a millisecond of every context's creation.
+struct Arena {
+  std::vector<std::pair<void **, size_t>> want;
+  size_t bytes = 0;
+};
+
+template <typename T>
+void dal(Arena &ar, T **p, int64_t count) {
+  ar.want.emplace_back(reinterpret_cast<void **>(p), ar.bytes);
+  const size_t b = (size_t)count * sizeof(T);
+  ar.bytes += ((b ? b : 16) + 255) & ~(size_t)255;
+}
+
+int alloc_all(leiden_ctx *c, const Arena &ar) {
+  char *base = nullptr;
+  if (cudaMalloc((void **)&base, ar.bytes) != cudaSuccess) {
     cudaGetLastError();
     return LEIDEN_ENOMEM;
   }
-  c->allocs.push_back(*p);
-  c->device_bytes += (int64_t)bytes;
+  c->allocs.push_back(base);
+  c->device_bytes += (int64_t)ar.bytes;
+  for (auto &w : ar.want) *w.first = base + w.second;
   return LEIDEN_OK;
-}
-
-template <typename T>
-int dal(leiden_ctx *c, T **p, int64_t count) {
-  return dalloc(c, reinterpret_cast<void **>(p), (size_t)count * sizeof(T));
 }
 
 void free_all(leiden_ctx *c) {
@@ -697,6 +708,7 @@ int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int
     }
   }
   int rc;
+  Phase ph(lp == 0 ? "resident_pass0" : "resident_pass");
   if (narrow) {
     rc = launch_team_pass<WT, int64_t>(ta, (int)nb, kind, c->st);
   } else {
@@ -1005,38 +1017,39 @@ int ctx_init(leiden_ctx *c, int64_t max_n, int64_t max_nnz) {
   const int64_t bh = bucket_blockhist_elems(max_n, MAX_KEYS);
   const int64_t scan_n = std::max<int64_t>(bh, 6 * n1 + 8);
   c->gcap = std::max<int64_t>(m, (int64_t)1 << 22);
-  int rc = LEIDEN_OK;
-  rc |= dal(c, &c->Ctop, n1); rc |= dal(c, &c->Cp, n1); rc |= dal(c, &c->CB, n1); rc |= dal(c, &c->rep, n1);
-  rc |= dal(c, &c->Kp, n1); rc |= dal(c, &c->Sp, n1); rc |= dal(c, &c->S2, n1); rc |= dal(c, &c->K0, n1);
-  rc |= dal(c, &c->Ktmp, n1);
-  rc |= dal(c, &c->ch, n1 + 16); rc |= dal(c, &c->ch2, n1 + 16); rc |= dal(c, &c->processed, n1 + 16);
-  rc |= dal(c, &c->affected, n1 + 16); rc |= dal(c, &c->stamp, n1 + 16); rc |= dal(c, &c->flag, n1 + 16);
-  rc |= dal(c, &c->prop_i, n1); rc |= dal(c, &c->prop_c, n1); rc |= dal(c, &c->prop_S, n1);
-  rc |= dal(c, &c->vlist, n1); rc |= dal(c, &c->clist, n1); rc |= dal(c, &c->cv, n1);
-  rc |= dal(c, &c->ccount, n1); rc |= dal(c, &c->coff, n1); rc |= dal(c, &c->ctdeg, n1);
-  rc |= dal(c, &c->hoff, n1); rc |= dal(c, &c->cdist, n1); rc |= dal(c, &c->ccur, n1);
-  rc |= dal(c, &c->off2tmp, 6 * n1 + 8);
-  rc |= dal(c, &c->scanned, scan_n + 1); rc |= dal(c, &c->koff_dev, MAX_KEYS + 1);
-  rc |= dal(c, &c->scan_tmp, scan_tmp_elems(scan_n) + 1);
-  rc |= dal(c, &c->blockhist, bh);
+  Arena ar;
+  dal(ar, &c->Ctop, n1); dal(ar, &c->Cp, n1); dal(ar, &c->CB, n1); dal(ar, &c->rep, n1);
+  dal(ar, &c->Kp, n1); dal(ar, &c->Sp, n1); dal(ar, &c->S2, n1); dal(ar, &c->K0, n1);
+  dal(ar, &c->Ktmp, n1);
+  dal(ar, &c->ch, n1 + 16); dal(ar, &c->ch2, n1 + 16); dal(ar, &c->processed, n1 + 16);
+  dal(ar, &c->affected, n1 + 16); dal(ar, &c->stamp, n1 + 16); dal(ar, &c->flag, n1 + 16);
+  dal(ar, &c->prop_i, n1); dal(ar, &c->prop_c, n1); dal(ar, &c->prop_S, n1);
+  dal(ar, &c->vlist, n1); dal(ar, &c->clist, n1); dal(ar, &c->cv, n1);
+  dal(ar, &c->ccount, n1); dal(ar, &c->coff, n1); dal(ar, &c->ctdeg, n1);
+  dal(ar, &c->hoff, n1); dal(ar, &c->cdist, n1); dal(ar, &c->ccur, n1);
+  dal(ar, &c->off2tmp, 6 * n1 + 8);
+  dal(ar, &c->scanned, scan_n + 1); dal(ar, &c->koff_dev, MAX_KEYS + 1);
+  dal(ar, &c->scan_tmp, scan_tmp_elems(scan_n) + 1);
+  dal(ar, &c->blockhist, bh);
   for (int k = 0; k < 2; k++) {
-    rc |= dal(c, &c->goff[k], n1); rc |= dal(c, &c->gidx[k], m); rc |= dal(c, &c->gw[k], m);
+    dal(ar, &c->goff[k], n1); dal(ar, &c->gidx[k], m); dal(ar, &c->gw[k], m);
   }
-  rc |= dal(c, &c->hidx, m); rc |= dal(c, &c->hw, m);
-  rc |= dal(c, &c->gkeys, c->gcap); rc |= dal(c, &c->gvals, c->gcap);
-  rc |= dal(c, &c->ctr, CTR_COUNT);
-  rc |= dal(c, &c->tctl, 1);
-  rc |= dal(c, &c->big, n1);
+  dal(ar, &c->hidx, m); dal(ar, &c->hw, m);
+  dal(ar, &c->gkeys, c->gcap); dal(ar, &c->gvals, c->gcap);
+  dal(ar, &c->ctr, CTR_COUNT);
+  dal(ar, &c->tctl, 1);
+  dal(ar, &c->big, n1);
   // giant-community buckets: a community of total degree T > 2048 gets at most
   // 2 * ceil(T / 2048) <= T / 512 buckets, so the total stays below nnz / 512
   c->bcap = m / 256 + n1 + 16;
-  rc |= dal(c, &c->bcnt, c->bcap); rc |= dal(c, &c->bpos, c->bcap);
-  rc |= dal(c, &c->hub.tsz, n1); rc |= dal(c, &c->hub.toff, n1);
-  rc |= dal(c, &c->hub.ioff, n1); rc |= dal(c, &c->hub.soff, n1);
-  rc |= dal(c, &c->hub.tot, 4);
+  dal(ar, &c->bcnt, c->bcap); dal(ar, &c->bpos, c->bcap);
+  dal(ar, &c->hub.tsz, n1); dal(ar, &c->hub.toff, n1);
+  dal(ar, &c->hub.ioff, n1); dal(ar, &c->hub.soff, n1);
+  dal(ar, &c->hub.tot, 4);
   c->hub_items = c->gcap / 4096 + 1024;
-  rc |= dal(c, &c->hub.psc, c->hub_items); rc |= dal(c, &c->hub.pc, c->hub_items);
-  rc |= dal(c, &c->hub.pkid, c->hub_items);
+  dal(ar, &c->hub.psc, c->hub_items); dal(ar, &c->hub.pc, c->hub_items);
+  dal(ar, &c->hub.pkid, c->hub_items);
+  int rc = alloc_all(c, ar);
   if (rc == LEIDEN_OK) {
     if (cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess) rc = LEIDEN_ENOMEM;
     for (int k = 0; k < leiden_ctx::NAUX && rc == LEIDEN_OK; k++) {
