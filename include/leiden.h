@@ -183,8 +183,11 @@ typedef struct {
   int64_t refine_moves[LEIDEN_STATS_PASSES];
   int64_t affected0;                            /* vertices unprocessed at the start */
   int64_t changed0;                             /* communities flagged changed before the first refinement */
-  /* device time of the local-move decide kernels, measured with CUDA events on
-   * the context stream when timing is enabled (leiden_ctx_set_timing) */
+  /* device time of the local-move decide phases when timing is enabled
+   * (leiden_ctx_set_timing), and their number, one per colour class and
+   * iteration: CUDA events around their kernels on the context stream or, for
+   * a pass that runs in one launch, the clock of its first block from the
+   * start of a phase to the barrier that ends it */
   double move_kernel_ms;
   int64_t move_kernel_launches;
   int64_t move_scanned_entries;                 /* CSR entries the decide kernels read */
@@ -194,8 +197,9 @@ typedef struct {
   /* time per pass: local-moving phase (with the vertex buckets), refinement
    * (with subset renumbering and the break), aggregation (with renumbering and
    * the dendrogram lookup), and the whole pass; host wall time, but for a pass
-   * that runs in one launch the phases are on the device clock (aggregation 0
-   * when it follows in launches of its own) */
+   * that runs in one launch the phases are on the device clock (the lookup,
+   * enqueued after it, is in neither; an aggregation in launches of its own
+   * adds its wall time) */
   double t_move_ms[LEIDEN_STATS_PASSES];
   double t_refine_ms[LEIDEN_STATS_PASSES];
   double t_agg_ms[LEIDEN_STATS_PASSES];
@@ -215,7 +219,7 @@ typedef struct {
 /* Copies the statistics of the last run into *out (HOST). */
 int leiden_get_stats(leiden_ctx *ctx, leiden_run_stats *out);
 
-/* Enables (1) or disables (0) CUDA-event timing of the local-move kernels. */
+/* Enables (1) or disables (0) timing of the local-move decide phases. */
 int leiden_ctx_set_timing(leiden_ctx *ctx, int32_t enable);
 
 /* Allocation-free modularity.  The paper has no counterpart: this entry point

@@ -751,7 +751,10 @@ int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int
     c->stats.refine_moves[lp] = (int64_t)h.rmoves;
     c->stats.t_move_ms[lp] = (double)(h.stamp[1] - h.stamp[0]) * 1e-6;
     c->stats.t_refine_ms[lp] = (double)(h.stamp[2] - h.stamp[1]) * 1e-6;
-    if (h.status == TEAM_AGGREGATED) c->stats.t_agg_ms[lp] = (double)(h.stamp[3] - h.stamp[2]) * 1e-6;
+    // renumbering, with the aggregation when the pass includes it; run_leiden
+    // adds one that follows in launches of its own
+    if (h.status == TEAM_AGGREGATED || h.status == TEAM_RENUMBERED)
+      c->stats.t_agg_ms[lp] = (double)(h.stamp[3] - h.stamp[2]) * 1e-6;
     c->stats.t_pass_ms[lp] = ms_since(t_start);
   }
   if (h.status == TEAM_CONVERGED) return 1;
@@ -802,8 +805,14 @@ int run_leiden(Run &r, const leiden_csr *g0) {
         lev.maxdeg = next.maxdeg;
         lev.kmax = next.kmax;
       } else if (rc == 2) {
+        const auto t_agg = std::chrono::steady_clock::now();
         rc = cur < 0 ? aggregate_level<int32_t>(r, g32, dst, nc, &nnz2)
                      : aggregate_level<int64_t>(r, g64, dst, nc, &nnz2);
+        if (lp < LEIDEN_STATS_PASSES) {
+          const double ms = ms_since(t_agg);
+          c->stats.t_agg_ms[lp] += ms;
+          c->stats.t_pass_ms[lp] += ms;
+        }
       }
     }
     if (rc == 3) {

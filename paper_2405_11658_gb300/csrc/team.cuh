@@ -1559,6 +1559,7 @@ __device__ __forceinline__ void team_pass(const GL &g, AR &a, const CT &ct, int 
     if (agg && i < nc) { a.cnt[i] = 0; a.K2[i] = 0; }
   }
   if (!agg) {
+    stamp_time(3);
     if (t.rank == 0 && threadIdx.x == 0) ctl->status = nc == n ? TEAM_NO_SHRINK : TEAM_RENUMBERED;
     return;
   }

@@ -34,7 +34,7 @@ struct TeamCtl {
   int64_t nc, nnz2;
   u64 maxdeg, kmax;        // of the aggregated level
   u64 decide_ns, subsweeps;
-  u64 stamp[4];            // globaltimer at the start and after local-moving, refinement, aggregation
+  u64 stamp[4];            // globaltimer at the start and after local-moving, refinement, aggregation (or renumbering)
   // end of the part the host reads back
   int64_t part[TEAM_MAX_BLOCKS];
   unsigned ktot[256 * 8], kcur[256 * 8];
