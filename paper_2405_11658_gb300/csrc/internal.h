@@ -231,8 +231,13 @@ void launch_buckets(const int64_t *off, int64_t n, int log2S, const TierTable &t
                     int64_t *scan_tmp, cudaStream_t s);
 int64_t bucket_blockhist_elems(int64_t n, int nkeys);
 
-// scan.cu
+// scan.cu.  Function attributes and occupancy belong to the current device, so
+// what has been set or asked is remembered per device.
+int current_device();
+// Lets `func` have `bytes` of dynamic shared memory.
 void ensure_smem(const void *func, size_t bytes);
+// Lets `func` be launched in clusters of more than 8 blocks.
+void ensure_wide_clusters(const void *func);
 // Blocks of `func` (threads, dynamic shared memory) resident at once on `sms`
 // SMs: the grid of a grid-stride kernel that leaves no partial last wave.
 int64_t resident_blocks(const void *func, int threads, size_t smem, int sms);

@@ -4,46 +4,67 @@
 // Used for the exclusive scans of the aggregation phase (Alg. leidenag:
 // community-vertex offsets and super-vertex offsets), the dense renumbering of
 // communities, the canonical relabelling and the batch application.
+#include <map>
 #include <mutex>
+#include <set>
 #include <unordered_map>
+#include <utility>
 
 #include "common.cuh"
 #include "internal.h"
 
 namespace lk {
 
+int current_device() {
+  int d = 0;
+  if (cudaGetDevice(&d) != cudaSuccess) (void)cudaGetLastError();
+  return d;
+}
+
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` (once per
-// kernel and size; the attribute outlives the call, so it is set only when
-// the requested size grows).
+// device, kernel and size; the attribute outlives the call, so it is set only
+// when the requested size grows).
 void ensure_smem(const void *func, size_t bytes) {
   if (bytes <= 32 * 1024) return;  // leaves room for static shared memory
   static std::mutex mu;
-  static std::unordered_map<const void *, size_t> done;
+  static std::map<std::pair<int, const void *>, size_t> done;
+  const int dev = current_device();
   std::lock_guard<std::mutex> lock(mu);
-  size_t &have = done[func];
+  size_t &have = done[{dev, func}];
   if (have >= bytes) return;
   if (cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess)
     have = bytes;
 }
 
+void ensure_wide_clusters(const void *func) {
+  static std::mutex mu;
+  static std::set<std::pair<int, const void *>> done;
+  const int dev = current_device();
+  std::lock_guard<std::mutex> lock(mu);
+  if (done.count({dev, func})) return;
+  if (cudaFuncSetAttribute(func, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+    done.insert({dev, func});
+}
+
 int64_t resident_blocks(const void *func, int threads, size_t smem, int sms) {
   struct Key {
     const void *f;
-    int t;
+    int d, t;
     size_t m;
-    bool operator==(const Key &o) const { return f == o.f && t == o.t && m == o.m; }
+    bool operator==(const Key &o) const { return f == o.f && d == o.d && t == o.t && m == o.m; }
   };
   struct Hash {
     size_t operator()(const Key &k) const {
-      return std::hash<const void *>()(k.f) ^ ((size_t)k.t << 20) ^ (k.m << 1);
+      return std::hash<const void *>()(k.f) ^ ((size_t)k.d << 40) ^ ((size_t)k.t << 20) ^ (k.m << 1);
     }
   };
   static std::mutex mu;
   static std::unordered_map<Key, int, Hash> per_sm;
   int nb = 0;
+  const Key key{func, current_device(), threads, smem};
   {
     std::lock_guard<std::mutex> lock(mu);
-    auto it = per_sm.find(Key{func, threads, smem});
+    auto it = per_sm.find(key);
     if (it != per_sm.end()) {
       nb = it->second;
     } else {
@@ -52,7 +73,7 @@ int64_t resident_blocks(const void *func, int threads, size_t smem, int sms) {
         nb = 0;
       }
       if (nb < 1) nb = 1;
-      per_sm[Key{func, threads, smem}] = nb;
+      per_sm[key] = nb;
     }
   }
   return (int64_t)nb * sms;

@@ -18,8 +18,6 @@
 // throughout, 14 ms as here.
 #include <limits.h>
 
-#include <mutex>
-
 #include "common.cuh"
 #include "internal.h"
 #include "small.h"
@@ -565,8 +563,7 @@ int launch_small(SmallHeader *hdr, const SmallJob *jobs, const SmallOpts &o, Sma
   auto k = small_leiden_k;
   const size_t smem = kSmem;
   ensure_smem((const void *)k, smem);
-  static std::once_flag once;
-  std::call_once(once, [&] { cudaFuncSetAttribute((const void *)k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); });
+  ensure_wide_clusters((const void *)k);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(blocks / cluster * cluster), 1, 1);
   cfg.blockDim = dim3(TEAM_THREADS, 1, 1);

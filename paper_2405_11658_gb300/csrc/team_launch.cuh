@@ -3,6 +3,8 @@
 // (team_*.cu), because one kernel takes the compiler a good twenty seconds.
 #pragma once
 
+#include <array>
+#include <map>
 #include <mutex>
 
 #include "team.cuh"
@@ -42,17 +44,20 @@ static size_t team_smem() {
   return (size_t)TEAM_WARPS * TEAM_WSLOTS * (sizeof(typename TableVal<ST>::type) + sizeof(int32_t));
 }
 
-// Whether a cluster of nb team blocks can be resident (asked once per size).
+// Whether a cluster of nb team blocks can be resident on the current device
+// (asked once per device and size).
 template <typename WT, typename ST>
 bool team_cluster_fits(int nb) {
   static std::mutex mu;
-  static int known[TEAM_MAX_CLUSTER + 1] = {};   // 0: not asked, 1: yes, 2: no
+  static std::map<int, std::array<int, TEAM_MAX_CLUSTER + 1>> known;   // by device; 0: not asked, 1: yes, 2: no
   if (nb < 2 || nb > TEAM_MAX_CLUSTER) return false;
+  const int dev = current_device();
   std::lock_guard<std::mutex> lock(mu);
-  if (known[nb]) return known[nb] == 1;
+  int &fits = known[dev][nb];
+  if (fits) return fits == 1;
   auto k = team_pass_k<WT, ST>;
   ensure_smem((const void *)k, team_smem<WT, ST>());
-  cudaFuncSetAttribute((const void *)k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  ensure_wide_clusters((const void *)k);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)nb, 1, 1);
   cfg.blockDim = dim3(TEAM_THREADS, 1, 1);
@@ -67,7 +72,7 @@ bool team_cluster_fits(int nb) {
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, (const void *)k, &cfg) != cudaSuccess) n = 0;
   (void)cudaGetLastError();
-  known[nb] = n > 0 ? 1 : 2;
+  fits = n > 0 ? 1 : 2;
   return n > 0;
 }
 

@@ -1,0 +1,94 @@
+"""What the host side launches, and what it does when a launch is refused, on a
+runtime without a device (tests/fake_cudart.cpp): kernels do nothing there, so
+a run ends early with an error; the log of its launches is what is checked."""
+from __future__ import annotations
+
+import ctypes as C
+import re
+import sys
+
+import numpy as np
+import pytest
+
+sys.path.insert(0, __file__.rsplit("/", 1)[0])
+import host_library  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    L, lib = host_library.load(tmp_path_factory.mktemp("host"))
+    return Host(L, lib)
+
+
+class Host:
+    def __init__(self, L, lib):
+        self.L, self.lib = L, lib
+
+    def reset(self, device=0, sms=152):
+        self.lib.fake_reset()
+        self.lib.fake_set_device(device)
+        self.lib.fake_set_sms(sms)
+
+    def log(self):
+        """The launches so far: (device, kernel, grid, block, cluster, cooperative, refused)."""
+        out = []
+        for ln in self.lib.fake_log().decode().splitlines():
+            m = re.match(r"(\d+) (\S+) grid (\d+) block (\d+) smem \d+ cluster (\d+)( coop)? (ok|refused)", ln)
+            out.append((int(m[1]), m[2], int(m[3]), int(m[4]), int(m[5]), bool(m[6]), m[7] == "refused"))
+        return out
+
+    def csr(self, n, nnz):
+        """A graph by its sizes alone: nothing reads its entries."""
+        self.off = np.zeros(n + 1, np.int64)
+        self.dummy = np.zeros(4, np.int32)
+        return self.L._Csr(n, nnz, self.off.ctypes.data, self.dummy.ctypes.data, self.dummy.ctypes.data)
+
+    def opts(self):
+        o = self.L._Opts()
+        self.lib.leiden_opts_default(C.byref(o))
+        return o
+
+    def static(self, n, nnz, tiers=None):
+        ctx = C.c_void_p()
+        assert self.lib.leiden_ctx_create(C.byref(ctx), None, C.c_int64(n), C.c_int64(nnz)) == 0
+        out = np.zeros(max(n, 1), np.int32)
+        g, o = self.csr(n, nnz), self.opts()
+        rc = self.lib.leiden_static(ctx, C.byref(g), C.byref(o), C.c_void_p(out.ctypes.data), None)
+        self.lib.leiden_ctx_destroy(ctx)
+        return rc
+
+    def batch(self, sizes):
+        """sizes: (n, nnz) of each graph."""
+        b = C.c_void_p()
+        assert self.lib.leiden_batch_create(C.byref(b), None, len(sizes), C.c_int64(sum(s[0] for s in sizes)),
+                                            C.c_int64(sum(s[1] for s in sizes)), 0, 0) == 0
+        items = (self.L._BatchItem * len(sizes))()
+        res = (self.L._BatchResult * len(sizes))()
+        keep = []
+        for it, (n, nnz) in zip(items, sizes):
+            it.g = self.csr(n, nnz)
+            out = np.zeros(n, np.int32)
+            keep.append((self.off, self.dummy, out))
+            it.out = out.ctypes.data
+        o = self.opts()
+        rc = self.lib.leiden_batch_run(b, len(sizes), items, C.byref(o), res)
+        self.lib.leiden_batch_destroy(b)
+        return rc
+
+
+def test_a_second_device_gets_its_own_attributes(host):
+    # the first device's calls must not stand in for the second's: a kernel
+    # whose shared-memory limit or cluster attribute is unset there is refused
+    for device in (0, 1):
+        host.reset(device)
+        host.static(2000, 18000)       # one cluster of 16 blocks
+        host.static(20000, 4000000)    # a cooperative grid
+        host.batch([(20000, 400000)] * 4)   # clusters of 16
+        log = host.log()
+        assert {d for d, *_ in log} == {device}
+        team = [x for x in log if "team_pass_k" in x[1]]
+        assert [(x[4], x[5]) for x in team] == [(16, False), (1, True)], team
+        assert [x[4] for x in log if "small_leiden_k" in x[1]] == [16]
+        assert not [x for x in log if x[6]]
+        rows = [x for x in log if "rows_k" in x[1] and "check" not in x[1]][-1]
+        assert rows[2] == 152 * ((2048 // rows[3]) >> device)   # its own occupancy
