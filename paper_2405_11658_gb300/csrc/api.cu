@@ -655,7 +655,8 @@ constexpr int64_t TEAM_BLOCK_SIZE = 2048;
 constexpr int64_t TEAM_AGG_NNZ = 5500000;
 
 // One pass on the team path; returns as pass() does, or 2 when the caller has
-// to aggregate, or 3 when the level's hubs exceed the scratch (nothing done).
+// to aggregate, or 3 when the level's hubs exceed the scratch or the blocks
+// cannot be resident together (nothing done).
 template <typename WT>
 int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int dst, const Buckets &b,
                    int64_t *nc_out, Buckets &next, int64_t *nnz_out) {
@@ -707,15 +708,11 @@ int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int
       kind = TEAM_CLUSTER;
     }
   }
-  int rc;
   Phase ph(lp == 0 ? "resident_pass0" : "resident_pass");
-  if (narrow) {
-    rc = launch_team_pass<WT, int64_t>(ta, (int)nb, kind, c->st);
-  } else {
-    rc = launch_team_pass<WT, i128>(ta, (int)nb, kind, c->st);
-    if (lp < LEIDEN_STATS_PASSES) c->stats.wide_passes |= 1u << lp;
-  }
-  if (rc) { check_cuda(c); return rc; }
+  int rc = narrow ? launch_team_pass<WT, int64_t>(ta, (int)nb, kind, c->st)
+                  : launch_team_pass<WT, i128>(ta, (int)nb, kind, c->st);
+  if (rc) return 3;
+  if (!narrow && lp < LEIDEN_STATS_PASSES) c->stats.wide_passes |= 1u << lp;
   cudaMemcpyAsync(c->h_tctl, c->tctl, TEAM_CTL_HEAD, cudaMemcpyDeviceToHost, c->st);
   cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   rc = sync(c);

@@ -17,7 +17,7 @@ using namespace lk;
 struct leiden_batch {
   cudaStream_t st = nullptr;     // the caller's stream: every run is ordered on it
   cudaStream_t cap = nullptr;    // private stream the CUDA graph is captured on
-  int device = 0, sms = 152;
+  int device = 0, sms = 152, max_cluster = 1;
   int32_t max_graphs = 0;
   int64_t max_n = 0, max_nnz = 0;
   char *arena = nullptr;
@@ -129,11 +129,13 @@ int capture(leiden_batch *b, const SmallOpts &so, int k) {
 // graphs of 1e3 vertices (1.1e4) a batch took 15% longer than with one 512-
 // thread block each.  64 graphs of 1e3..1e4 vertices (1.1e4 .. 1.1e5): single
 // blocks 28.4 ms, clusters of 2 for all 19.7, of 4 for the 20 largest 18.3, of
-// 4 for all 20.0, of 8 for the 20 largest 26.9.
-int cluster_log2(int count, int sms, const std::vector<int64_t> &sizes, int32_t *wide) {
+// 4 for all 20.0, of 8 for the 20 largest 26.9.  Clusters have at most `most`
+// blocks, what the device can keep resident.
+int cluster_log2(int count, int sms, int most, const std::vector<int64_t> &sizes, int32_t *wide) {
   *wide = 0;
   for (int k = 4; k > 0; k--) {
     const int c = 1 << k;
+    if (c > most) continue;
     const int w = std::min(count, std::max(0, (sms - count) / (c - 1)));
     if (3 * w < count || sizes[0] < (int64_t)6144 * c) continue;
     while (*wide < w && sizes[*wide] >= (int64_t)3072 * c) ++*wide;
@@ -163,6 +165,7 @@ extern "C" int leiden_batch_create(leiden_batch **out, void *stream, int32_t max
       cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess) {
     rc = LEIDEN_ECUDA;
   }
+  if (!rc) b->max_cluster = small_max_cluster();
   b->arena_bytes = small_layout_bound(max_total_n, max_total_nnz, max_graphs);
   b->desc_bytes = sizeof(SmallHeader) + (size_t)max_graphs * sizeof(SmallJob);
   b->res_bytes = (size_t)max_graphs * sizeof(SmallResult);
@@ -229,7 +232,7 @@ extern "C" int leiden_batch_run(leiden_batch *b, int32_t count, const leiden_bat
   hdr->count = count;
   std::vector<int64_t> sizes(count);
   for (int k = 0; k < count; k++) sizes[k] = items[order[k]].g.nnz + items[order[k]].g.n;
-  const int lc = cluster_log2(count, b->sms, sizes, &hdr->wide);
+  const int lc = cluster_log2(count, b->sms, b->max_cluster, sizes, &hdr->wide);
   hdr->next = 0;
   hdr->next1 = (uint32_t)hdr->wide;
   int64_t at = 0;

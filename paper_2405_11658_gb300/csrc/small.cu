@@ -558,25 +558,41 @@ __global__ void __launch_bounds__(TEAM_THREADS, 1) small_leiden_k(SmallHeader *h
   }
 }
 
+// The launch of `blocks` blocks in clusters of `cluster`.
+static void small_config(int blocks, int cluster, cudaStream_t s, cudaLaunchAttribute *attr, cudaLaunchConfig_t *cfg) {
+  ensure_smem((const void *)small_leiden_k, kSmem);
+  ensure_wide_clusters((const void *)small_leiden_k);
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3((unsigned)(blocks / cluster * cluster), 1, 1);
+  cfg->blockDim = dim3(TEAM_THREADS, 1, 1);
+  cfg->dynamicSmemBytes = kSmem;
+  cfg->stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)cluster;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+}
+
+int small_max_cluster() {
+  for (int c = 16; c > 1; c >>= 1) {
+    cudaLaunchAttribute attr{};
+    cudaLaunchConfig_t cfg;
+    small_config(c, c, nullptr, &attr, &cfg);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, (const void *)small_leiden_k, &cfg) == cudaSuccess && n > 0) return c;
+    (void)cudaGetLastError();
+  }
+  return 1;
+}
+
 int launch_small(SmallHeader *hdr, const SmallJob *jobs, const SmallOpts &o, SmallResult *results, SmallCtl *ctl,
                  int blocks, int cluster, cudaStream_t s) {
-  auto k = small_leiden_k;
-  const size_t smem = kSmem;
-  ensure_smem((const void *)k, smem);
-  ensure_wide_clusters((const void *)k);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(blocks / cluster * cluster), 1, 1);
-  cfg.blockDim = dim3(TEAM_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
   cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)cluster;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, k, hdr, jobs, o, results, ctl) != cudaSuccess) return LEIDEN_ECUDA;
+  cudaLaunchConfig_t cfg;
+  small_config(blocks, cluster, s, &attr, &cfg);
+  if (cudaLaunchKernelEx(&cfg, small_leiden_k, hdr, jobs, o, results, ctl) != cudaSuccess) return LEIDEN_ECUDA;
   return LEIDEN_OK;
 }
 

@@ -112,10 +112,11 @@ __host__ __device__ inline int64_t small_layout_bound(int64_t n, int64_t nnz, in
   return n * 97 + nnz * 61 + graphs * (34 * 256 + 8192);
 }
 
-// Threads of a block, blocks of a cluster at most.
-static constexpr int SMALL_MAX_CLUSTER = 16;
 struct SmallCtl;
 size_t small_ctl_bytes(int blocks);
+// Blocks of the largest cluster (1, 2, 4, 8 or 16) that can be resident on the
+// current device.
+int small_max_cluster();
 // Enqueues the kernel: `blocks` blocks in clusters of `cluster`; jobs before
 // hdr->wide are run by whole clusters, the others by single blocks.
 int launch_small(SmallHeader *hdr, const SmallJob *jobs, const SmallOpts &o, SmallResult *results, SmallCtl *ctl,

@@ -84,7 +84,8 @@ struct TeamArgs {
   const uint8_t *in_range;
   TeamCtl *ctl;
 };
-// Launches the pass over nb blocks (one per SM at most) as `kind`.
+// Launches the pass over nb blocks (one per SM at most) as `kind`; an error
+// when the runtime refuses the launch (nothing is enqueued then).
 static constexpr int TEAM_MAX_CLUSTER = 16;
 template <typename WT, typename ST>
 bool team_cluster_fits(int nb);

@@ -98,8 +98,11 @@ int launch_team_pass(const TeamArgs<WT> &args, int nb, int kind, cudaStream_t s)
   }
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, k, args, kind) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return LEIDEN_ECUDA;
+  }
   note_launch();
-  if (cudaLaunchKernelEx(&cfg, k, args, kind) != cudaSuccess) return LEIDEN_ECUDA;
   return LEIDEN_OK;
 }
 

@@ -92,3 +92,26 @@ def test_a_second_device_gets_its_own_attributes(host):
         assert not [x for x in log if x[6]]
         rows = [x for x in log if "rows_k" in x[1] and "check" not in x[1]][-1]
         assert rows[2] == 152 * ((2048 // rows[3]) >> device)   # its own occupancy
+
+
+@pytest.mark.parametrize("n,nnz,coop,cluster", [(2000, 18000, 0, 1), (20000, 4000000, 1, 0)])
+def test_a_refused_resident_launch_runs_the_multi_kernel_path(host, n, nnz, coop, cluster):
+    host.reset()
+    host.lib.fake_refuse(coop, cluster)
+    host.static(n, nnz)
+    kernels = [x[1] for x in host.log()]
+    team = [k for k, name in enumerate(kernels) if "team_pass_k" in name]
+    assert team and host.log()[team[0]][6]
+    # the class lists of the multi-kernel path are its first launch
+    assert any("bucket_count_k" in name for name in kernels[team[0] + 1:])
+    assert host.lib.fake_pending_error() == 0
+
+
+@pytest.mark.parametrize("most", [16, 8, 4, 2, 1])
+def test_batch_clusters_fit_the_device(host, most):
+    host.reset()
+    host.lib.fake_set_max_cluster(most)
+    assert host.batch([(20000, 400000)] * 4) == 0
+    small = [x for x in host.log() if "small_leiden_k" in x[1]]
+    assert [x[4] for x in small] == [most] and not small[0][6]
+    assert host.lib.fake_pending_error() == 0
