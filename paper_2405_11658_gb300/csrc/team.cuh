@@ -678,9 +678,8 @@ __device__ __forceinline__ void team_hub_add(const AR &a, int64_t at, uint64_t t
   atomicOr(a.err, 16ull);
 }
 
-// Prefix sums of every class's hub items; false when a class has more hubs
-// than the bitmap holds or its tables exceed the scratch (the same answer in
-// every block).
+// Prefix sums of every class's hub items; false when a class's tables exceed
+// the scratch (the same answer in every block).
 template <typename WT, typename ST, typename GL, typename AR>
 __device__ __forceinline__ bool team_hub_setup(const GL &g, const AR &a, int S, Team &t,
                                                TeamShared<ST> &sm) {
@@ -719,14 +718,23 @@ __device__ __forceinline__ bool team_hub_setup(const GL &g, const AR &a, int S, 
         a.hub_done[p - h0] = 0;
       }
     }
-    if (threadIdx.x == 0 && (p1 - p0 > TEAM_MAX_HUBS || cs * HUB_SLOTS > a.tcap || ci > INT_MAX / 2))
+    if (threadIdx.x == 0 && (cs * HUB_SLOTS > a.tcap || ci > INT_MAX / 2))
       t.ctl->too_big = 1;
   }
   if (!t.sync()) return false;
   return *(volatile int32_t *)&t.ctl->too_big == 0;
 }
 
-// Which hubs of the class are to be decided, into sm.hbits; whether any is.
+// Whether hub i is to be decided in this sub-sweep.  Its flags change only once
+// all its items are done (processed) or after the sub-sweep's barrier.
+template <bool REFINE, typename AR, typename CT>
+__device__ __forceinline__ bool team_hub_active(const AR &a, const CT &ct, int32_t i) {
+  return REFINE ? (a.ch[a.CB[i]] && a.C[i] == i && a.Sig[i] == a.K[i])
+                : (!a.processed[i] && (!ct.in_range || ct.in_range[i]));
+}
+
+// Which hubs of the class are to be decided, the first TEAM_MAX_HUBS of them
+// into sm.hbits; whether any is.
 template <bool REFINE, typename ST, typename AR, typename CT>
 __device__ __forceinline__ bool team_hub_bits(const AR &a, const CT &ct, const int32_t *list, int m,
                                               TeamShared<ST> &sm) {
@@ -734,20 +742,23 @@ __device__ __forceinline__ bool team_hub_bits(const AR &a, const CT &ct, const i
   for (int base = 0; base < m; base += TEAM_THREADS) {
     const int k = base + (int)threadIdx.x;
     bool act = false;
-    if (k < m) {
-      const int32_t i = list[k];
-      act = REFINE ? (a.ch[a.CB[i]] && a.C[i] == i && a.Sig[i] == a.K[i])
-                   : (!a.processed[i] && (!ct.in_range || ct.in_range[i]));
-    }
+    if (k < m) act = team_hub_active<REFINE>(a, ct, list[k]);
     const unsigned mk = __ballot_sync(FULL_MASK, act);
-    if ((threadIdx.x & 31) == 0 && base + (int)threadIdx.x < m) sm.hbits[(base + (int)threadIdx.x) >> 5] = mk;
+    if ((threadIdx.x & 31) == 0 && k < m && k < TEAM_MAX_HUBS) sm.hbits[(base + (int)threadIdx.x) >> 5] = mk;
     any |= mk != 0;
   }
   return __syncthreads_or(any) != 0;
 }
 
-template <bool REFINE, typename WT, typename ST, typename GL, typename AR>
-__device__ __forceinline__ void team_hub_insert(const GL &g, const AR &a, const Team &t,
+// team_hub_active of the class's k-th hub, from the bits.
+template <bool REFINE, typename ST, typename AR, typename CT>
+__device__ __forceinline__ bool team_hub_bit(const AR &a, const CT &ct, const int32_t *list, int k,
+                                             const TeamShared<ST> &sm) {
+  return k < TEAM_MAX_HUBS ? (sm.hbits[k >> 5] >> (k & 31)) & 1u : team_hub_active<REFINE>(a, ct, list[k]);
+}
+
+template <bool REFINE, typename WT, typename ST, typename GL, typename AR, typename CT>
+__device__ __forceinline__ void team_hub_insert(const GL &g, const AR &a, const CT &ct, const Team &t,
                                                 const int32_t *list, const int32_t *pi, const int32_t *ps, int m,
                                                 int32_t *keys, typename TableVal<ST>::type *vals,
                                                 TeamShared<ST> &sm) {
@@ -756,7 +767,7 @@ __device__ __forceinline__ void team_hub_insert(const GL &g, const AR &a, const 
   const int total = pi[m - 1];
   for (int w = sub * t.nb + t.rank; w < total; w += t.nb * TEAM_NSUB) {
     const int k = team_find(pi, m, w);
-    if (!((sm.hbits[k >> 5] >> (k & 31)) & 1u)) continue;
+    if (!team_hub_bit<REFINE>(a, ct, list, k, sm)) continue;
     const int32_t i = list[k];
     const int64_t e0 = g.off[i], e1 = g.off[i + 1];
     const int64_t c0 = e0 + (int64_t)(w - (k ? pi[k - 1] : 0)) * HUB_ITEM;
@@ -791,7 +802,7 @@ __device__ __forceinline__ void team_hub_scan(const GL &g, const AR &a, const CT
   const int total = ps[m - 1];
   for (int w = sub * t.nb + t.rank; w < total; w += t.nb * TEAM_NSUB) {
     const int k = team_find(ps, m, w);
-    if (!((sm.hbits[k >> 5] >> (k & 31)) & 1u)) continue;
+    if (!team_hub_bit<REFINE>(a, ct, list, k, sm)) continue;
     const int32_t i = list[k];
     const int32_t d = a.C[i];
     const int64_t Ki = a.K[i];
@@ -920,7 +931,7 @@ __device__ __forceinline__ bool team_decide_class(const GL &g, const AR &a, cons
   if (m7 > 0) {
     hubs = team_hub_bits<REFINE, ST>(a, ct, a.vlist + ko[7 * S], m7, sm);
     if (hubs)
-      team_hub_insert<REFINE, WT, ST>(g, a, t, a.vlist + ko[7 * S], a.hub_i + hub0, a.hub_s + hub0, m7, keys +
+      team_hub_insert<REFINE, WT, ST>(g, a, ct, t, a.vlist + ko[7 * S], a.hub_i + hub0, a.hub_s + hub0, m7, keys +
                                       threadIdx.x / TEAM_SUB * (TEAM_WSLOTS * (TEAM_SUB / 32)), vals +
                                       threadIdx.x / TEAM_SUB * (TEAM_WSLOTS * (TEAM_SUB / 32)), sm);
     if (ko[6 * S + 1] > ko[6 * S]) __syncthreads();   // the block tier pools the sub-blocks' tables

@@ -16,7 +16,8 @@ enum { TEAM_BLOCK = 0, TEAM_CLUSTER = 1, TEAM_GRID = 2 };
 enum { TEAM_NONE = 0, TEAM_CONVERGED = 1, TEAM_NO_SHRINK = 2, TEAM_RENUMBERED = 3, TEAM_AGGREGATED = 4, TEAM_TOO_BIG = 5 };
 
 // Distinct candidates of a vertex the block's table takes (half its slots);
-// vertices with more are hubs.  Hubs per colour class at most.
+// vertices with more are hubs.  Hubs of a colour class whose eligibility is
+// looked up once a sub-sweep (any beyond them are asked again per item).
 static constexpr int64_t TEAM_MAX_CAND = 8192;
 static constexpr int TEAM_MAX_HUBS = 16384;
 static constexpr int TEAM_MAX_BLOCKS = 1024;
