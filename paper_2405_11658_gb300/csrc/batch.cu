@@ -24,22 +24,22 @@ struct leiden_batch {
   int64_t arena_bytes = 0;
   char *d_desc = nullptr;        // SmallHeader, then SmallJob[max_graphs]
   SmallResult *d_res = nullptr;
-  SmallCtl *d_ctl = nullptr;     // control words of every block
+  SmallCtl *d_ctl = nullptr;     // control words of every block (d_desc's allocation)
   char *h_desc = nullptr;        // pinned staging of d_desc
   SmallResult *h_res = nullptr;  // pinned copy of d_res
   size_t desc_bytes = 0, res_bytes = 0;
-  // one captured graph per cluster size (2^k blocks) used so far, with the
-  // options baked into it
-  static constexpr int SIZES = 5;
-  cudaGraph_t graph[SIZES] = {};
-  cudaGraphExec_t exec[SIZES] = {};
-  SmallOpts captured[SIZES] = {};
+  // one captured graph per shape used so far (clusters of 2^k blocks, of 512 or
+  // 1024 threads), with the options baked into it
+  static constexpr int SHAPES = 10;
+  cudaGraph_t graph[SHAPES] = {};
+  cudaGraphExec_t exec[SHAPES] = {};
+  SmallOpts captured[SHAPES] = {};
 };
 
 namespace {
 
 void release(leiden_batch *b) {
-  for (int k = 0; k < leiden_batch::SIZES; k++) {
+  for (int k = 0; k < leiden_batch::SHAPES; k++) {
     if (b->exec[k]) cudaGraphExecDestroy(b->exec[k]);
     if (b->graph[k]) cudaGraphDestroy(b->graph[k]);
   }
@@ -89,8 +89,16 @@ int check_item(const leiden_batch_item &it) {
   return LEIDEN_OK;
 }
 
-// (Re)captures upload + kernel + download for opts `so` and clusters of 2^k.
-int capture(leiden_batch *b, const SmallOpts &so, int k) {
+// Cluster size (2^log2) and threads of a block, and the graphs run by clusters.
+struct Shape {
+  int log2 = 0, threads = 512;
+  int32_t wide = 0;
+  int index() const { return 2 * log2 + (threads == 1024); }
+};
+
+// (Re)captures upload + kernel + download for opts `so` and a shape.
+int capture(leiden_batch *b, const SmallOpts &so, const Shape &sh) {
+  const int k = sh.index();
   if (b->exec[k]) { cudaGraphExecDestroy(b->exec[k]); b->exec[k] = nullptr; }
   if (b->graph[k]) { cudaGraphDestroy(b->graph[k]); b->graph[k] = nullptr; }
   if (cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
@@ -100,7 +108,9 @@ int capture(leiden_batch *b, const SmallOpts &so, int k) {
   SmallHeader *hdr = reinterpret_cast<SmallHeader *>(b->d_desc);
   const SmallJob *jobs = reinterpret_cast<const SmallJob *>(b->d_desc + sizeof(SmallHeader));
   cudaMemcpyAsync(b->d_desc, b->h_desc, b->desc_bytes, cudaMemcpyHostToDevice, b->cap);
-  const int rc = launch_small(hdr, jobs, so, b->d_res, b->d_ctl, b->sms, 1 << k, b->cap);
+  const int rc = sh.threads == 512
+                     ? launch_small<512>(hdr, jobs, so, b->d_res, b->d_ctl, b->sms, 1 << sh.log2, b->cap)
+                     : launch_small<1024>(hdr, jobs, so, b->d_res, b->d_ctl, b->sms, 1 << sh.log2, b->cap);
   cudaMemcpyAsync(b->h_res, b->d_res, b->res_bytes, cudaMemcpyDeviceToHost, b->cap);
   cudaGraph_t g = nullptr;
   if (cudaStreamEndCapture(b->cap, &g) != cudaSuccess || !g || rc) {
@@ -119,29 +129,40 @@ int capture(leiden_batch *b, const SmallOpts &so, int k) {
   return LEIDEN_OK;
 }
 
-// Clusters of 2^k blocks for the largest `*wide` of the graphs (sizes: their
+// Clusters of 2^k blocks for the largest `wide` of the graphs (sizes: their
 // vertices + entries, largest first), single blocks for the others.  A cluster
 // of c blocks for w graphs leaves sms - w c blocks for the other count - w, so
 // w = (sms - count) / (c - 1) keeps every graph on SMs of its own; the largest
 // c that still covers a third of the graphs (their sizes differ, and the
 // largest ones finish last).  A graph below 6144 c is not worth the cluster's
-// barriers, about 1 us each against the block's 0.05: with clusters of 4 for
-// graphs of 1e3 vertices (1.1e4) a batch took 15% longer than with one 512-
-// thread block each.  64 graphs of 1e3..1e4 vertices (1.1e4 .. 1.1e5): single
-// blocks 28.4 ms, clusters of 2 for all 19.7, of 4 for the 20 largest 18.3, of
-// 4 for all 20.0, of 8 for the 20 largest 26.9.  Clusters have at most `most`
-// blocks, what the device can keep resident.
-int cluster_log2(int count, int sms, int most, const std::vector<int64_t> &sizes, int32_t *wide) {
-  *wide = 0;
+// barriers, about 1 us each against the block's 0.05.  Clusters have at most
+// `most` blocks, what the device can keep resident.  64 graphs of 1e3..1e4
+// vertices (1.1e4 .. 1.1e5) get clusters of 4 for up to 29 of them; with 1024
+// threads throughout, single blocks took 28.4 ms, clusters of 2 for all 19.7,
+// of 4 for all 20.0, of 8 for the 20 largest 26.9, of 4 for the 20 largest 18.3.
+//
+// 512 threads (see small.cuh) while no block has much of a graph; with more
+// colour classes S, a sub-sweep has less of it.  ms with 1024 / 512 threads by
+// the largest share of a block: S = 8: 3.3e3 4.7 / 2.7, 2.7e4 to 4.9e4 14.2 /
+// 12.7 (the 64 graphs), 21.0 / 20.6 and 17.3 / 17.2, 5.2e4 18.2 / 18.7, 1.1e5
+// 33.5 / 36.2, 3.2e5 65.9 / 78.6; S = 1: about 3e4 7.3 / 7.0, 5.5e4 12.5 /
+// 13.2; S = 32: 1.1e5 46.6 / 45.1, 2.5e5 40.8 / 41.4, 3.2e5 60.7 / 64.5;
+// S = 256: 5.5e4 132 / 81.
+Shape batch_shape(int count, int sms, int most, int log2S, const std::vector<int64_t> &sizes) {
+  Shape sh;
   for (int k = 4; k > 0; k--) {
     const int c = 1 << k;
     if (c > most) continue;
     const int w = std::min(count, std::max(0, (sms - count) / (c - 1)));
     if (3 * w < count || sizes[0] < (int64_t)6144 * c) continue;
-    while (*wide < w && sizes[*wide] >= (int64_t)3072 * c) ++*wide;
-    return k;
+    sh.log2 = k;
+    while (sh.wide < w && sizes[sh.wide] >= (int64_t)3072 * c) ++sh.wide;
+    break;
   }
-  return 0;
+  int64_t share = sizes[0] >> sh.log2;   // sizes[0] is on a cluster if any graph is
+  if (sh.wide < count) share = std::max(share, sizes[sh.wide]);
+  if (share > 24576 + ((int64_t)3072 << log2S)) sh.threads = 1024;
+  return sh;
 }
 
 bool same_opts(const SmallOpts &a, const SmallOpts &b) { return memcmp(&a, &b, sizeof(SmallOpts)) == 0; }
@@ -165,15 +186,16 @@ extern "C" int leiden_batch_create(leiden_batch **out, void *stream, int32_t max
       cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess) {
     rc = LEIDEN_ECUDA;
   }
-  if (!rc) b->max_cluster = small_max_cluster();
+  if (!rc) b->max_cluster = std::min(small_max_cluster<512>(), small_max_cluster<1024>());
   b->arena_bytes = small_layout_bound(max_total_n, max_total_nnz, max_graphs);
   b->desc_bytes = sizeof(SmallHeader) + (size_t)max_graphs * sizeof(SmallJob);
   b->res_bytes = (size_t)max_graphs * sizeof(SmallResult);
   // one device and one pinned allocation for the descriptors, the results and
   // the blocks' control words
+  const size_t ctl_bytes = (size_t)b->sms * sizeof(SmallCtl);
   const size_t desc_al = (b->desc_bytes + 255) & ~(size_t)255, res_al = (b->res_bytes + 255) & ~(size_t)255;
   if (!rc && (cudaMalloc(&b->arena, (size_t)b->arena_bytes) != cudaSuccess ||
-              cudaMalloc(&b->d_desc, desc_al + res_al + small_ctl_bytes(b->sms)) != cudaSuccess ||
+              cudaMalloc(&b->d_desc, desc_al + res_al + ctl_bytes) != cudaSuccess ||
               cudaMallocHost(&b->h_desc, desc_al + b->res_bytes) != cudaSuccess))
     rc = LEIDEN_ENOMEM;
   if (rc) {
@@ -200,7 +222,7 @@ extern "C" void leiden_batch_destroy(leiden_batch *b) {
 
 extern "C" int leiden_batch_device_bytes(leiden_batch *b, int64_t *out) {
   if (!b || !out) return LEIDEN_EINVAL;
-  *out = b->arena_bytes + (int64_t)b->desc_bytes + (int64_t)b->res_bytes + (int64_t)small_ctl_bytes(b->sms);
+  *out = b->arena_bytes + (int64_t)b->desc_bytes + (int64_t)b->res_bytes + (int64_t)b->sms * (int64_t)sizeof(SmallCtl);
   return LEIDEN_OK;
 }
 
@@ -232,7 +254,9 @@ extern "C" int leiden_batch_run(leiden_batch *b, int32_t count, const leiden_bat
   hdr->count = count;
   std::vector<int64_t> sizes(count);
   for (int k = 0; k < count; k++) sizes[k] = items[order[k]].g.nnz + items[order[k]].g.n;
-  const int lc = cluster_log2(count, b->sms, b->max_cluster, sizes, &hdr->wide);
+  const Shape sh = batch_shape(count, b->sms, b->max_cluster, so.log2S, sizes);
+  const int x = sh.index();
+  hdr->wide = sh.wide;
   hdr->next = 0;
   hdr->next1 = (uint32_t)hdr->wide;
   int64_t at = 0;
@@ -260,13 +284,13 @@ extern "C" int leiden_batch_run(leiden_batch *b, int32_t count, const leiden_bat
   }
   if (at > b->arena_bytes) return LEIDEN_ENOMEM;  // cannot happen within the totals; kept as a guard
   // the previous run's graph is still in flight until this stream point
-  if (!b->exec[lc] || !same_opts(so, b->captured[lc])) {
+  if (!b->exec[x] || !same_opts(so, b->captured[x])) {
     cudaStreamSynchronize(b->st);
-    rc = capture(b, so, lc);
+    rc = capture(b, so, sh);
     if (rc) return rc;
   }
   note_launch();
-  if (cudaGraphLaunch(b->exec[lc], b->st) != cudaSuccess) {
+  if (cudaGraphLaunch(b->exec[x], b->st) != cudaSuccess) {
     cudaGetLastError();
     return LEIDEN_ECUDA;
   }

@@ -1,4 +1,5 @@
-// small.cu -- many small graphs in one persistent launch (leiden_batch_run).
+// small.cuh -- many small graphs in one persistent launch (leiden_batch_run).
+// Compiled for two block sizes (small_512.cu, small_1024.cu).
 //
 // Each team of blocks (team.cuh) runs the whole of Alg. leiden for one graph
 // at a time -- marking (Alg. naive / delta / frontier), every pass, the
@@ -13,9 +14,15 @@
 // What bounds it: one graph's chain of sub-sweeps, each two barriers and the
 // dependent loads of one vertex; a cluster shortens the work between the
 // barriers, and with fewer graphs than SMs the others would be idle anyway.
-// 64 graphs of 1e3..1e4 vertices, half of them updates: 50 ms with a 512-
-// thread block per graph, tables cleared per vertex and 128-bit scores
-// throughout, 14 ms as here.
+// On the smallest graphs it is the code itself: 1024 threads leave 64 registers
+// each, and the spilled words of a block (270 KB) do not fit the L1 that the
+// tables leave, so every reload waits for L2 (L1 hit rate 34%).  512 threads
+// hold everything in 128 registers; with more of a graph to a block, 1024's
+// gathers in flight count for more (batch.cu has the rule).  ms with one 512-thread block per graph, tables cleared per
+// vertex and 128-bit scores throughout / 1024 threads here / 512 threads here:
+// 64 graphs of 1e3..1e4 vertices, half of them updates 47.8 / 14.2 / 12.7; 8
+// graphs of up to 300 vertices 3.2 / 4.7 / 2.7; 88 of up to 1000 8.3 / 8.0 /
+// 5.9; 60 R-MAT of scale 14 176 / 69 / 81.
 #include <limits.h>
 
 #include "common.cuh"
@@ -24,18 +31,7 @@
 #include "team.cuh"
 
 namespace lk {
-
-// Control words of one block (of a cluster: those of its first block).
-struct SmallCtl {
-  TeamCtl t;
-  u64 err;                  // input checks and device consistency flags
-  u64 two_m, kmax, inside;
-  u64 sq[2];
-  u64 affected;
-  int32_t job;
-};
-
-size_t small_ctl_bytes(int blocks) { return (size_t)blocks * sizeof(SmallCtl); }
+inline namespace LK_TEAM_SPACE {
 
 namespace {
 
@@ -575,7 +571,10 @@ static void small_config(int blocks, int cluster, cudaStream_t s, cudaLaunchAttr
   cfg->numAttrs = 1;
 }
 
-int small_max_cluster() {
+}  // namespace LK_TEAM_SPACE
+
+template <>
+int small_max_cluster<LK_TEAM_THREADS>() {
   for (int c = 16; c > 1; c >>= 1) {
     cudaLaunchAttribute attr{};
     cudaLaunchConfig_t cfg;
@@ -587,8 +586,9 @@ int small_max_cluster() {
   return 1;
 }
 
-int launch_small(SmallHeader *hdr, const SmallJob *jobs, const SmallOpts &o, SmallResult *results, SmallCtl *ctl,
-                 int blocks, int cluster, cudaStream_t s) {
+template <>
+int launch_small<LK_TEAM_THREADS>(SmallHeader *hdr, const SmallJob *jobs, const SmallOpts &o, SmallResult *results,
+                                  SmallCtl *ctl, int blocks, int cluster, cudaStream_t s) {
   cudaLaunchAttribute attr{};
   cudaLaunchConfig_t cfg;
   small_config(blocks, cluster, s, &attr, &cfg);

@@ -1,5 +1,5 @@
 // small.h -- device-visible descriptors of the persistent many-graph kernel
-// (small.cu) and the workspace layout of one graph, shared by the kernel and
+// (small.cuh) and the workspace layout of one graph, shared by the kernel and
 // its host driver (batch.cu).
 #pragma once
 
@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "leiden.h"
+#include "team.h"
 
 namespace lk {
 
@@ -112,14 +113,31 @@ __host__ __device__ inline int64_t small_layout_bound(int64_t n, int64_t nnz, in
   return n * 97 + nnz * 61 + graphs * (34 * 256 + 8192);
 }
 
-struct SmallCtl;
-size_t small_ctl_bytes(int blocks);
+// Control words of one block (of a cluster: those of its first block).
+struct SmallCtl {
+  TeamCtl t;
+  u64 err;                  // input checks and device consistency flags
+  u64 two_m, kmax, inside;
+  u64 sq[2];
+  u64 affected;
+  int32_t job;
+};
+
+// The kernel with THREADS (512 or 1024) threads a block.
 // Blocks of the largest cluster (1, 2, 4, 8 or 16) that can be resident on the
 // current device.
+template <int THREADS>
 int small_max_cluster();
 // Enqueues the kernel: `blocks` blocks in clusters of `cluster`; jobs before
 // hdr->wide are run by whole clusters, the others by single blocks.
+template <int THREADS>
 int launch_small(SmallHeader *hdr, const SmallJob *jobs, const SmallOpts &o, SmallResult *results, SmallCtl *ctl,
                  int blocks, int cluster, cudaStream_t s);
+template <> int small_max_cluster<512>();
+template <> int small_max_cluster<1024>();
+template <> int launch_small<512>(SmallHeader *, const SmallJob *, const SmallOpts &, SmallResult *, SmallCtl *, int,
+                                  int, cudaStream_t);
+template <> int launch_small<1024>(SmallHeader *, const SmallJob *, const SmallOpts &, SmallResult *, SmallCtl *, int,
+                                   int, cudaStream_t);
 
 }  // namespace lk

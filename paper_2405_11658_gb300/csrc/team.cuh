@@ -31,11 +31,21 @@
 
 namespace lk {
 
-static constexpr int TEAM_THREADS = 1024;
+// Threads of a block: 1024 unless the including file says otherwise (512; see
+// small.cuh).  The code of each shape has a namespace of its own.
+#ifndef LK_TEAM_THREADS
+#define LK_TEAM_THREADS 1024
+#endif
+#define LK_TEAM_CAT2(a, b) a##b
+#define LK_TEAM_CAT(a, b) LK_TEAM_CAT2(a, b)
+#define LK_TEAM_SPACE LK_TEAM_CAT(team_, LK_TEAM_THREADS)
+inline namespace LK_TEAM_SPACE {
+
+static constexpr int TEAM_THREADS = LK_TEAM_THREADS;
 static constexpr int TEAM_WARPS = TEAM_THREADS / 32;
 // Hashtable slots per warp; a sub-block of 8 warps pools 8 of them, the whole
-// block all 32 (16384 slots).
-static constexpr int TEAM_WSLOTS = 512;
+// block all of them (16384 slots).
+static constexpr int TEAM_WSLOTS = 16384 / TEAM_WARPS;
 static constexpr int TEAM_SUB = 256;                     // threads of a sub-block
 static constexpr int TEAM_NSUB = TEAM_THREADS / TEAM_SUB;
 // Degree tiers: one lane per vertex, 16 lanes, a warp with one, four or eight
@@ -1079,7 +1089,7 @@ __device__ __forceinline__ int64_t team_block_sum(int64_t v, TeamShared<ST> &sm)
   __syncthreads();
   if (lane == 0) sm.red64[warp] = v;
   __syncthreads();
-  int64_t r = sm.red64[lane];
+  int64_t r = lane < TEAM_WARPS ? sm.red64[lane] : 0;
   for (int o = 16; o; o >>= 1) r += shfl_xor_i64(r, o);
   return r;
 }
@@ -1123,7 +1133,7 @@ __device__ __forceinline__ int64_t team_scan(int64_t n, Team &t, TeamShared<ST> 
     __syncthreads();
     if (lane == 31) sm.red64[warp] = incl;
     __syncthreads();
-    int64_t ws = sm.red64[lane], wi = ws;
+    int64_t ws = lane < TEAM_WARPS ? sm.red64[lane] : 0, wi = ws;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int64_t y = shfl_i64(wi, (lane - o) & 31);
@@ -1230,7 +1240,7 @@ __device__ __forceinline__ int team_local_move(const GL &g, const AR &a, const C
         if ((threadIdx.x & 31) == 0) sm.red128[threadIdx.x >> 5] = acc;
         __syncthreads();
         if (threadIdx.x < 32) {
-          acc = sm.red128[threadIdx.x];
+          acc = threadIdx.x < TEAM_WARPS ? sm.red128[threadIdx.x] : 0;
           for (int o = 16; o; o >>= 1) acc += shfl_xor_i128(acc, o);
           if (threadIdx.x == 0 && acc != 0) atomic_add_i128(sums, acc);
         }
@@ -1591,4 +1601,5 @@ __device__ __forceinline__ void team_pass(const GL &g, AR &a, const CT &ct, int 
   if (t.rank == 0 && threadIdx.x == 0) ctl->status = TEAM_AGGREGATED;
 }
 
+}  // namespace LK_TEAM_SPACE
 }  // namespace lk

@@ -12,6 +12,7 @@ import pytest
 
 sys.path.insert(0, __file__.rsplit("/", 1)[0])
 import host_library  # noqa: E402
+from batch_shapes import SHAPES  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -57,7 +58,7 @@ class Host:
         self.lib.leiden_ctx_destroy(ctx)
         return rc
 
-    def batch(self, sizes):
+    def batch(self, sizes, subsets=8):
         """sizes: (n, nnz) of each graph."""
         b = C.c_void_p()
         assert self.lib.leiden_batch_create(C.byref(b), None, len(sizes), C.c_int64(sum(s[0] for s in sizes)),
@@ -71,6 +72,7 @@ class Host:
             keep.append((self.off, self.dummy, out))
             it.out = out.ctypes.data
         o = self.opts()
+        o.det_subsets = subsets
         rc = self.lib.leiden_batch_run(b, len(sizes), items, C.byref(o), res)
         self.lib.leiden_batch_destroy(b)
         return rc
@@ -115,3 +117,20 @@ def test_batch_clusters_fit_the_device(host, most):
     small = [x for x in host.log() if "small_leiden_k" in x[1]]
     assert [x[4] for x in small] == [most] and not small[0][6]
     assert host.lib.fake_pending_error() == 0
+
+
+@pytest.mark.parametrize("name", list(SHAPES))
+def test_batch_shapes(host, name):
+    sizes, cluster, threads, _ = SHAPES[name]
+    host.reset()
+    assert host.batch([(s // 10, s - s // 10) for s in sizes]) == 0
+    assert [(x[4], x[3]) for x in host.log() if "small_leiden_k" in x[1]] == [(cluster, threads)]
+
+
+@pytest.mark.parametrize("share,subsets,threads", [(27648, 1, 512), (27649, 1, 1024), (49152, 8, 512), (49153, 8, 1024),
+                                                   (122880, 32, 512), (122881, 32, 1024)])
+def test_batch_threads_by_the_share_of_a_block(host, share, subsets, threads):
+    host.reset()
+    host.lib.fake_set_max_cluster(1)
+    assert host.batch([(100, share - 100), (100, 900)], subsets) == 0
+    assert [x[3] for x in host.log() if "small_leiden_k" in x[1]] == [threads]
