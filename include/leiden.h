@@ -338,7 +338,10 @@ int leiden_batch_device_bytes(leiden_batch *b, int64_t *out);
  *     which runs every ready small request in one persistent launch
  *     (leiden_batch_run), so a new launch can start while another runs;
  *   - larger graphs go to `large_slots` workers, each with its own context and
- *     stream, so their updates overlap on the device.
+ *     stream: one's host work and short kernels overlap another's passes, while
+ *     the resident passes themselves (DET, one block per SM) take turns.  While
+ *     a small graph is resident they leave 32 SMs to the small workers, whose
+ *     requests then do not wait for a pass to end.
  * Results are DET: each request's membership does not depend on what else
  * ran beside it.
  * ------------------------------------------------------------------------- */

@@ -45,6 +45,7 @@ struct leiden_ctx {
   int64_t max_n = 0, max_nnz = 0;
   TierTable tiers{};
   bool tiers_set = false;  // the caller chose another table than the default
+  int team_sms = INT_MAX;  // SMs a resident pass takes at most
   int agg_uniform = 0;   // aggregation policy (leiden_ctx_set_agg_policy)
   std::vector<void *> allocs;
   int64_t device_bytes = 0;
@@ -96,6 +97,8 @@ struct leiden_ctx {
 };
 
 cudaStream_t lk::ctx_stream(leiden_ctx *c) { return c->st; }
+int lk::ctx_sms(leiden_ctx *c) { return c->sms; }
+void lk::ctx_limit_team(leiden_ctx *c, int sms) { c->team_sms = sms; }
 
 lk::CtxScope::CtxScope(leiden_ctx *c) {
   if (c && c->green.cu) pushed = green_push(c->green);
@@ -697,7 +700,7 @@ int team_pass_host(Run &r, GraphView<WT> g, int64_t nnz, int lp, double tau, int
   ta.agg_slots = (!c->agg_uniform && nnz <= TEAM_AGG_NNZ && 2 * slots <= c->gcap) ? slots : 0;
   ta.ctl = c->tctl;
   cudaMemsetAsync(c->tctl, 0, sizeof(TeamCtl), c->st);
-  int64_t nb = std::min<int64_t>(c->sms, (nnz + g.n + TEAM_BLOCK_SIZE - 1) / TEAM_BLOCK_SIZE);
+  int64_t nb = std::min<int64_t>(std::min(c->team_sms, c->sms), (nnz + g.n + TEAM_BLOCK_SIZE - 1) / TEAM_BLOCK_SIZE);
   int kind = nb > 1 ? TEAM_GRID : TEAM_BLOCK;
   const bool narrow = !LK_FORCE_WIDE_SCORES && narrow_scores(r, b);
   // a context on a share of the SMs may not hold a whole cluster

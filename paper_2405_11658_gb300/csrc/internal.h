@@ -45,6 +45,10 @@ int tiers_from_public(const leiden_tier_table *p, TierTable *out);
 void tiers_to_public(const TierTable &tt, leiden_tier_table *out);
 // The stream a context is bound to.
 cudaStream_t ctx_stream(leiden_ctx *c);
+// The SMs a context runs on, and the most of them its resident passes take (a
+// pass keeps its SMs to itself until it ends).
+int ctx_sms(leiden_ctx *c);
+void ctx_limit_team(leiden_ctx *c, int sms);
 
 // green.cu: a green context (the primary context restricted to a share of the
 // SMs).  green_push makes it current on the calling thread; green_pop undoes

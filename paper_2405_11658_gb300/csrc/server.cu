@@ -6,11 +6,12 @@
 //     of a small graph into one persistent launch (leiden_batch_run) after
 //     building each G^t, so one launch can start while another runs;
 //   * `large_slots` workers, each with its own leiden_ctx and stream, run the
-//     updates of large graphs concurrently on the device.
+//     updates of large graphs, pass by pass in turn on the device.
 // Host code only; every step on the device is a library call.
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <deque>
@@ -77,6 +78,7 @@ struct leiden_server {
   std::unordered_map<int32_t, Resident *> graphs;
   std::unordered_map<int64_t, Request *> reqs;
   int64_t pending = 0;            // requests not yet done
+  std::atomic<int> small_resident{0};
   int64_t workspace_bytes = 0, resident_bytes = 0;
   leiden_server_stats st{};
   // workers
@@ -153,6 +155,19 @@ void finish(leiden_server *s, Resident *g, std::vector<Request *> &done) {
   s->cv.notify_all();
 }
 
+// SMs the resident passes of large graphs leave to the small workers while a
+// small graph is resident.  A pass holds its SMs for milliseconds, and a small
+// request is a few dozen short launches one after the other: with no SM to
+// spare each of them waited for a whole pass.  Latency p50 (ms) of a small request alone / of 16 at once, and
+// the large graphs' updates/s, with two R-MAT graphs of scale 20 under update:
+// 22 / 70 / 33.8 with none left, 18 / 56 / 34.4 with 8, 13 / 48 / 35.2 with 16,
+// 14 / 45 / 35.5 with 32, 16 / 48 / 34.4 with 64; with two 9e6-vertex grids 21 /
+// 72 / 25.8, 16 / 60 / 26.2, 14 / 57 / 28.1, 9 / 32 / 28.0, 8 / 47 / 27.2; one
+// launch per tier and sub-sweep gave 39 / 65 / 22.6 and 23 / 38 / 15.1.  An
+// update beside idle small graphs takes 3% longer (Chung-Lu of 6e7 entries 47.1
+// -> 48.6 ms).
+constexpr int kSmallSms = 32;
+
 // One request of a large graph on worker k.
 void run_large(leiden_server *s, int k, Resident *g, Request *r) {
   leiden_ctx *ctx = s->large_ctx[k];
@@ -163,6 +178,8 @@ void run_large(leiden_server *s, int k, Resident *g, Request *r) {
   int rc = LEIDEN_OK;
   double q = 0.0;
   leiden_ctx_set_tiers(ctx, g->tuned ? &g->tiers : nullptr);
+  const int sms = lk::ctx_sms(ctx);
+  lk::ctx_limit_team(ctx, s->small_resident.load() > 0 ? std::max(sms - kSmallSms, (sms + 1) / 2) : sms);
   if (r->is_static) {
     leiden_csr c = csr_of(*g, g->csr, g->nnz);
     if (s->cfg.autotune_trials > 0) {
@@ -560,6 +577,7 @@ extern "C" int leiden_server_admit(leiden_server *s, int64_t n, int64_t nnz, con
     g->queue.push_back(r);
     s->pending++;
     s->st.resident_graphs++;
+    if (small) s->small_resident++;
     s->cv.notify_all();
   }
   *graph_id = g->id;
@@ -653,6 +671,7 @@ extern "C" int leiden_server_evict(leiden_server *s, int32_t graph_id) {
   s->graphs.erase(graph_id);
   s->resident_bytes -= g->bytes;
   s->st.resident_graphs--;
+  if (g->small) s->small_resident--;
   free_graph(g);
   delete g;
   s->cv.notify_all();

@@ -7,7 +7,9 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
 #include <map>
+#include <mutex>
 #include <string>
 #include <utility>
 
@@ -18,6 +20,7 @@ int g_max_cluster = 16;             // larger clusters never fit
 bool g_refuse_coop = false, g_refuse_cluster = false;
 cudaError_t g_last = cudaSuccess;
 std::string g_log;
+std::recursive_mutex g_mu;             // the server calls from its workers' threads
 std::map<std::pair<int, const void *>, std::map<int, int>> g_attr;   // (device, kernel) -> attributes
 
 std::map<const void *, std::string> &names() {
@@ -31,6 +34,7 @@ cudaError_t fail(cudaError_t e) {
 }
 
 cudaError_t launch(const void *f, dim3 grid, dim3 block, size_t smem, int cluster, bool coop) {
+  std::lock_guard<std::recursive_mutex> lock(g_mu);
   const auto &at = g_attr[{g_device, f}];
   auto have = [&](int a, int d) { auto i = at.find(a); return i == at.end() ? d : i->second; };
   cudaError_t e = cudaSuccess;
@@ -50,7 +54,7 @@ thread_local Call t_call;
 
 void *token() {
   static char t[64];
-  static int k = 0;
+  static std::atomic<unsigned> k{0};
   return &t[k++ % 64];
 }
 
@@ -103,10 +107,12 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void
   return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, cluster, coop);
 }
 cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute a, int v) {
+  std::lock_guard<std::recursive_mutex> lock(g_mu);
   g_attr[{g_device, f}][(int)a] = v;
   return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *f, const cudaLaunchConfig_t *c) {
+  std::lock_guard<std::recursive_mutex> lock(g_mu);
   const auto &at = g_attr[{g_device, f}];
   auto have = [&](int a, int d) { auto i = at.find(a); return i == at.end() ? d : i->second; };
   const int cl = (int)c->attrs[0].val.clusterDim.x;

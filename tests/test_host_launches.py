@@ -134,3 +134,40 @@ def test_batch_threads_by_the_share_of_a_block(host, share, subsets, threads):
     host.lib.fake_set_max_cluster(1)
     assert host.batch([(100, share - 100), (100, 900)], subsets) == 0
     assert [x[3] for x in host.log() if "small_leiden_k" in x[1]] == [threads]
+
+
+def admit(host, srv, n, nnz):
+    """Admits a graph of these sizes and waits for its Static run."""
+    off = np.zeros(n + 1, np.int64)
+    off[n] = nnz
+    idx = np.zeros(max(nnz, 1), np.int32)
+    gid, rid = C.c_int32(), C.c_int64()
+    assert host.lib.leiden_server_admit(srv, C.c_int64(n), C.c_int64(nnz), C.c_void_p(off.ctypes.data),
+                                        C.c_void_p(idx.ctypes.data), C.c_void_p(idx.ctypes.data), C.byref(gid),
+                                        C.byref(rid)) == 0
+    info = host.L._RequestInfo()
+    assert host.lib.leiden_server_wait(srv, rid, C.c_double(-1.0), C.byref(info)) == 0
+    return gid
+
+
+def test_the_server_leaves_sms_to_the_small_workers(host):
+    # a large graph's pass takes 32 SMs less while a small graph is resident
+    host.reset()
+    cfg = host.L._ServerConfig()
+    host.lib.leiden_server_config_default(C.byref(cfg))
+    n, nnz = 20000, 4000000
+    cfg.small_max_n, cfg.small_max_nnz, cfg.large_max_n, cfg.large_max_nnz = 1000, 10000, n, 2 * nnz
+    srv = C.c_void_p()
+    assert host.lib.leiden_server_create(C.byref(srv), C.byref(cfg)) == 0
+
+    def large():
+        first = len(host.log())
+        admit(host, srv, n, nnz)
+        return [x[2] for x in host.log()[first:] if "team_pass_k" in x[1]]
+
+    assert large() == [152]
+    small = admit(host, srv, 100, 1000)
+    assert large() == [152 - 32]
+    assert host.lib.leiden_server_evict(srv, small) == 0
+    assert large() == [152]
+    host.lib.leiden_server_destroy(srv)
