@@ -109,11 +109,12 @@ def peaks():
         return 6800.0, "fallback"
 
 
-# The decide kernels' sources: a DRAM-traffic figure measured by ncu (stored
-# under profiles/) stays valid only while these files are unchanged.
-DECIDE_SOURCES = ("paper_2405_11658_gb300/csrc/move.cu", "paper_2405_11658_gb300/csrc/hub.cu",
-                  "paper_2405_11658_gb300/csrc/internal.h", "paper_2405_11658_gb300/csrc/common.cuh",
-                  "paper_2405_11658_gb300/csrc/api.cu")
+# The sources of the decide phase, as the multi-kernel path's kernels and as part
+# of the resident pass: a DRAM-traffic figure measured by ncu (stored under
+# profiles/) stays valid only while these files are unchanged.
+DECIDE_SOURCES = tuple("paper_2405_11658_gb300/csrc/" + f for f in (
+    "move.cu", "hub.cu", "internal.h", "common.cuh", "api.cu", "team.cuh", "team.h", "team_launch.cuh", "team_n32.cu",
+    "team_n64.cu", "team_w32.cu", "team_w64.cu"))
 TRAFFIC_FILES = {"cl": os.path.join(ROOT, "profiles", "decide_traffic_cl.json"),
                  "rmat": os.path.join(ROOT, "profiles", "decide_traffic_rmat22.json")}
 
@@ -1234,7 +1235,9 @@ def record_traffic(args):
     dram__bytes_write.sum, gpu__time_duration.sum; --nvtx-include
     "local_move_pass0/") and the JSON line the same --profile-static command
     printed: DRAM bytes of the decide kernels per colour class and per scanned
-    CSR entry, next to their algorithmic bytes."""
+    CSR entry, next to their algorithmic bytes.  A capture without decide
+    kernels -- of a resident pass, whose one launch does more than decide -- has
+    no such figure and is refused."""
     import csv
     rows = list(csv.reader(open(args.record_traffic)))
     start = next(k for k, r in enumerate(rows) if r and r[0] == "ID")
@@ -1254,6 +1257,9 @@ def record_traffic(args):
             kernels += 1
         elif r[mn] == "dram__bytes_write.sum":
             wr += v
+    if not kernels:
+        print(f"{args.record_traffic}: no decide kernel in this capture, nothing recorded", file=sys.stderr)
+        return 1
     prof = None
     for ln in open(args.profile_json):
         ln = ln.strip()
@@ -1279,9 +1285,10 @@ def run_profile_static(args):
     ``rmat``; ``--cl-div k`` takes the Chung-Lu recipe at 1/k of the vertices
     and edges) with the decide kernels timed; prints the run's statistics as
     one JSON line.  A profiler run over this command sees exactly one run's
-    launches (local-moving inside the NVTX range "local_move", its first pass
-    in "local_move_pass0", refinement in "refine", aggregation in
-    "aggregate")."""
+    launches (a resident pass inside the NVTX range "resident_pass", the first
+    one in "resident_pass0"; on the multi-kernel path local-moving in
+    "local_move", its first pass in "local_move_pass0", refinement in "refine";
+    aggregation in "aggregate")."""
     import torch
     torch.cuda.set_device(0)
     import paper_2405_11658_gb300 as L
