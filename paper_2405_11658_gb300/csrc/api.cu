@@ -869,7 +869,7 @@ int setup_run(leiden_ctx *c, const leiden_csr *g, const leiden_opts *o, Run &r) 
   if (rc) return rc;
   cudaMemsetAsync(&c->ctr[CTR_ERROR], 0, sizeof(u64), c->st);
   launch_row_sums(GraphView<int32_t>{g->n, g->off, g->idx, g->w}, g->nnz, c->K0, &c->ctr[CTR_SCRATCH0],
-                  &c->ctr[CTR_ERROR], c->st);
+                  &c->ctr[CTR_ERROR], c->sms, c->st);
   cudaMemcpyAsync(c->h_ctr, c->ctr, CTR_COUNT * sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   rc = sync(c);
   if (rc) return rc;
@@ -896,7 +896,7 @@ int modularity_of(leiden_ctx *c, const leiden_csr *g, const int32_t *C, int64_t 
                   double *q_out) {
   if (!unchecked && g->nnz > kModMaxNnz) return LEIDEN_EOVERFLOW;
   GraphView<int32_t> gv{g->n, g->off, g->idx, g->w};
-  launch_modularity_terms(gv, g->nnz, C, c->Ktmp, &c->ctr[CTR_SCRATCH0], &c->ctr[CTR_ERROR], c->st);
+  launch_modularity_terms(gv, g->nnz, C, c->Ktmp, &c->ctr[CTR_SCRATCH0], &c->ctr[CTR_ERROR], c->sms, c->st);
   cudaMemcpyAsync(&c->h_ctr[CTR_SCRATCH0], &c->ctr[CTR_SCRATCH0], 4 * sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   cudaMemcpyAsync(&c->h_ctr[CTR_ERROR], &c->ctr[CTR_ERROR], sizeof(u64), cudaMemcpyDeviceToHost, c->st);
   int rc = sync(c);
@@ -1357,6 +1357,7 @@ int leiden_apply_batch(leiden_ctx *c, const leiden_csr *g, const leiden_edges *d
   w.counts = &c->ctr[CTR_SCRATCH0];
   w.scan_tmp = c->scan_tmp;
   w.err = &c->ctr[CTR_ERROR];
+  w.sms = c->sms;
   rc = apply_batch(g->n, g->off, g->idx, g->w, nd, nd ? del->src : nullptr, nd ? del->dst : nullptr,
                    nd ? del->w : nullptr, ni, ni ? ins->src : nullptr, ni ? ins->dst : nullptr,
                    ni ? ins->w : nullptr, off_out, idx_out, w_out, cap_nnz, nnz_out, w, c->st);

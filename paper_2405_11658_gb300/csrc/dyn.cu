@@ -547,7 +547,7 @@ int apply_batch(int64_t n, const int64_t *off, const int32_t *idx, const int32_t
                                                       off, idx, w, wk.newdeg, wk.big, wk.pt, wk.pp, wk.counts, wk.err);
     // a row with more than BA_ROW_SERIAL updates needs that many in the batch
     if (2 * (nd + ni) > BA_ROW_SERIAL)
-      LK_COUNTED ba_row_big_k<<<gridd(2 * (nd + ni) / BA_ROW_SERIAL, 1, 152 * 6), BA_BIG_THREADS, 0, s>>>(
+      LK_COUNTED ba_row_big_k<<<gridd(2 * (nd + ni) / BA_ROW_SERIAL, 1, wk.sms * 6), BA_BIG_THREADS, 0, s>>>(
           wk.trow, wk.uoff, wk.ut, wk.uw, wk.uk, wk.Rp, wk.Np, wk.cnt, off, idx, w, wk.newdeg, wk.big, wk.pt, wk.pp,
           wk.counts, wk.err);
   }
@@ -569,7 +569,7 @@ int apply_batch(int64_t n, const int64_t *off, const int32_t *idx, const int32_t
   if (T > 0) {
     LK_COUNTED ba_merge_k<<<gridd(T * BA_MERGE_LANES, 256, 152 * 32), 256, 0, s>>>(
         T, wk.trow, wk.uoff, wk.cnt, wk.ut, wk.uw, wk.uk, wk.Rp, wk.Np, off, idx, w, off_out, idx_out, w_out, wk.err);
-    LK_COUNTED ba_merge_pieces_k<<<152 * 8, 256, 0, s>>>(wk.counts, wk.pt, wk.pp, wk.trow, wk.uoff, wk.cnt, wk.ut,
+    LK_COUNTED ba_merge_pieces_k<<<wk.sms * 8, 256, 0, s>>>(wk.counts, wk.pt, wk.pp, wk.trow, wk.uoff, wk.cnt, wk.ut,
                                                          wk.uw, wk.uk, wk.Rp, wk.Np, off, idx, w, off_out, idx_out,
                                                          w_out, wk.err);
   }

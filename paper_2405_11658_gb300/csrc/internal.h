@@ -238,6 +238,7 @@ int64_t bucket_blockhist_elems(int64_t n, int nkeys);
 // scan.cu.  Function attributes and occupancy belong to the current device, so
 // what has been set or asked is remembered per device.
 int current_device();
+int device_sms();
 // Lets `func` have `bytes` of dynamic shared memory.
 void ensure_smem(const void *func, size_t bytes);
 // Lets `func` be launched in clusters of more than 8 blocks.
@@ -252,7 +253,7 @@ int64_t scan_tmp_elems(int64_t n);
 // misc.cu
 // One pass that checks a CSR of nnz entries (a malformed one sets 512 in *err;
 // nothing outside the arrays is touched) and writes K; acc[3] = 2m.
-void launch_row_sums(GraphView<int32_t> g, int64_t nnz, int64_t *K, u64 *acc, u64 *err, cudaStream_t s);
+void launch_row_sums(GraphView<int32_t> g, int64_t nnz, int64_t *K, u64 *acc, u64 *err, int sms, cudaStream_t s);
 void launch_iota(int32_t *a, int64_t n, cudaStream_t s);
 void launch_fill_u8(uint8_t *a, uint8_t v, int64_t n, cudaStream_t s);
 void launch_copy_i64(int64_t *dst, const int64_t *src, int64_t n, cudaStream_t s);
@@ -272,7 +273,7 @@ void launch_canonical(int64_t n, const int32_t *C, int32_t *out, int32_t *minv, 
 // acc[1..2] sum of Sigma_c^2 (i128), acc[3] 2m.  Checks as launch_row_sums,
 // and the labels against [0, n).
 void launch_modularity_terms(GraphView<int32_t> g, int64_t nnz, const int32_t *C, int64_t *Sig_tmp, u64 *acc,
-                             u64 *err, cudaStream_t s);
+                             u64 *err, int sms, cudaStream_t s);
 void launch_update_weights(int64_t count, const int32_t *src, const int32_t *dst,
                            const int32_t *w, int sign, const int32_t *Cprev, int64_t *K,
                            int64_t *Sig, cudaStream_t s);
@@ -350,6 +351,7 @@ struct BatchWork {
   uint32_t *bits;    // [nnz/32 + 1] row starts
   int64_t *scan_tmp;
   u64 *err;
+  int sms;
 };
 int apply_batch(int64_t n, const int64_t *off, const int32_t *idx, const int32_t *w,
                 int64_t nd, const int32_t *ds, const int32_t *dd, const int32_t *dw,

@@ -168,13 +168,13 @@ __global__ void check_graph_rows_k(int64_t n, int64_t nnz, const int64_t *off, c
 
 template <bool MOD>
 static void launch_rows(GraphView<int32_t> g, int64_t nnz, const int32_t *C, int64_t *K, int64_t *Sig, u64 *acc,
-                        u64 *err, cudaStream_t s) {
-  LK_COUNTED check_graph_rows_k<<<grid_for(g.n > 0 ? g.n : 1, 256, 152 * 32), 256, 0, s>>>(g.n, nnz, g.off, C, err);
+                        u64 *err, int sms, cudaStream_t s) {
+  LK_COUNTED check_graph_rows_k<<<grid_for(g.n > 0 ? g.n : 1, 256, sms * 32), 256, 0, s>>>(g.n, nnz, g.off, C, err);
   if (g.n <= 0) return;
   auto k2 = rows_k<2, MOD>;
   auto k8 = rows_k<8, MOD>;
   const bool two = nnz <= 8 * g.n;
-  const int64_t cap = resident_blocks(two ? (const void *)k2 : (const void *)k8, ROWS_THREADS, 0, 152);
+  const int64_t cap = resident_blocks(two ? (const void *)k2 : (const void *)k8, ROWS_THREADS, 0, sms);
   // pieces of 256 .. 2048 items, small ones where the graph is too short to
   // give every resident warp one of the longer
   int64_t ch = (g.n + nnz) / (cap * ROWS_WARPS);
@@ -185,10 +185,10 @@ static void launch_rows(GraphView<int32_t> g, int64_t nnz, const int32_t *C, int
   else LK_COUNTED k8<<<(unsigned)blocks, ROWS_THREADS, 0, s>>>(g, nnz, C, K, Sig, acc, err, ch);
 }
 
-void launch_row_sums(GraphView<int32_t> g, int64_t nnz, int64_t *K, u64 *acc, u64 *err, cudaStream_t s) {
+void launch_row_sums(GraphView<int32_t> g, int64_t nnz, int64_t *K, u64 *acc, u64 *err, int sms, cudaStream_t s) {
   cudaMemsetAsync(acc, 0, 4 * sizeof(u64), s);
   if (g.n > 0) cudaMemsetAsync(K, 0, (size_t)g.n * sizeof(int64_t), s);
-  launch_rows<false>(g, nnz, nullptr, K, nullptr, acc, err, s);
+  launch_rows<false>(g, nnz, nullptr, K, nullptr, acc, err, sms, s);
 }
 
 __global__ void iota_k(int32_t *a, int64_t n) { GRID_STRIDE(i, n) a[i] = (int32_t)i; }
@@ -331,11 +331,11 @@ __global__ void mod_sq_k(int64_t n, const int64_t *Sig, u64 *acc) {
   if (threadIdx.x == 0 && s != 0) atomic_add_i128(&acc[1], s);
 }
 void launch_modularity_terms(GraphView<int32_t> g, int64_t nnz, const int32_t *C, int64_t *Sig_tmp, u64 *acc,
-                             u64 *err, cudaStream_t s) {
+                             u64 *err, int sms, cudaStream_t s) {
   cudaMemsetAsync(acc, 0, 4 * sizeof(u64), s);
   if (g.n > 0) cudaMemsetAsync(Sig_tmp, 0, (size_t)g.n * sizeof(int64_t), s);
-  launch_rows<true>(g, nnz, C, nullptr, Sig_tmp, acc, err, s);
-  if (g.n > 0) LK_COUNTED mod_sq_k<<<grid_for(g.n, 256, 152 * 8), 256, 0, s>>>(g.n, Sig_tmp, acc);
+  launch_rows<true>(g, nnz, C, nullptr, Sig_tmp, acc, err, sms, s);
+  if (g.n > 0) LK_COUNTED mod_sq_k<<<grid_for(g.n, 256, sms * 8), 256, 0, s>>>(g.n, Sig_tmp, acc);
 }
 
 // Sigma[c] = sum of K over members of c (Sigma zeroed first).

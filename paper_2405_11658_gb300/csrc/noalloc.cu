@@ -79,7 +79,7 @@ extern "C" int leiden_modularity_noalloc(const leiden_csr *g, const int32_t *mem
   // and flagged), so the checks and the terms take one pass and one wait.
   cudaMemsetAsync(acc + 8, 0, sizeof(unsigned long long), s);
   lk::GraphView<int32_t> gv{g->n, g->off, g->idx, g->w};
-  lk::launch_modularity_terms(gv, g->nnz, membership, sig, acc, acc + 8, s);  // zeroes sig[0..n), acc[0..3]
+  lk::launch_modularity_terms(gv, g->nnz, membership, sig, acc, acc + 8, lk::device_sms(), s);  // zeroes sig[0..n), acc[0..3]
   cudaMemcpyAsync(h, acc, 9 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
   if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return LEIDEN_ECUDA;
   if (h[8]) return LEIDEN_EINVAL;

@@ -21,6 +21,15 @@ int current_device() {
   return d;
 }
 
+int device_sms() {
+  int n = 0;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, current_device()) != cudaSuccess || n < 1) {
+    (void)cudaGetLastError();
+    n = 1;
+  }
+  return n;
+}
+
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` (once per
 // device, kernel and size; the attribute outlives the call, so it is set only
 // when the requested size grows).

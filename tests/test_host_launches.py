@@ -171,3 +171,16 @@ def test_the_server_leaves_sms_to_the_small_workers(host):
     assert host.lib.leiden_server_evict(srv, small) == 0
     assert large() == [152]
     host.lib.leiden_server_destroy(srv)
+
+
+def test_the_csr_pass_follows_the_sms_of_the_device(host):
+    # one wave on a device (or a context's share) of 8 SMs, not on 152
+    host.reset(sms=8)
+    n, nnz = 20000, 4000000
+    host.static(n, nnz)
+    g = host.csr(n, nnz)
+    lab, q = np.zeros(n, np.int32), C.c_double()
+    assert host.lib.leiden_modularity_noalloc(C.byref(g), C.c_void_p(lab.ctypes.data), C.c_double(1.0), None,
+                                              C.byref(q)) == 0
+    rows = [x for x in host.log() if "rows_k" in x[1] and "check" not in x[1]]
+    assert len(rows) == 2 and all(x[2] == 8 * (2048 // x[3]) for x in rows), rows
