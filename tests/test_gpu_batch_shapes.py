@@ -3,15 +3,11 @@ is checked in test_host_launches.py) gives each graph the result of a context.
 All arithmetic is integer, so every comparison is exact."""
 from __future__ import annotations
 
-import os
-import sys
-
 import pytest
 
 from paper_2405_11658_gb300 import synth as S
 
-sys.path.insert(0, os.path.dirname(os.path.abspath(__file__)))
-from batch_shapes import SHAPES  # noqa: E402
+from tests.batch_shapes import SHAPES
 
 pytestmark = pytest.mark.gpu
 

@@ -5,14 +5,12 @@ from __future__ import annotations
 
 import ctypes as C
 import re
-import sys
 
 import numpy as np
 import pytest
 
-sys.path.insert(0, __file__.rsplit("/", 1)[0])
-import host_library  # noqa: E402
-from batch_shapes import SHAPES  # noqa: E402
+from tests import host_library
+from tests.batch_shapes import SHAPES
 
 
 @pytest.fixture(scope="module")
