@@ -21,7 +21,11 @@ enum { TEAM_NONE = 0, TEAM_CONVERGED = 1, TEAM_NO_SHRINK = 2, TEAM_RENUMBERED = 
 static constexpr int64_t TEAM_MAX_CAND = 8192;
 static constexpr int TEAM_MAX_HUBS = 16384;
 static constexpr int TEAM_MAX_BLOCKS = 1024;
-static constexpr u64 TEAM_SPIN_LIMIT = 1ull << 24;   // polls of a grid barrier (several seconds)
+// Polls of a grid barrier before it gives up (the default takes several seconds).
+#ifndef LK_TEAM_SPIN_LIMIT
+#define LK_TEAM_SPIN_LIMIT (1ull << 24)
+#endif
+static constexpr u64 TEAM_SPIN_LIMIT = LK_TEAM_SPIN_LIMIT;
 
 // Control words of a team, zeroed before every pass.
 struct TeamCtl {
