@@ -274,7 +274,7 @@ typedef struct leiden_batch leiden_batch;
  * max_total_n vertices and max_total_nnz CSR entries summed over the run's
  * graphs (about 100 B per vertex plus 60 B per entry).  `threads` (128..512,
  * multiple of 32; 0) and blocks_per_sm (1..4; 0) are checked and otherwise
- * without effect: the kernel has one shape, chosen for the SMs it runs on.
+ * without effect: each run picks the kernel's shape by its graphs' sizes.
  * Errors: LEIDEN_EINVAL, LEIDEN_ENOMEM, LEIDEN_ECUDA. */
 int leiden_batch_create(leiden_batch **out, void *cuda_stream, int32_t max_graphs, int64_t max_total_n,
                         int64_t max_total_nnz, int32_t threads, int32_t blocks_per_sm);

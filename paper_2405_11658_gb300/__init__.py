@@ -487,7 +487,10 @@ STATIC = 0
 
 class Batch:
     """A ``leiden_batch``: many small graphs per call, each run whole by one
-    thread block or one cluster of one persistent, CUDA-graph-captured launch."""
+    thread block or one cluster of one persistent, CUDA-graph-captured launch.
+    ``threads`` (128..512, a multiple of 32, or 0) and ``blocks_per_sm`` (1..4
+    or 0) are checked and otherwise without effect: the library picks the shape
+    of the launch by the sizes of each call's graphs."""
 
     def __init__(self, max_graphs: int, max_total_n: int, max_total_nnz: int, threads: int = 0,
                  blocks_per_sm: int = 0, stream=None):

@@ -638,6 +638,13 @@ int pass_body(Run &r, GraphView<WT> g, int lp, double tau, int dst, int64_t *nc_
 // 2.3e8 with hubs (Chung-Lu): the launches, the fork to the auxiliary streams
 // and their join cost more than the sub-sweep itself on the small levels, and
 // on the large ones the tiers of a class run back to back without a tail each.
+// The largest first levels are level or slower, because 32 warps an SM keep
+// fewer gathers in flight than the tier kernels do once C' and Sigma' leave L2:
+// local-moving and refinement of the first level (ms) 68 -> 60 at 1.25e7
+// vertices / 5.0e8 entries, 125 -> 128 at 2.5e7 / 1.0e9 and 254 -> 279 at 5e7 /
+// 2.0e9 (Chung-Lu), 124 -> 90 at 6e7 / 1.3e8 (k-mer), 86 -> 88 at 3.4e7 / 7.9e8
+// (R-MAT).  The whole Static gains at each of these sizes (598 -> 475, 1082 ->
+// 893, 2128 -> 1838, 429 -> 252 and 580 -> 454 ms).
 bool team_takes(const Run &r, int64_t n) {
   return r.o->sched == LEIDEN_DET && !r.c->tiers_set && n > 0 && n < ((int64_t)1 << 30);
 }

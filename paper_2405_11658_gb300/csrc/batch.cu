@@ -172,7 +172,7 @@ bool same_opts(const SmallOpts &a, const SmallOpts &b) { return memcmp(&a, &b, s
 extern "C" int leiden_batch_create(leiden_batch **out, void *stream, int32_t max_graphs, int64_t max_total_n,
                                    int64_t max_total_nnz, int32_t threads, int32_t blocks_per_sm) {
   if (!out || max_graphs < 1 || max_total_n < 0 || max_total_nnz < 0) return LEIDEN_EINVAL;
-  // the kernel has one shape; the two arguments are only checked
+  // each run picks its shape (batch_shape); the two arguments are only checked
   if (threads && (threads < 128 || threads > 512 || threads % 32)) return LEIDEN_EINVAL;
   if (blocks_per_sm && (blocks_per_sm < 1 || blocks_per_sm > 4)) return LEIDEN_EINVAL;
   leiden_batch *b = new leiden_batch();

@@ -19,8 +19,8 @@
 // scan), and equal communities meet in shared-memory atomics instead of a
 // match across the warp.  Measured (Static of a 1e4-vertex planted partition,
 // 480 sub-sweeps): 13.7 ms with one launch per tier and sub-sweep, 8.2 ms on
-// resident blocks with the tables cleared and scanned, 6.0 ms as here; R-MAT
-// scale 22 with hubs 123 -> 100 ms, Chung-Lu of 2.5e8 entries 290 -> 247 ms.
+// resident blocks with the tables cleared and scanned, 6.3 ms as here; R-MAT
+// scale 22 with hubs 122 -> 89 ms, Chung-Lu of 2.5e8 entries 294 -> 231 ms.
 #pragma once
 
 #include <limits.h>
