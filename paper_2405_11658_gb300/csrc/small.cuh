@@ -43,6 +43,7 @@ static_assert(sizeof(TeamShared<int64_t>) <= sizeof(WideShared), "one shared blo
 // plain shared words that the compiler keeps in registers, they spilled
 // thousands of bytes in a thread of a 1024-thread block.
 struct SmallArrays {
+  static constexpr bool MANY_HUBS = true;
   Held<int32_t *> C, CB, rep, vlist;
   Held<int64_t *> K, Sig, Sig2;
   Held<uint8_t *> ch, ch2, processed, stamp, exists;

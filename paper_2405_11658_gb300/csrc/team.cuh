@@ -688,8 +688,9 @@ __device__ __forceinline__ void team_hub_add(const AR &a, int64_t at, uint64_t t
   atomicOr(a.err, 16ull);
 }
 
-// Prefix sums of every class's hub items; false when a class's tables exceed
-// the scratch (the same answer in every block).
+// Prefix sums of every class's hub items; false when a class has too many hubs
+// (see MANY_HUBS) or its tables exceed the scratch (the same answer in every
+// block).
 template <typename WT, typename ST, typename GL, typename AR>
 __device__ __forceinline__ bool team_hub_setup(const GL &g, const AR &a, int S, Team &t,
                                                TeamShared<ST> &sm) {
@@ -728,7 +729,8 @@ __device__ __forceinline__ bool team_hub_setup(const GL &g, const AR &a, int S, 
         a.hub_done[p - h0] = 0;
       }
     }
-    if (threadIdx.x == 0 && (cs * HUB_SLOTS > a.tcap || ci > INT_MAX / 2))
+    if (threadIdx.x == 0 &&
+        ((!AR::MANY_HUBS && p1 - p0 > TEAM_MAX_HUBS) || cs * HUB_SLOTS > a.tcap || ci > INT_MAX / 2))
       t.ctl->too_big = 1;
   }
   if (!t.sync()) return false;
@@ -754,7 +756,7 @@ __device__ __forceinline__ bool team_hub_bits(const AR &a, const CT &ct, const i
     bool act = false;
     if (k < m) act = team_hub_active<REFINE>(a, ct, list[k]);
     const unsigned mk = __ballot_sync(FULL_MASK, act);
-    if ((threadIdx.x & 31) == 0 && k < m && k < TEAM_MAX_HUBS) sm.hbits[(base + (int)threadIdx.x) >> 5] = mk;
+    if ((threadIdx.x & 31) == 0 && k < m && (!AR::MANY_HUBS || k < TEAM_MAX_HUBS)) sm.hbits[(base + (int)threadIdx.x) >> 5] = mk;
     any |= mk != 0;
   }
   return __syncthreads_or(any) != 0;
@@ -764,7 +766,8 @@ __device__ __forceinline__ bool team_hub_bits(const AR &a, const CT &ct, const i
 template <bool REFINE, typename ST, typename AR, typename CT>
 __device__ __forceinline__ bool team_hub_bit(const AR &a, const CT &ct, const int32_t *list, int k,
                                              const TeamShared<ST> &sm) {
-  return k < TEAM_MAX_HUBS ? (sm.hbits[k >> 5] >> (k & 31)) & 1u : team_hub_active<REFINE>(a, ct, list[k]);
+  if (AR::MANY_HUBS && k >= TEAM_MAX_HUBS) return team_hub_active<REFINE>(a, ct, list[k]);
+  return (sm.hbits[k >> 5] >> (k & 31)) & 1u;
 }
 
 template <bool REFINE, typename WT, typename ST, typename GL, typename AR, typename CT>

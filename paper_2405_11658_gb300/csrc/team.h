@@ -16,8 +16,8 @@ enum { TEAM_BLOCK = 0, TEAM_CLUSTER = 1, TEAM_GRID = 2 };
 enum { TEAM_NONE = 0, TEAM_CONVERGED = 1, TEAM_NO_SHRINK = 2, TEAM_RENUMBERED = 3, TEAM_AGGREGATED = 4, TEAM_TOO_BIG = 5 };
 
 // Distinct candidates of a vertex the block's table takes (half its slots);
-// vertices with more are hubs.  Hubs of a colour class whose eligibility is
-// looked up once a sub-sweep (any beyond them are asked again per item).
+// vertices with more are hubs.  Hubs of a colour class whose eligibility a
+// block notes once a sub-sweep.
 static constexpr int64_t TEAM_MAX_CAND = 8192;
 static constexpr int TEAM_MAX_HUBS = 16384;
 static constexpr int TEAM_MAX_BLOCKS = 1024;
@@ -48,6 +48,11 @@ static constexpr size_t TEAM_CTL_HEAD = offsetof(TeamCtl, part);
 
 // Arrays of the current level; n and nnz bound them all.
 struct TeamArrays {
+  // A class with more hubs than a block notes makes the pass give up
+  // (TEAM_TOO_BIG; the context runs it on the multi-kernel path).  Where there
+  // is no other path, the hubs beyond are asked again per item, which cost
+  // hub-heavy passes of a context 1% (Chung-Lu DF) for code they hardly reach.
+  static constexpr bool MANY_HUBS = false;
   int32_t *C, *CB, *rep, *vlist;
   int64_t *K, *Sig, *Sig2;
   uint8_t *ch, *ch2, *processed, *stamp, *exists;
